@@ -341,6 +341,19 @@ cbfm_status cbfm_wait_selftest(int32_t kind, double limit_s, void *stream);
  */
 cbfm_status cbfm_gram_inverse(const double *A, int64_t n, int32_t nbatch, double *Ainv, void *stream);
 
+/*
+ * cbfm_matmul_f64 -- one FP64 product of the dense algebra on caller matrices:
+ * a testing hook for both of its forms (the paper has no counterpart).
+ *   C = op(A) op(B) (+ C when accumulate), complex128 row-major, host or device;
+ *   op(A) is M x K, op(B) K x N; op 0 = as stored, 1 = transposed, 2 =
+ *   conjugate transposed, 3 = conjugated
+ *   unit  0 = the form the library takes at these sizes, 1 = FP64 units,
+ *         2 = tensor cores (operands cut into exact digits)
+ * Returns CBFM_EINVAL on bad arguments.
+ */
+cbfm_status cbfm_matmul_f64(const double *A, const double *B, double *C, int64_t M, int64_t N, int64_t K, int32_t opA,
+                            int32_t opB, int32_t unit, int32_t accumulate, void *stream);
+
 /* G^CBF as complex128 row-major (n_cbf, n_cbf), host or device; after cbfm_cmp_setup or cbfm_cmp_setup_inexact. */
 cbfm_status cbfm_gram_export(cbfm_red_t red, double *G, void *stream);
 

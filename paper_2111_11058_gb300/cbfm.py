@@ -75,6 +75,7 @@ def lib():
             "cbfm_cmp_setup_inexact": [_vp, _f64, _i32, _i32, _vp],
             "cbfm_gram_export": [_vp, _vp, _vp],
             "cbfm_gram_inverse": [_vp, _i64, _i32, _vp, _vp],
+            "cbfm_matmul_f64": [_vp, _vp, _vp, _i64, _i64, _i64, _i32, _i32, _i32, _i32, _vp],
             "cbfm_wait_selftest": [_i32, _f64, _vp],
             "cbfm_solve": [_vp, _vp, _i32, _f64, _i32, _i32, _i32, _i32, _vp, _vp, _i32, _vp, _vp, _vp, _vp],
             "cbfm_session_create": [_vp, _vp, _i32, _f64, _i32, _i32, _i32, _vp],
@@ -106,7 +107,7 @@ def exported_symbols():
     """Names of the C entry points declared in include/cbfm.h."""
     return ["cbfm_mesh", "cbfm_mesh_edges", "cbfm_mesh_info", "cbfm_mesh_cells", "cbfm_build_cbfs", "cbfm_cbf_import",
             "cbfm_cbf_export", "cbfm_assemble_reduced", "cbfm_assemble_reduced_batch", "cbfm_assemble_mom", "cbfm_tdiag_setup", "cbfm_build_ipcbfs", "cbfm_tuning", "cbfm_red_export", "cbfm_red_export_noalloc", "cbfm_cmp_setup", "cbfm_cmp_setup_inexact", "cbfm_gram_export",
-            "cbfm_gram_inverse", "cbfm_wait_selftest", "cbfm_solve", "cbfm_session_create", "cbfm_session_join",
+            "cbfm_gram_inverse", "cbfm_matmul_f64", "cbfm_wait_selftest", "cbfm_solve", "cbfm_session_create", "cbfm_session_join",
             "cbfm_session_run", "cbfm_session_results", "cbfm_free", "cbfm_last_error", "cbfm_launch_count",
             "cbfm_profile", "cbfm_profile_read"]
 
@@ -152,6 +153,21 @@ def gram_inverse(A, stream=None) -> np.ndarray:
     out = np.zeros_like(A)
     _check(lib().cbfm_gram_inverse(ctypes.c_void_p(A.ctypes.data), n, nb, ctypes.c_void_p(out.ctypes.data),
                                    _stream(stream)))
+    return out
+
+
+def matmul_f64(A, B, opA: int = 0, opB: int = 0, unit: int = 0, C=None, stream=None) -> np.ndarray:
+    """cbfm_matmul_f64: op(A) op(B) (+ C) in FP64 by the form named by unit (testing hook)."""
+    A = np.ascontiguousarray(A, np.complex128)
+    B = np.ascontiguousarray(B, np.complex128)
+    M, K = A.shape if opA in (0, 3) else A.shape[::-1]
+    K2, N = B.shape if opB in (0, 3) else B.shape[::-1]
+    if K != K2:
+        raise ValueError("inner sizes differ")
+    out = np.zeros((M, N), np.complex128) if C is None else np.array(C, np.complex128)
+    p = lambda x: ctypes.c_void_p(x.ctypes.data)  # noqa: E731
+    _check(lib().cbfm_matmul_f64(p(A), p(B), p(out), M, N, K, int(opA), int(opB), int(unit), 0 if C is None else 1,
+                                 _stream(stream)))
     return out
 
 

@@ -1393,6 +1393,31 @@ cbfm_status cbfm_gram_inverse(const double *A, int64_t n, int32_t nbatch, double
     });
 }
 
+cbfm_status cbfm_matmul_f64(const double *A, const double *B, double *C, int64_t M, int64_t N, int64_t K, int32_t opA,
+                            int32_t opB, int32_t unit, int32_t accumulate, void *stream) {
+    return guarded([&] {
+        StreamScope ss_((cudaStream_t)stream);   // scratch is stream-ordered on the caller's stream
+        CBFM_REQUIRE(A && B && C, "NULL matrix");
+        CBFM_REQUIRE(M >= 1 && N >= 1 && K >= 1 && M <= 65536 && N <= 65536 && K <= 65536, "sizes must be in [1, 65536]");
+        CBFM_REQUIRE(opA >= 0 && opA <= 3 && opB >= 0 && opB <= 3, "op must be 0 (N), 1 (T), 2 (H) or 3 (conj)");
+        CBFM_REQUIRE(unit >= 0 && unit <= 2, "unit must be 0 (by size), 1 (FP64 units) or 2 (tensor cores)");
+        cudaStream_t st = (cudaStream_t)stream;
+        DevBuf<z64> a, b, c;
+        a.alloc((size_t)M * K);
+        b.alloc((size_t)K * N);
+        c.alloc((size_t)M * N);
+        copy_in(a.p, A, sizeof(z64) * M * K, st);
+        copy_in(b.p, B, sizeof(z64) * K * N, st);
+        copy_in(c.p, C, sizeof(z64) * M * N, st);
+        const GemmDesc d{M, N, K, 0, (opA == 0 || opA == 3) ? K : M, 0, (opB == 0 || opB == 3) ? N : K, 0, N};
+        if (unit == 2) gemm_oz(d, opA, opB, a.p, b.p, c.p, accumulate != 0, st, false);
+        else if (unit == 1) gemm_grouped<double>({d, GemmDesc{}}, opA, opB, a.p, b.p, c.p, accumulate != 0, st);
+        else gemm_grouped<double>({d}, opA, opB, a.p, b.p, c.p, accumulate != 0, st);
+        copy_out(C, c.p, sizeof(z64) * M * N, st);
+        CBFM_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
 cbfm_status cbfm_gram_export(cbfm_red_t red, double *G, void *stream) {
     return guarded([&] {
         StreamScope ss_((cudaStream_t)stream);   // scratch is stream-ordered on the caller's stream

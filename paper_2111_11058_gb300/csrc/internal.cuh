@@ -120,6 +120,24 @@ struct GemmDesc {
 template <typename T>
 void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> *A, const cx<T> *B, cx<T> *C,
                   bool accumulate, cudaStream_t st, double alpha = 1.0);
+// Tensor-core form of one FP64 product (k_oz.cu): C = +-op(A) op(B) [+ C].  oz_takes: where it is the faster one.
+bool oz_takes(int64_t M, int64_t N, int64_t K);
+void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z64 *C, bool accumulate, cudaStream_t st,
+             bool neg);
+// Scratch and error word of the tensor-core products launched on this thread while an object is alive: the caller
+// reads *err (nonzero: a device wait expired) at a point where it waits for the stream anyway.  Without one every
+// product allocates its own and waits.
+struct OzWork;
+extern thread_local OzWork *g_oz;
+struct OzWork {
+    DevBuf<unsigned char> buf;
+    int *err;
+    OzWork *prev;
+    explicit OzWork(int *e) : err(e), prev(g_oz) { g_oz = this; }
+    ~OzWork() { g_oz = prev; }
+    OzWork(const OzWork &) = delete;
+    OzWork &operator=(const OzWork &) = delete;
+};
 // Profiling label of the FP64 products launched while an object is alive
 // (reported as "site:<label>" beside the kernel's own record).
 extern thread_local const char *g_gemm_site;

@@ -536,8 +536,12 @@ GemmDesc sub_desc(GemmDesc d, int opA, int opB, int64_t r0, int64_t rows, int64_
     return d;
 }
 constexpr int64_t TT = 32;   // tile edge of the FP64 product kernel
+// The splits below spare the FP64 units the zero part of a triangular or
+// Hermitian product.  A product the tensor cores take stays whole: there the second
+// packing of an operand costs more than the zeros (all operands hold them).
 // The block upper triangle (tiles on or above the diagonal) of a Hermitian square product
 std::vector<GemmDesc> upper_tiles(const GemmDesc &d, int opA, int opB) {
+    if (oz_takes(d.M, d.N, d.K)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT)
         g.push_back(sub_desc(d, opA, opB, r0, std::min(TT, d.M - r0), r0, d.N - r0, 0, d.K));
@@ -545,6 +549,7 @@ std::vector<GemmDesc> upper_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(A) lower triangular (row i is zero beyond column i): row tiles summed up to their last row
 std::vector<GemmDesc> lower_a_tiles(const GemmDesc &d, int opA, int opB) {
+    if (oz_takes(d.M, d.N, d.K)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT) {
         const int64_t rows = std::min(TT, d.M - r0);
@@ -554,6 +559,7 @@ std::vector<GemmDesc> lower_a_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(A) upper triangular (row i is zero before column i): row tiles summed from their first row
 std::vector<GemmDesc> upper_a_tiles(const GemmDesc &d, int opA, int opB) {
+    if (oz_takes(d.M, d.N, d.K)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT)
         if (r0 < d.K) g.push_back(sub_desc(d, opA, opB, r0, std::min(TT, d.M - r0), 0, d.N, r0, d.K - r0));
@@ -561,6 +567,7 @@ std::vector<GemmDesc> upper_a_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(B) upper triangular (column j is zero below row j): column tiles summed up to their last column
 std::vector<GemmDesc> upper_b_tiles(const GemmDesc &d, int opA, int opB) {
+    if (oz_takes(d.M, d.N, d.K)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t c0 = 0; c0 < d.N; c0 += TT) {
         const int64_t cols = std::min(TT, d.N - c0);
@@ -879,6 +886,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     c.status.alloc(1);
     c.Dinv.alloc((size_t)CH_NPAN * CH_B * CH_B);
     CBFM_CUDA(cudaMemsetAsync(c.err.p, 0, sizeof(int), st));
+    OzWork oz_(c.err.p);   // scratch of the tensor-core products; their error word is read with the Cholesky's
     c.rnrm.alloc(PCHOL_MAX);
     c.scale.alloc(PCHOL_MAX);
     c.dev.alloc(1 + GD_CTAS);   // the deviation and its per-CTA partials
@@ -1138,10 +1146,16 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             // row block r of the new column meets only the Q blocks i >= r - 1.
             if (d0 > 0) {
                 std::vector<GemmDesc> proj, upd;
-                for (int i = 0; i < J; ++i)
+                // on the tensor cores one product over all blocks (Qh holds the zeros)
+                const bool whole = oz_takes(d0, pjc, d1);
+                if (whole) {
+                    proj.push_back(GemmDesc{d0, pjc, d1, 0, dcap, 0, p, 0, p});
+                    upd.push_back(GemmDesc{d1, pjc, d0, 0, dcap, 0, p, 0, p});
+                }
+                for (int i = 0; i < J && !whole; ++i)
                     proj.push_back(GemmDesc{dims[i + 1] - dims[i], pjc, dims[i + 2], dims[i], dcap, 0, p,
                                             dims[i] * p, p});
-                for (int r = 0; r <= J; ++r) {
+                for (int r = 0; r <= J && !whole; ++r) {
                     const int64_t k0 = dims[std::max(0, r - 1)];
                     if (k0 >= d0) continue;
                     upd.push_back(GemmDesc{dims[r + 1] - dims[r], pjc, d0 - k0, dims[r] * dcap + k0, dcap, k0 * p,
@@ -1251,7 +1265,10 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     else if (pc == CBFM_PC_TDIAG) tdiag_recover(rd, Y.p, d_x, p, st);
     else if (pc == CBFM_PC_CMP_INEXACT) cmp_inner_apply(rd, Y.p, d_x, p, st);
     else CBFM_CUDA(cudaMemcpyAsync(d_x, Y.p, sizeof(z64) * p * n, cudaMemcpyDeviceToDevice, st));
+    int h_err = 0;   // the products since the last Cholesky
+    CBFM_CUDA(cudaMemcpyAsync(&h_err, c.err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     CBFM_CUDA(cudaStreamSynchronize(st));
+    if (h_err) throw Fail{CBFM_ETIMEOUT, "block GMRES: a device wait expired"};
     // iterations counted from the block iteration a right-hand side joined at
     for (int q = 0; q < p; ++q)
         out.iters[q] = conv_at[q] >= 0 ? conv_at[q] - join_at[q] : -(total_blocks - join_at[q]) - 1;

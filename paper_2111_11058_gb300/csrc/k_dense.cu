@@ -1425,8 +1425,16 @@ void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> 
             fl += flop_per_cmac * d.M * d.N * d.K;
             by += (double)(d.M * d.K + d.K * d.N + d.M * d.N) * sizeof(cx<T>);
         }
-        prof_add_work(sizeof(T) == 8 ? "k_gemm_z64" : "k_gemm_c32", fl, by);
         if (sizeof(T) == 8) prof_add_work(g_gemm_site ? g_gemm_site : "site:other", fl, by);   // per solver step
+        if constexpr (sizeof(T) == 8) {
+            // one large product: on the tensor cores, cut into exact digits
+            if (g.size() == 1 && (alpha == 1.0 || alpha == -1.0) && oz_takes(g[0].M, g[0].N, g[0].K)) {
+                ProfScope site_(g_gemm_site ? g_gemm_site : "site:other", st);
+                gemm_oz(g[0], opA, opB, A, B, C, accumulate, st, alpha < 0.0);
+                return;
+            }
+        }
+        prof_add_work(sizeof(T) == 8 ? "k_gemm_z64" : "k_gemm_c32", fl, by);
     }
     if constexpr (sizeof(T) == 8) {
         gemm_sk(g, opA, opB, A, B, C, accumulate, st, alpha);
