@@ -1307,9 +1307,20 @@ cbfm_status cbfm_cmp_setup(cbfm_red_t red, void *stream) {
             launched("k_place_neg_adjoint");
         }
         int hinfo = 0;
+        std::vector<std::complex<double>> hdiag(nh);   // the diagonal of the first half (the second is minus its conjugate)
         CBFM_CUDA(cudaMemcpyAsync(&hinfo, info.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CBFM_CUDA(cudaMemcpy2DAsync(hdiag.data(), sizeof(z64), r->G.p, sizeof(z64) * (n + 1), sizeof(z64), nh,
+                                    cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaStreamSynchronize(st));
         if (hinfo) throw Fail{CBFM_ESINGULAR, "G^CBF is singular"};
+        {
+            double lo = INFINITY, hi = 0.0;
+            for (const std::complex<double> &g : hdiag) {
+                lo = std::min(lo, std::abs(g));
+                hi = std::max(hi, std::abs(g));
+            }
+            r->gram_spread = lo > 0.0 ? hi / lo : INFINITY;
+        }
         // B = A (G^CBF)^{-1}: GMRES then needs one product per iteration
         std::vector<GemmDesc> gb{GemmDesc{n, n, n, 0, n, 0, n, 0, n}};
         if (r->prec != CBFM_FP64) {

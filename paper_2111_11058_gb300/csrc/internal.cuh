@@ -80,6 +80,7 @@ struct Red : HandleBase {
     DevBuf<z64> B64;              // B = A (G^CBF)^{-1}, the operator GMRES iterates with
     DevBuf<c32> B32;
     bool cmp_ready = false;
+    double gram_spread = 0.0;     // largest over smallest modulus on the diagonal of G^CBF (cbfm_cmp_setup)
     // T-diagonal arrangement (Eq. (MoM_T)): Bt = A P D^{-1} (P swaps the column halves),
     // tdinv[k] = 1 / D_{p(k)}: the recovery x_k = y_{p(k)} tdinv[k]
     DevBuf<z64> Bt64;
@@ -138,6 +139,24 @@ struct OzWork {
     OzWork(const OzWork &) = delete;
     OzWork &operator=(const OzWork &) = delete;
 };
+// While an object made with true is alive, oz_takes() answers no on this thread (products stay on the FP64 units).
+extern thread_local bool g_oz_hold;
+struct OzHold {
+    bool prev;
+    explicit OzHold(bool hold) : prev(g_oz_hold) { g_oz_hold = prev || hold; }
+    ~OzHold() { g_oz_hold = prev; }
+    OzHold(const OzHold &) = delete;
+    OzHold &operator=(const OzHold &) = delete;
+};
+// A matrix cut into digits once and multiplied many times (the operator of an iterative solve): n_rows x n_k,
+// row-major, complex64 (widened exactly) or complex128.
+struct OzMat {
+    DevBuf<unsigned char> buf;
+    int64_t rows = 0, K = 0;
+    void pack(const void *X, bool f32, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st);
+};
+// out[r] = M in[r] for n rows of leading dimensions ldi and ldo, FP64
+void gemm_oz_rows(const OzMat &M, const z64 *in, int64_t ldi, z64 *out, int64_t ldo, int64_t n, cudaStream_t st);
 // Profiling label of the FP64 products launched while an object is alive
 // (reported as "site:<label>" beside the kernel's own record).
 extern thread_local const char *g_gemm_site;

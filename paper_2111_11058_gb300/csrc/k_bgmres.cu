@@ -598,6 +598,10 @@ constexpr double ORTH_TOL = 1e-12;
 // under ORTH_TOL); otherwise its coefficients are formed and applied when
 // they exceed ORTH_TOL of the block.
 constexpr double GS_KEEP = 0.1;
+// Spread of the diagonal of G^CBF (the CBFs' singular values) up to which a mixed-precision solve forms its basis
+// on the tensor cores; measured 1e3 to 5e3 on cubes, spheres and cylinders with even triangles, 1.4e4 to 1e5 on
+// spheroids and cylinders with pole triangles.
+constexpr double SPREAD_MAX = 1e4;
 
 // ||M - I||_F of the m x m Gram matrix in ctx.M (host sync).
 double gram_dev(Ctx &c, int m) {
@@ -970,11 +974,25 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     CBFM_CUDA(cudaMemcpyAsync(h_bn.data(), bnorm.p, sizeof(double) * p, cudaMemcpyDeviceToHost, st));
     CBFM_CUDA(cudaStreamSynchronize(st));
 
+    // Where the operator's product is FP32, its rounding errors depend on the last bits of the basis, and the
+    // reduced system amplifies them: with the CBFs' singular values spread over SPREAD_MAX and more (tiny triangles
+    // beside large ones) the currents move by 1e-5 of their norm and 1e-3 of their rms at single edges when the
+    // sums of the basis are only reordered (1.5e-6 and 6e-5 where the spread is below 5e3).  Those systems keep the FP64 units' sums for the basis
+    // and the FP32 solution update, so that their results stay reproducible; everything else goes to the tensor
+    // cores.
+    const bool tc_basis = rd.prec == CBFM_FP64 || (pc == CBFM_PC_CMP && rd.gram_spread <= SPREAD_MAX);
+    OzMat op;   // FP64 operator cut into digits once per solve
     auto applyB = [&](const z64 *in, z64 *out, int rows) {
         if (pc == CBFM_PC_CMP_INEXACT) {
             if (zin.p == nullptr) zin.alloc((size_t)p * n);
             cmp_inner_apply(rd, in, zin.p, rows, st);
             in = zin.p;
+        }
+        if (rd.prec == CBFM_FP64 && oz_takes(rows, n, n)) {
+            if (op.rows == 0) op.pack(pc_op64(rd, pc), false, n, n, n, st);
+            GemmSite site_("site:operator");
+            gemm_oz_rows(op, in, n, out, n, rows, st);
+            return;
         }
         if (rd.prec != CBFM_FP64)
             rows_times(n, nullptr, pc_op32(rd, pc), in, out, rows, false, st, s_in.p, s_out.p);
@@ -1054,7 +1072,11 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
         CBFM_CUDA(cudaMemsetAsync(E1S.p, 0, sizeof(z64) * dcap2 * p, st));
         CBFM_CUDA(cudaMemsetAsync(Qh.p, 0, sizeof(z64) * dcap2 * dcap, st));
         CBFM_CUDA(cudaMemsetAsync(Rh.p, 0, sizeof(z64) * dcap * dcap, st));
-        const int p1 = cholqr2_rows(c, tmp.p, p, n, V.p, E1S.p, rank_tol, 0.0, drop_tol);
+        int p1;
+        {
+            OzHold hold_(!tc_basis);
+            p1 = cholqr2_rows(c, tmp.p, p, n, V.p, E1S.p, rank_tol, 0.0, drop_tol);
+        }
         CBFM_CUDA(cudaMemcpyAsync(Rv.p, E1S.p, sizeof(z64) * dcap2 * p, cudaMemcpyDeviceToDevice, st));
         if (p1 == 0) {   // residual block is zero: current iterate is exact
             for (int r = 0; r < p; ++r) {
@@ -1083,6 +1105,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             // others are orthogonal to the basis to ~10 u already), gathered into Ws
             {
                 GemmSite site_("site:gs1");
+                OzHold hold_(!tc_basis);
                 gemm_grouped<double>({GemmDesc{pjc, d1, n, 0, n, 0, n, 0, dcap}}, 0, 2, W.p, V.p, tmp2.p, false, st);
                 gemm_grouped<double>({GemmDesc{pjc, n, d1, 0, dcap, 0, n, 0, n}}, 0, 0, tmp2.p, V.p, W.p, true, st,
                                      -1.0);
@@ -1104,6 +1127,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                 }
             if (!sel.empty()) {
                 GemmSite site_("site:gs2");
+                OzHold hold_(!tc_basis);
                 const int k = (int)sel.size();
                 const bool all = k == pjc;
                 if (!all) {
@@ -1130,7 +1154,11 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                 if (!all) CBFM_CUDA(cudaStreamSynchronize(st));   // sel is a host vector of this scope
             }
             // orthonormalise the new block (pivoted: drops dependent directions)
-            const int r = wref > 0.0 ? cholqr2_rows(c, W.p, pjc, n, V.p + d1 * n, Rw.p, rank_tol, wref, drop_tol) : 0;
+            int r = 0;
+            if (wref > 0.0) {
+                OzHold hold_(!tc_basis);
+                r = cholqr2_rows(c, W.p, pjc, n, V.p + d1 * n, Rw.p, rank_tol, wref, drop_tol);
+            }
             const int rr = r;
             const int64_t d2 = d1 + rr;
             // new block column of Hbar (d2 x pjc, ld p): [C; R_W]
@@ -1234,7 +1262,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             gemm_grouped<double>({GemmDesc{pi, p, pi, a0 * p, p, 0, p, a0 * p, p}}, 0, 0, RinvBlk.p, tmp2.p, Z.p,
                                  false, st);
         }
-        if (rd.prec != CBFM_FP64) {
+        if (rd.prec != CBFM_FP64 && !(tc_basis && oz_takes(p, n, dJ))) {
             // mixed precision: the solution update Y += Z^T V (not part of the orthogonalisation or the
             // residual) in FP32, like the operator product
             if (V32.p == nullptr) {
@@ -1259,7 +1287,15 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
         d_x = x_all->p;
     }
     if (pc == CBFM_PC_CMP) {   // G^CBF^{-1} is block diagonal (its two halves)
-        if (rd.prec != CBFM_FP64) rows_times(n, nullptr, rd.Ginv32.p, Y.p, d_x, p, true, st, s_in.p, s_out.p);
+        if (tc_basis && oz_takes(p, n / 2, n / 2)) {
+            // the inverse the operator was formed with: the complex64 one on the mixed path
+            const int64_t h = n / 2;
+            for (int64_t o = 0; o < n; o += h) {
+                if (rd.prec != CBFM_FP64) op.pack(rd.Ginv32.p + o * n + o, true, h, h, n, st);
+                else op.pack(rd.Ginv.p + o * n + o, false, h, h, n, st);
+                gemm_oz_rows(op, Y.p + o, n, d_x + o, n, p, st);
+            }
+        } else if (rd.prec != CBFM_FP64) rows_times(n, nullptr, rd.Ginv32.p, Y.p, d_x, p, true, st, s_in.p, s_out.p);
         else rows_times(n, rd.Ginv.p, nullptr, Y.p, d_x, p, true, st, nullptr, nullptr);
     }
     else if (pc == CBFM_PC_TDIAG) tdiag_recover(rd, Y.p, d_x, p, st);

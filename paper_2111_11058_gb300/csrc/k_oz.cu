@@ -42,6 +42,7 @@ namespace cbfm {
 
 namespace cg = cooperative_groups;
 thread_local OzWork *g_oz = nullptr;
+thread_local bool g_oz_hold = false;
 
 namespace {
 
@@ -74,9 +75,9 @@ constexpr int OZ_BAD = 0x7fff;   // row exponent of a row with an infinity or Na
 constexpr int PK_WARPS = 16, PK_KEEP = 4;
 
 struct OzPack {
-    const z64 *X;
+    const void *X;         // complex128, or complex64 (widened exactly) where f32 is set
     int64_t off, rs, cs;   // element (row r, k): X[off + r rs + k cs]
-    int conj;
+    int conj, f32;
     int rows;              // rows in use (the rest of the last tile is zero)
     int groups;            // 8-row groups, padding included
     int expand;            // right operand: two real rows per row
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(32 * PK_WARPS) k_oz_pack(const __grid_constant
     const int rr = lane >> 2, ch = lane & 3;
     const int r = g * 8 + rr;
     const bool live = r < P.rows;
-    const z64 *X = P.X + P.off + (int64_t)r * P.rs;
+    const int64_t x0 = P.off + (int64_t)r * P.rs;
     __shared__ uint32_t s_mx[PK_WARPS][8];
     double2 keep[PK_KEEP][4];
     uint32_t mx = 0;
@@ -146,7 +147,15 @@ __global__ void __launch_bounds__(32 * PK_WARPS) k_oz_pack(const __grid_constant
         for (int q = 0; q < 4; ++q) {
             const int k = kb * 16 + ch * 4 + q;
             v[q] = make_double2(0.0, 0.0);
-            if (live && k < pp.K) v[q] = *reinterpret_cast<const double2 *>(X + (int64_t)k * P.cs);
+            if (live && k < pp.K) {
+                const int64_t i = x0 + (int64_t)k * P.cs;
+                if (P.f32) {
+                    const float2 f = reinterpret_cast<const float2 *>(P.X)[i];
+                    v[q] = make_double2((double)f.x, (double)f.y);
+                } else {
+                    v[q] = reinterpret_cast<const double2 *>(P.X)[i];
+                }
+            }
         }
     };
     auto top = [&](const double2 (&v)[4]) {
@@ -544,74 +553,49 @@ void set_smem_once(F *f, int bytes) {
 
 }  // namespace
 
-bool oz_takes(int64_t M, int64_t N, int64_t K) {
-    if (M < 1 || N < 1 || K < 1 || M > (1 << 24) || N > (1 << 24) || K > (1 << 18)) return false;
-    const Shape s = oz_shape(M, N, K);
-    if (s.bytes > ((size_t)2 << 30) || s.mt * s.nt > (1 << 24)) return false;
-    return 1.0 * M * N * K > 2.0e6;
-}
+namespace {
 
-void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z64 *C, bool accumulate, cudaStream_t st,
-             bool neg) {
-    const Shape s = oz_shape(d.M, d.N, d.K);
-    const int nkb = (int)((d.K + 15) / 16);
-    const size_t na = (size_t)s.mt * nkb * OZ_A_STAGE, nbb = (size_t)s.nt * nkb * OZ_B_STAGE;
-    DevBuf<unsigned char> own;
-    DevBuf<int> own_err;
-    unsigned char *ws;
-    int *err;
-    if (g_oz) {
-        if (g_oz->buf.n < s.bytes) g_oz->buf.alloc(s.bytes);
-        ws = g_oz->buf.p;
-        err = g_oz->err;
-    } else {
-        own.alloc(s.bytes);
-        own_err.alloc(1);
-        CBFM_CUDA(cudaMemsetAsync(own_err.p, 0, sizeof(int), st));
-        ws = own.p;
-        err = own_err.p;
-    }
-    int *E = reinterpret_cast<int *>(ws + na + nbb);
-    // rows of op(A) and columns of op(B) with their strides along K
-    const bool rowA = opA == 0 || opA == 3, rowB = opB == 0 || opB == 3;
-    OzPack a{A, d.a_off, rowA ? d.lda : 1, rowA ? 1 : d.lda, opA >= 2, (int)d.M, 0, 0, nullptr, nullptr};
-    OzPack b{B, d.b_off, rowB ? 1 : d.ldb, rowB ? d.ldb : 1, opB >= 2, (int)d.N, 0, 0, nullptr, nullptr};
-    OzPack2 pp;
-    pp.p[0] = s.swap ? b : a;
-    pp.p[1] = s.swap ? a : b;
-    pp.p[0].groups = (int)(s.mt * OZ_M / 8);
-    pp.p[0].out = ws;
-    pp.p[0].E = E;
-    pp.p[1].groups = (int)(s.nt * OZ_NC / 8);
-    pp.p[1].expand = 1;
-    pp.p[1].out = ws + na;
-    pp.p[1].E = E + s.mt * OZ_M;
-    pp.K = (int)d.K;
-    pp.nkb = nkb;
-    {
-        ProfScope ps_("k_oz_pack", st);
-        k_oz_pack<<<pp.p[0].groups + pp.p[1].groups, 32 * PK_WARPS, 0, st>>>(pp);
-        launched("k_oz_pack");
-    }
-    OzArgs g;
-    g.A = ws;
-    g.B = ws + na;
-    g.EA = E;
-    g.EB = E + s.mt * OZ_M;
-    g.C = C + d.c_off;
-    g.ldc = d.ldc;
-    g.rows = (int)s.rows;
-    g.cols = (int)s.cols;
-    g.nkb = nkb;
-    g.tn = (int)s.nt;
-    g.swap = s.swap;
-    g.accumulate = accumulate;
-    g.neg = neg;
-    g.err = err;
+// 8-row groups of an operand: the left one padded to OZ_M rows per tile, the right one to OZ_NC complex columns
+OzPack pack_of(const void *X, bool f32, int64_t off, int64_t rs, int64_t cs, bool conj, int64_t rows, bool right,
+               uint8_t *out, int *E) {
+    OzPack p;
+    p.X = X;
+    p.off = off;
+    p.rs = rs;
+    p.cs = cs;
+    p.conj = conj;
+    p.f32 = f32;
+    p.rows = (int)rows;
+    const int64_t t = right ? OZ_NC : OZ_M;
+    p.groups = (int)((rows + t - 1) / t * t / 8);
+    p.expand = right;
+    p.out = out;
+    p.E = E;
+    return p;
+}
+OzPack pack_a(const GemmDesc &d, int op, const z64 *A, bool right, uint8_t *out, int *E) {   // rows of op(A)
+    const bool row = op == 0 || op == 3;
+    return pack_of(A, false, d.a_off, row ? d.lda : 1, row ? 1 : d.lda, op >= 2, d.M, right, out, E);
+}
+OzPack pack_b(const GemmDesc &d, int op, const z64 *B, bool right, uint8_t *out, int *E) {   // columns of op(B)
+    const bool row = op == 0 || op == 3;
+    return pack_of(B, false, d.b_off, row ? 1 : d.ldb, row ? d.ldb : 1, op >= 2, d.N, right, out, E);
+}
+void launch_pack(const OzPack *p, int np, int64_t K, cudaStream_t st) {
+    OzPack2 pp{};
+    for (int i = 0; i < np; ++i) pp.p[i] = p[i];
+    pp.K = (int)K;
+    pp.nkb = (int)((K + 15) / 16);
+    int g = p[0].groups + (np > 1 ? p[1].groups : 0);
+    ProfScope ps_("k_oz_pack", st);
+    k_oz_pack<<<g, 32 * PK_WARPS, 0, st>>>(pp);
+    launched("k_oz_pack");
+}
+void launch_gemm(OzArgs g, int64_t mt, cudaStream_t st) {
     // CTAs per tile: the K stages are shared while the tiles leave SMs idle, down to one drain's worth of stages
-    const int64_t tiles = s.mt * s.nt;
+    const int64_t tiles = mt * g.tn;
     int cs = 1;
-    while (cs < 8 && tiles * cs * 2 <= sm_count() && nkb >= 2 * OZ_CHUNK * cs) cs *= 2;
+    while (cs < 8 && tiles * cs * 2 <= sm_count() && g.nkb >= 2 * OZ_CHUNK * cs) cs *= 2;
     g.cs = cs;
     set_smem_once(k_oz_gemm, OZ_SMEM);
     cudaLaunchConfig_t cfg = {};
@@ -626,18 +610,94 @@ void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z6
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    {
-        prof_add_work("k_oz_gemm", 8.0 * d.M * d.N * d.K, 16.0 * (d.M * d.K + d.K * d.N + d.M * d.N));
-        ProfScope ps_("k_oz_gemm", st);
-        CBFM_CUDA(cudaLaunchKernelEx(&cfg, k_oz_gemm, g));
-        launched("k_oz_gemm");
+    ProfScope ps_("k_oz_gemm", st);
+    CBFM_CUDA(cudaLaunchKernelEx(&cfg, k_oz_gemm, g));
+    launched("k_oz_gemm");
+}
+// this thread's scratch of at least `bytes`, or a buffer of the call's own
+struct Scratch {
+    DevBuf<unsigned char> own;
+    DevBuf<int> own_err;
+    unsigned char *p;
+    int *err;
+    cudaStream_t st;
+    Scratch(size_t bytes, cudaStream_t s) : st(s) {
+        if (g_oz) {
+            if (g_oz->buf.n < bytes) g_oz->buf.alloc(bytes);
+            p = g_oz->buf.p;
+            err = g_oz->err;
+        } else {
+            own.alloc(bytes);
+            own_err.alloc(1);
+            CBFM_CUDA(cudaMemsetAsync(own_err.p, 0, sizeof(int), st));
+            p = own.p;
+            err = own_err.p;
+        }
     }
-    if (!g_oz) {
+    void check() {   // without an OzWork: wait and report
+        if (g_oz) return;
         int h = 0;
         CBFM_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaStreamSynchronize(st));
         if (h) throw Fail{CBFM_ETIMEOUT, "tensor-core FP64 product: a device wait expired"};
     }
+};
+
+}  // namespace
+
+bool oz_takes(int64_t M, int64_t N, int64_t K) {
+    if (g_oz_hold || M < 1 || N < 1 || K < 1 || M > (1 << 24) || N > (1 << 24) || K > (1 << 18)) return false;
+    const Shape s = oz_shape(M, N, K);
+    if (s.bytes > ((size_t)2 << 30) || s.mt * s.nt > (1 << 24)) return false;
+    return 1.0 * M * N * K > 2.0e6;
+}
+
+void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z64 *C, bool accumulate, cudaStream_t st,
+             bool neg) {
+    const Shape s = oz_shape(d.M, d.N, d.K);
+    const int nkb = (int)((d.K + 15) / 16);
+    const size_t na = (size_t)s.mt * nkb * OZ_A_STAGE, nbb = (size_t)s.nt * nkb * OZ_B_STAGE;
+    Scratch ws(s.bytes, st);
+    int *EA = reinterpret_cast<int *>(ws.p + na + nbb), *EB = EA + s.mt * OZ_M;
+    OzPack p[2];
+    if (s.swap) {
+        p[0] = pack_b(d, opB, B, false, ws.p, EA);
+        p[1] = pack_a(d, opA, A, true, ws.p + na, EB);
+    } else {
+        p[0] = pack_a(d, opA, A, false, ws.p, EA);
+        p[1] = pack_b(d, opB, B, true, ws.p + na, EB);
+    }
+    prof_add_work("k_oz_gemm", 8.0 * d.M * d.N * d.K, 16.0 * (d.M * d.K + d.K * d.N + d.M * d.N));
+    launch_pack(p, 2, d.K, st);
+    launch_gemm(OzArgs{ws.p, ws.p + na, EA, EB, C + d.c_off, d.ldc, (int)s.rows, (int)s.cols, nkb, (int)s.nt, 1,
+                       s.swap ? 1 : 0, accumulate ? 1 : 0, neg ? 1 : 0, ws.err},
+                s.mt, st);
+    ws.check();
+}
+
+void OzMat::pack(const void *X, bool f32, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st) {
+    rows = n_rows;
+    K = n_k;
+    const int64_t mt = (rows + OZ_M - 1) / OZ_M;
+    const size_t na = (size_t)mt * ((K + 15) / 16) * OZ_A_STAGE;
+    buf.alloc(na + 4 * (size_t)(mt * OZ_M));
+    const OzPack p = pack_of(X, f32, 0, ld, 1, false, rows, false, buf.p, reinterpret_cast<int *>(buf.p + na));
+    launch_pack(&p, 1, K, st);
+}
+
+void gemm_oz_rows(const OzMat &M, const z64 *in, int64_t ldi, z64 *out, int64_t ldo, int64_t n, cudaStream_t st) {
+    const int64_t mt = (M.rows + OZ_M - 1) / OZ_M, nt = (n + OZ_NC - 1) / OZ_NC;
+    const int nkb = (int)((M.K + 15) / 16);
+    const size_t na = (size_t)mt * nkb * OZ_A_STAGE, nbb = (size_t)nt * nkb * OZ_B_STAGE;
+    Scratch ws(nbb + 4 * (size_t)(nt * OZ_NC), st);
+    int *EB = reinterpret_cast<int *>(ws.p + nbb);
+    const OzPack p = pack_of(in, false, 0, ldi, 1, false, n, true, ws.p, EB);
+    prof_add_work("k_oz_gemm", 8.0 * M.rows * n * M.K, 16.0 * (M.rows * M.K + n * (M.rows + M.K)));
+    launch_pack(&p, 1, M.K, st);
+    launch_gemm(OzArgs{M.buf.p, ws.p, reinterpret_cast<const int *>(M.buf.p + na), EB, out, ldo, (int)M.rows, (int)n,
+                       nkb, (int)nt, 1, 1, 0, 0, ws.err},
+                mt, st);
+    ws.check();
 }
 
 }  // namespace cbfm
