@@ -208,9 +208,6 @@ struct GmresOut {
     std::vector<int> iters;
     std::vector<double> resid;
 };
-// out[r] = M in[r] for rows with mask[r] != 0 (M32 != NULL: complex64 / FP32 arithmetic)
-void apply_rows(const Red &rd, const z64 *M64, const c32 *M32, const z64 *in, z64 *out, int nrhs, const int *mask,
-                cudaStream_t st);
 GmresOut gmres_solve(Red &r, const z64 *d_b, int nrhs, double tol, int maxit, int restart, int pc,
                      z64 *d_x, cudaStream_t st);
 // Block GMRES over all right-hand sides at once (k_bgmres.cu); maxit counts block iterations,
