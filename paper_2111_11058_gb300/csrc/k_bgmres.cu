@@ -978,9 +978,9 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     // reduced system amplifies them: with the CBFs' singular values spread over SPREAD_MAX and more (tiny triangles
     // beside large ones) the currents move by 1e-5 of their norm and 1e-3 of their rms at single edges when the
     // sums of the basis are only reordered (1.5e-6 and 6e-5 where the spread is below 5e3).  Those systems keep the FP64 units' sums for the basis
-    // and the FP32 solution update, so that their results stay reproducible; everything else goes to the tensor
-    // cores.
-    const bool tc_basis = rd.prec == CBFM_FP64 || (pc == CBFM_PC_CMP && rd.gram_spread <= SPREAD_MAX);
+    // and the FP32 solution update, so that their results stay reproducible, and so do the slowly converging
+    // systems without the CMP; everything else goes to the tensor cores.
+    const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.gram_spread <= SPREAD_MAX);
     OzMat op;   // FP64 operator cut into digits once per solve
     auto applyB = [&](const z64 *in, z64 *out, int rows) {
         if (pc == CBFM_PC_CMP_INEXACT) {
@@ -988,7 +988,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             cmp_inner_apply(rd, in, zin.p, rows, st);
             in = zin.p;
         }
-        if (rd.prec == CBFM_FP64 && oz_takes(rows, n, n)) {
+        if (tc_basis && rd.prec == CBFM_FP64 && oz_takes(rows, n, n)) {
             if (op.rows == 0) op.pack(pc_op64(rd, pc), false, n, n, n, st);
             GemmSite site_("site:operator");
             gemm_oz_rows(op, in, n, out, n, rows, st);

@@ -12,6 +12,7 @@
 // cancelled strongly (||w_after|| < ||w_before|| / sqrt 2, the Daniel-Gragg-
 // Kaufman-Stewart criterion).
 #include <algorithm>
+#include <atomic>
 #include <vector>
 
 #include "internal.cuh"
@@ -21,7 +22,16 @@ namespace cbfm {
 namespace {
 
 constexpr int JB = 8;          // basis vectors per block in k_dots
-constexpr double DGKS_ETA2 = 0.5;   // (1 / sqrt 2)^2
+
+// Two orders of the FP64 sums.  The slowly converging systems without the CMP
+// (the conventional MoM, restarted every few hundred steps) carry a change of
+// rounding through hundreds of steps: their iterates, stopped at the same
+// tolerance, move by up to 1e-4 of the currents when only the order of a sum
+// changes.  They keep one fixed order (ORD: k_dots<true>, k_orth_ord, k_update_y, k_finish_ord,
+// k_matvec64_ord; four partial sums over the basis, one over the columns of the
+// product), so that results stay reproducible; the systems with the CMP, which
+// do not amplify it (1e-13), take the faster order.
+constexpr double DGKS_ETA = 0.70710678118654752, DGKS_ETA2 = 0.5;   // 1 / sqrt 2 and its square
 
 __device__ __forceinline__ double block_sum(double v, double *sh) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -49,6 +59,7 @@ __device__ __forceinline__ double warp_total(const double *__restrict__ p, int n
 // nrm2.  Second pass: only where the first cancelled strongly, ||w||^2 after
 // it (the sum of part[r][0..nc)) below DGKS_ETA2 nrm2; the x == 0 blocks
 // store that decision in flag and count the work (reo_work += k + 1).
+template <bool ORD>
 __global__ void __launch_bounds__(32 * JB) k_dots(int64_t n, int nrhs, int k, const z64 *__restrict__ V,
                                                   const z64 *__restrict__ w, z64 *__restrict__ h, int hld,
                                                   const int *__restrict__ done, double *__restrict__ nrm2,
@@ -59,7 +70,13 @@ __global__ void __launch_bounds__(32 * JB) k_dots(int64_t n, int nrhs, int k, co
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (part) {
         __shared__ int s_again;
-        if (warp == 0) {
+        if (ORD) {   // the sum over w itself, in the order of k_finish_ord
+            double s = 0;
+            for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += norm2(w[(int64_t)r * n + i]);
+            __shared__ double sh[32];
+            s = block_sum(s, sh);
+            if (threadIdx.x == 0) s_again = sqrt(s) < DGKS_ETA * sqrt(nrm2[r]);
+        } else if (warp == 0) {
             const double s = warp_total(part + (int64_t)r * nc, nc);
             if (lane == 0) s_again = s < DGKS_ETA2 * nrm2[r];
         }
@@ -81,12 +98,22 @@ __global__ void __launch_bounds__(32 * JB) k_dots(int64_t n, int nrhs, int k, co
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const z64 a = v[i + 32 * u], b = x[i + 32 * u];
+                if (ORD) {
+                    re[u] += a.re * b.re + a.im * b.im;
+                    im[u] += a.re * b.im - a.im * b.re;
+                    continue;
+                }
                 re[u] = fma(a.im, b.im, fma(a.re, b.re, re[u]));   // written as a sum it is a product, an FMA and an add
                 im[u] = fma(-a.im, b.re, fma(a.re, b.im, im[u]));
             }
         }
         for (; i < n; i += 32) {
             const z64 a = v[i], b = x[i];
+            if (ORD) {
+                re[0] += a.re * b.re + a.im * b.im;
+                im[0] += a.re * b.im - a.im * b.re;
+                continue;
+            }
             re[0] = fma(a.im, b.im, fma(a.re, b.re, re[0]));
             im[0] = fma(-a.im, b.re, fma(a.re, b.im, im[0]));
         }
@@ -109,6 +136,62 @@ __global__ void __launch_bounds__(32 * JB) k_dots(int64_t n, int nrhs, int k, co
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) nrm2[r] = s;
     }
+}
+
+// ORD: w[r][i] -= sum_{j<=k} V[j][r][i] h[r][j] for the rows with mask[r] == want, in four partial sums over j = u, u +
+// 4, ... (the last k + 1 mod 4 terms in the first one, which starts at w), added as (0 + 1) + (2 + 3).  A warp takes one
+// partial sum of 32 entries, a block all four: four times the blocks of a thread that walks all of an entry's
+// terms, for small systems, and the same FP64 work, which bounds it on large ones (two lanes per entry, one for each
+// component, loaded every basis element twice: 99 us against 78 at n = 2304, 32 right-hand sides).
+__global__ void __launch_bounds__(128) k_orth_ord(int64_t n, int nrhs, int k, const z64 *__restrict__ V,
+                                                  const z64 *__restrict__ h, int hld, const int *__restrict__ mask,
+                                                  int want, z64 *__restrict__ w) {
+    const int r = blockIdx.y;
+    if (mask[r] != want) return;
+    const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 32LL + lane;
+    __shared__ z64 s_acc[3][32];
+    const z64 *hr = h + (int64_t)r * hld;
+    z64 acc(0, 0);
+    if (i < n) {
+        const z64 *v = V + (int64_t)r * n + i;
+        const int64_t stride = (int64_t)nrhs * n;
+        if (u == 0) acc = w[(int64_t)r * n + i];
+        auto sub = [&](z64 a, z64 b) {
+            acc.re = __dsub_rn(acc.re, fma(a.re, b.re, -__dmul_rn(a.im, b.im)));
+            acc.im = __dsub_rn(acc.im, fma(a.im, b.re, __dmul_rn(a.re, b.im)));
+        };
+        const int kmain = (k + 1) & ~3;
+        int j = u;
+        for (; j + 12 < kmain; j += 16) {
+            z64 a[4], b[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                a[q] = v[(j + 4 * q) * stride];
+                b[q] = hr[j + 4 * q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sub(a[q], b[q]);
+        }
+        for (; j < kmain; j += 4) sub(v[j * stride], hr[j]);
+        if (u == 0)
+            for (j = kmain; j <= k; ++j) sub(v[j * stride], hr[j]);
+    }
+    if (u > 0) s_acc[u - 1][lane] = acc;
+    __syncthreads();
+    if (u == 0 && i < n) w[(int64_t)r * n + i] = (acc + s_acc[0][lane]) + (s_acc[1][lane] + s_acc[2][lane]);
+}
+
+// ORD: y[rhs] += sum_{j < kc} z_j V[j][rhs], ascending j
+__global__ void k_update_y(int64_t n, int nrhs, int m, const z64 *__restrict__ V, const z64 *__restrict__ z,
+                           const int *__restrict__ kconv, const int *__restrict__ active, z64 *__restrict__ y) {
+    const int r = blockIdx.y;
+    if (!active[r]) return;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    z64 acc = y[(int64_t)r * n + i];
+    for (int j = 0; j < kconv[r]; ++j) acc += V[((int64_t)j * nrhs + r) * n + i] * z[(int64_t)r * m + j];
+    y[(int64_t)r * n + i] = acc;
 }
 
 // w[r][i] += sgn sum_{j < cnt[r] or m} V[j][r][i] h[r][j] for the rows with
@@ -199,46 +282,51 @@ __device__ __forceinline__ void affine_after(z64 &A, z64 &B, z64 A1, z64 B1) {  
     B = b;
     A = A * A1;
 }
-__global__ void __launch_bounds__(256) k_finish(int64_t n, int nrhs, int k, int m, int last,
-                                                const z64 *__restrict__ h1, const z64 *__restrict__ h2,
-                                                int *__restrict__ flag, int hld, z64 *__restrict__ H,
-                                                double *__restrict__ cs, z64 *__restrict__ sn, z64 *__restrict__ g,
-                                                const double *__restrict__ bnorm, double tol, int *__restrict__ done,
-                                                int *__restrict__ kconv, double *__restrict__ resid,
-                                                int *__restrict__ n_active, const double *__restrict__ part1,
-                                                const double *__restrict__ part2, int nc, const z64 *__restrict__ w,
-                                                z64 *__restrict__ V, c32 *__restrict__ x32) {
-    const int r = blockIdx.x;
-    if (done[r]) return;
-    __shared__ z64 col[1024];
-    __shared__ z64 s_A[4], s_B[4];
-    __shared__ double s_nrm;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool re = flag[r] != 0;
-    for (int j = tid; j <= k; j += blockDim.x) {
-        z64 v = h1[(int64_t)r * hld + j];
-        if (re) v += h2[(int64_t)r * hld + j];
-        col[j] = v;
+struct RotState {   // one right-hand side's least-squares state of a cycle (see gmres_solve)
+    z64 *H, *sn, *g;
+    double *cs, *resid;
+    const double *bnorm;
+    int *done, *flag, *kconv, *n_active;   // flag, n_active: NULL in the cluster kernel
+    double tol;
+};
+// The new rotation that zeroes (a, nrm) in column k, the residual and the convergence test (one thread).
+__device__ __forceinline__ void new_rotation(const RotState &S, int r, int k, int m, int last, double nrm, z64 a) {
+    z64 *Hr = S.H + (int64_t)r * (m + 1) * m;
+    z64 *gr = S.g + (int64_t)r * (m + 1);
+    // new rotation zeroing (a, nrm)
+    double na = sqrt(norm2(a)), nb = nrm;
+    double cc;
+    z64 ss;
+    if (nb == 0.0) { cc = 1.0; ss = z64(0, 0); }
+    else if (na == 0.0) { cc = 0.0; ss = z64(1, 0); }
+    else {
+        double t = sqrt(na * na + nb * nb);
+        cc = na / t;
+        ss = a * (nb / (na * t));            // (a/|a|) nb / t, nb real
     }
-    if (warp == 4) {
-        const double s = sqrt(warp_total((re ? part2 : part1) + (int64_t)r * nc, nc));
-        if (lane == 0) s_nrm = s;
+    S.cs[(int64_t)r * m + k] = cc;
+    S.sn[(int64_t)r * m + k] = ss;
+    Hr[(int64_t)k * m + k] = cc * a + ss * nb;
+    z64 gk = gr[k];
+    gr[k] = cc * gk;
+    gr[k + 1] = -(conj(ss) * gk);
+    double res = sqrt(norm2(gr[k + 1])) / S.bnorm[r];
+    S.resid[r] = res;
+    if (res <= S.tol || nb == 0.0 || last) {
+        S.kconv[r] = k + 1;
+        S.done[r] = res <= S.tol || nb == 0.0 ? 1 : 2;
+        if (S.flag) S.flag[r] = 0;
+    } else if (S.n_active) {
+        atomicAdd(S.n_active + k, 1);
     }
-    __syncthreads();
-    const double nrm = s_nrm;
-    if (warp >= 4) {
-        const double inv = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-        const z64 *x = w + (int64_t)r * n;
-        z64 *vn = V + ((int64_t)(k + 1) * nrhs + r) * n;
-        for (int64_t i = tid - 128; i < n; i += 128) {
-            const z64 v = x[i] * inv;
-            vn[i] = v;
-            if (x32) x32[(int64_t)r * n + i] = c32((float)v.re, (float)v.im);
-        }
-        return;
-    }
-    const double *cr = cs + (int64_t)r * m;
-    const z64 *sr = sn + (int64_t)r * m;
+}
+// Column k (col[0..k], shared) and the norm of the new vector through the previous rotations and a new one; called by
+// FIN_LANES threads (four whole warps, named barrier 1).
+__device__ __forceinline__ void rotate_column(const RotState &S, int r, int k, int m, int last, double nrm, int tid,
+                                              const z64 *col, z64 *s_A, z64 *s_B) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const double *cr = S.cs + (int64_t)r * m;
+    const z64 *sr = S.sn + (int64_t)r * m;
     const int chunk = (k + FIN_LANES - 1) / FIN_LANES, j0 = min(k, tid * chunk), j1 = min(k, j0 + chunk);
     const z64 a0 = col[0];
     z64 A(1, 0), B(0, 0);
@@ -274,7 +362,7 @@ __global__ void __launch_bounds__(256) k_finish(int64_t n, int nrhs, int k, int 
             a = t;
         }
     }
-    z64 *Hr = H + (int64_t)r * (m + 1) * m;
+    z64 *Hr = S.H + (int64_t)r * (m + 1) * m;
     for (int j = j0; j < j1; ++j) {
         const z64 b = col[j + 1];
         const double c = cr[j];
@@ -286,37 +374,105 @@ __global__ void __launch_bounds__(256) k_finish(int64_t n, int nrhs, int k, int 
     }
     // the lane whose chunk ends at k holds a_k (lane 0 when there is no rotation yet)
     if (k == 0 ? tid == 0 : (j0 < k && j1 == k)) {
-        z64 *gr = g + (int64_t)r * (m + 1);
-        // new rotation zeroing (a, nrm)
-        double na = sqrt(norm2(a)), nb = nrm;
-        double cc;
-        z64 ss;
-        if (nb == 0.0) { cc = 1.0; ss = z64(0, 0); }
-        else if (na == 0.0) { cc = 0.0; ss = z64(1, 0); }
-        else {
-            double t = sqrt(na * na + nb * nb);
-            cc = na / t;
-            ss = a * (nb / (na * t));            // (a/|a|) nb / t, nb real
+        new_rotation(S, r, k, m, last, nrm, a);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_finish(int64_t n, int nrhs, int k, int m, int last,
+                                                const z64 *__restrict__ h1, const z64 *__restrict__ h2, int hld,
+                                                const __grid_constant__ RotState S, const double *__restrict__ part1,
+                                                const double *__restrict__ part2, int nc, const z64 *__restrict__ w,
+                                                z64 *__restrict__ V, c32 *__restrict__ x32) {
+    const int r = blockIdx.x;
+    if (S.done[r]) return;
+    __shared__ z64 col[1024];
+    __shared__ z64 s_A[4], s_B[4];
+    __shared__ double s_nrm;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool re = S.flag[r] != 0;
+    for (int j = tid; j <= k; j += blockDim.x) {
+        z64 v = h1[(int64_t)r * hld + j];
+        if (re) v += h2[(int64_t)r * hld + j];
+        col[j] = v;
+    }
+    if (warp == 4) {
+        const double s = sqrt(warp_total((re ? part2 : part1) + (int64_t)r * nc, nc));
+        if (lane == 0) s_nrm = s;
+    }
+    __syncthreads();
+    const double nrm = s_nrm;
+    if (warp >= 4) {
+        const double inv = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+        const z64 *x = w + (int64_t)r * n;
+        z64 *vn = V + ((int64_t)(k + 1) * nrhs + r) * n;
+        for (int64_t i = tid - 128; i < n; i += 128) {
+            const z64 v = x[i] * inv;
+            vn[i] = v;
+            if (x32) x32[(int64_t)r * n + i] = c32((float)v.re, (float)v.im);
         }
-        cs[(int64_t)r * m + k] = cc;
-        sn[(int64_t)r * m + k] = ss;
-        Hr[(int64_t)k * m + k] = cc * a + ss * nb;
-        z64 gk = gr[k];
-        gr[k] = cc * gk;
-        gr[k + 1] = -(conj(ss) * gk);
-        double res = sqrt(norm2(gr[k + 1])) / bnorm[r];
-        resid[r] = res;
-        if (res <= tol || nb == 0.0) {
-            kconv[r] = k + 1;
-            done[r] = 1;
-            flag[r] = 0;
-        } else if (last) {
-            kconv[r] = k + 1;
-            done[r] = 2;
-            flag[r] = 0;
-        } else {
-            atomicAdd(n_active + k, 1);
+        return;
+    }
+    rotate_column(S, r, k, m, last, nrm, tid, col, s_A, s_B);
+}
+
+// ORD: column k and V[k+1] = w / ||w|| as k_finish, the norm and the rotations in one fixed order: a_{j+1} walked step by
+// step by two lanes (real and imaginary part: three dependent FP64 operations a step), col[j] = c_j a_j + s_j
+// col[j+1] by all threads afterwards.  Dynamic shared memory: finish_ord_smem(k).
+constexpr size_t finish_ord_smem(int k) { return (size_t)(k + 1) * (3 * sizeof(z64) + sizeof(double)); }
+__global__ void __launch_bounds__(256) k_finish_ord(int64_t n, int nrhs, int k, int m, int last,
+                                                    const z64 *__restrict__ h1, const z64 *__restrict__ h2, int hld,
+                                                    const __grid_constant__ RotState S, const z64 *__restrict__ w,
+                                                    z64 *__restrict__ V, c32 *__restrict__ x32) {
+    const int r = blockIdx.x;
+    if (S.done[r]) return;
+    extern __shared__ __align__(16) unsigned char fo_raw[];
+    z64 *col = reinterpret_cast<z64 *>(fo_raw), *av = col + k + 1, *ssn = av + k + 1;
+    double *scs = reinterpret_cast<double *>(ssn + k + 1);
+    __shared__ double sh[32], s_nrm;
+    const int tid = threadIdx.x;
+    const bool re = S.flag[r] != 0;
+    for (int j = tid; j <= k; j += blockDim.x) {
+        z64 v = h1[(int64_t)r * hld + j];
+        if (re) v += h2[(int64_t)r * hld + j];
+        col[j] = v;
+        if (j < k) {
+            scs[j] = S.cs[(int64_t)r * m + j];
+            ssn[j] = S.sn[(int64_t)r * m + j];
         }
+    }
+    const z64 *x = w + (int64_t)r * n;
+    double s = 0;
+    for (int64_t i = tid; i < n; i += blockDim.x) s += norm2(x[i]);
+    s = block_sum(s, sh);   // contains __syncthreads: col, scs and ssn are visible afterwards
+    if (tid == 0) s_nrm = sqrt(s);
+    __syncthreads();
+    const double nrm = s_nrm;
+    if (tid < 32) {
+        const int c = tid & 1;
+        double own = c == 0 ? col[0].re : col[0].im;
+        for (int j = 0; j < k; ++j) {
+            const double oth = __shfl_xor_sync(0xffffffffu, own, 1);
+            if (tid < 2) reinterpret_cast<double *>(av + j)[c] = own;
+            const double b = reinterpret_cast<const double *>(col + j + 1)[c];
+            const double x1 = fma(ssn[j].re, own, (c == 0 ? ssn[j].im : -ssn[j].im) * oth);   // conj(s) a
+            own = fma(scs[j], b, -x1);
+        }
+        const double oth = __shfl_xor_sync(0xffffffffu, own, 1);
+        if (tid == 0) new_rotation(S, r, k, m, last, nrm, z64(own, oth));
+    } else {
+        const double inv = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+        z64 *vn = V + ((int64_t)(k + 1) * nrhs + r) * n;
+        for (int64_t i = tid - 32; i < n; i += blockDim.x - 32) {
+            const z64 v = x[i] * inv;
+            vn[i] = v;
+            if (x32) x32[(int64_t)r * n + i] = c32((float)v.re, (float)v.im);
+        }
+    }
+    __syncthreads();
+    z64 *Hr = S.H + (int64_t)r * (m + 1) * m;
+    for (int j = tid; j < k; j += blockDim.x) {
+        const z64 a = av[j], b = col[j + 1];
+        Hr[(int64_t)j * m + k] = scs[j] * a + ssn[j] * b;
     }
 }
 
@@ -437,6 +593,335 @@ __global__ void __launch_bounds__(256) k_matvec64(int64_t n, int nrhs, const z64
     }
 }
 
+// ORD: the FP64 product with one sum over ascending k per component: a warp
+// takes 16 output rows (two lanes each, real and imaginary part) of one
+// right-hand side, four right-hand sides a block, both operands through a
+// three-stage cp.async pipeline.  Bound: the chain of 2 n dependent FP64 FMAs
+// (n = 960: 64 us; a thread with four outputs and both components took 520 us).
+constexpr int MO_K = 16, MO_PITCH = MO_K + 1, MO_R = 4;
+__global__ void __launch_bounds__(32 * MO_R) k_matvec64_ord(int64_t n, int nrhs, const z64 *__restrict__ M,
+                                                            const z64 *__restrict__ in, z64 *__restrict__ out,
+                                                            const int *__restrict__ done) {
+    __shared__ __align__(16) z64 Ms[MV_STAGES][MV_N][MO_PITCH];
+    __shared__ __align__(16) z64 Xs[MV_STAGES][MO_R][MO_PITCH];
+    const int tid = threadIdx.x, lane = tid & 31, row = lane >> 1, c = lane & 1, q = tid >> 5;
+    const int64_t r0 = (int64_t)blockIdx.y * MO_R, c0 = (int64_t)blockIdx.x * MV_N;
+    bool any = false;
+    for (int a = 0; a < MO_R; ++a) any |= r0 + a < nrhs && (!done || done[r0 + a] == 0);
+    if (!any) return;
+    const bool mine = r0 + q < nrhs && (!done || done[r0 + q] == 0);   // the same in a warp
+    const int nst = (int)((n + MO_K - 1) / MO_K);
+    auto fetch = [&](int s) {
+        if (s < nst) {
+            const int b = s % MV_STAGES;
+            for (int e = tid; e < (MV_N + MO_R) * MO_K; e += 32 * MO_R) {
+                const int rw = e / MO_K, kk = e % MO_K;
+                const int64_t kx = (int64_t)s * MO_K + kk;
+                if (rw < MV_N) {
+                    const bool live = c0 + rw < n && kx < n;
+                    cp16(&Ms[b][rw][kk], live ? M + (c0 + rw) * n + kx : M, live);
+                } else {
+                    const int64_t r = r0 + rw - MV_N;
+                    const bool live = r < nrhs && kx < n;
+                    cp16(&Xs[b][rw - MV_N][kk], live ? in + r * n + kx : in, live);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    double acc = 0.0;
+    for (int s = 0; s < MV_STAGES - 1; ++s) fetch(s);
+    for (int s = 0; s < nst; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(MV_STAGES - 2) : "memory");
+        __syncthreads();
+        fetch(s + MV_STAGES - 1);
+        const int b = s % MV_STAGES;
+        if (mine) {
+#pragma unroll
+            for (int kk = 0; kk < MO_K; ++kk) {
+                const z64 x = Xs[b][q][kk], e = Ms[b][row][kk];
+                acc = fma(x.re, c == 0 ? e.re : e.im, acc);
+                acc = fma(x.im, c == 0 ? -e.im : e.re, acc);
+            }
+        }
+    }
+    if (mine && c0 + row < n) reinterpret_cast<double *>(out + (r0 + q) * n + c0 + row)[c] = acc;
+}
+
+// ------------------------------------------------- whole cycle on a cluster
+// The Arnoldi cycle of few right-hand sides of moderate order in one launch: a
+// cluster of CC CTAs per right-hand side.  As separate kernels an iteration is
+// six dependent launches of ~7 us that mostly wait (45 us at n = 222, one
+// right-hand side, whatever its work); here it is three hardware cluster
+// barriers (two more where the second Gram-Schmidt pass runs).  CTA c owns the
+// entries [c per, (c + 1) per) of w and of every basis vector.  Iteration k:
+//   x = V[k] = w / ||w|| staged in shared memory by every CTA (own entries written to V);
+//   own rows of w' = B x;                                                | barrier
+//   h_j = V[j]^H w', one warp per j over all warps of the cluster;       | barrier
+//   own entries w' -= sum_j V[j] h_j, partial norms;                     | barrier
+// The rotations of column k (four extra warps of CTA 0) run beside the product and
+// the dot products of iteration k + 1; a convergence is seen after its second
+// barrier, so the cycle runs at most one iteration too many.  Every thread of
+// the cluster reaches every barrier: all decisions are taken from values written
+// before the barrier ahead of them.
+// The complex64 product sums over ascending k in one thread per row, as the
+// kernels above do.
+constexpr int GC_WARPS = 8, GC_THREADS = 32 * GC_WARPS + FIN_LANES;
+constexpr int GC_NMAX = 1024, GC_CL = 16;
+constexpr int GC_K = 16, GC_PITCH = GC_K + 2;   // complex64 product: values of k per stage
+struct GmresCl {
+    int64_t n;
+    int nrhs, m, mc, hld;
+    const z64 *M64;
+    const c32 *M32;
+    z64 *V, *w, *h1, *h2;      // w: two buffers of nrhs x n; h1, h2: two buffers of nrhs x hld (by the parity of k)
+    double *part;              // nrhs x 2 (parity of k) x 3 x 16 partial norms: before, after the first, the second pass
+    unsigned long long *reo;
+    RotState rot;
+};
+__device__ __forceinline__ void cl_arrive_all() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait_all() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ z64 ldcg(const z64 *p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+    return z64(v.x, v.y);
+}
+
+template <bool F32>
+__global__ void __launch_bounds__(GC_THREADS) k_gmres_cl(const __grid_constant__ GmresCl P) {
+    constexpr int CC = GC_CL, ROWS = GC_NMAX / CC;   // most entries a CTA owns
+    __shared__ __align__(16) z64 x_s[F32 ? 1 : GC_NMAX];
+    __shared__ __align__(16) c32 x32_s[F32 ? GC_NMAX : 2];
+    __shared__ __align__(16) c32 Ms[F32 ? 2 : 1][F32 ? ROWS : 1][GC_PITCH];
+    __shared__ z64 s_acc[32 * GC_WARPS];
+    __shared__ double s_red[GC_WARPS];
+    __shared__ z64 col[1024], s_A[4], s_B[4];
+    const int r = blockIdx.x / CC, c = blockIdx.x % CC;
+    if (P.rot.done[r]) return;   // the whole cluster
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = (int)P.n;
+    const int per = (n + CC - 1) / CC, i0 = min(n, c * per), own = min(n, i0 + per) - i0;
+    const int64_t nn = (int64_t)P.nrhs * P.n;
+    const bool rotw = warp >= GC_WARPS;
+    int W = 8;                                     // entries per slot of the update
+    while (W < per) W <<= 1;
+    // sum of the CC partial norms p, in every thread
+    auto total = [&](const double *p) {
+        double s = lane < CC ? __ldcg(p + lane) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    };
+    auto cta_sync = [&] { asm volatile("bar.sync 2, 256;" ::: "memory"); };   // the GC_WARPS computing warps
+    double nrm = 0.0;
+    bool again = false;
+    for (int k = 0;; ++k) {
+        const bool fin = k == P.mc;   // the cycle is over: only the last column's rotations remain
+        double *part = P.part + ((int64_t)r * 2 + (k & 1)) * 3 * 16;
+        z64 *w = P.w + (int64_t)(k & 1) * nn + (int64_t)r * P.n;
+        const z64 *wp = P.w + (int64_t)((k & 1) ^ 1) * nn + (int64_t)r * P.n;
+        z64 *h1 = P.h1 + ((int64_t)(k & 1) * P.nrhs + r) * P.hld, *h2 = P.h2 + ((int64_t)(k & 1) * P.nrhs + r) * P.hld;
+        if (rotw) {
+            cl_arrive_all();
+            if (c == 0 && k > 0) {   // column k - 1
+                const z64 *g1 = P.h1 + ((int64_t)((k & 1) ^ 1) * P.nrhs + r) * P.hld;
+                const z64 *g2 = P.h2 + ((int64_t)((k & 1) ^ 1) * P.nrhs + r) * P.hld;
+                const int q = tid - 32 * GC_WARPS;
+                for (int j = q; j < k; j += FIN_LANES) {
+                    z64 v = ldcg(g1 + j);
+                    if (again) v += ldcg(g2 + j);
+                    col[j] = v;
+                }
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                rotate_column(P.rot, r, k - 1, P.m, fin ? 1 : 0, nrm, q, col, s_A, s_B);
+                __syncwarp();
+            }
+            cl_wait_all();
+            if (fin) break;
+            cl_arrive_all();
+            cl_wait_all();
+        } else {
+            if (fin) {
+                cl_arrive_all();
+                cl_wait_all();
+                break;
+            }
+            // x = V[k]
+            const double inv = k == 0 ? 1.0 : (nrm > 0.0 ? 1.0 / nrm : 0.0);
+            z64 *vk = P.V + ((int64_t)k * P.nrhs + r) * P.n;
+            for (int i = tid; i < n; i += 32 * GC_WARPS) {
+                z64 v = ldcg(k == 0 ? vk + i : wp + i);
+                if (k > 0) {
+                    v = v * inv;
+                    if (i >= i0 && i < i0 + own) vk[i] = v;
+                }
+                if (F32) x32_s[i] = c32((float)v.re, (float)v.im);
+                else x_s[i] = v;
+            }
+            cta_sync();
+            // own rows of the product, and their squared norm
+            double s2 = 0.0;
+            if (F32) {
+                const int nst = (n + GC_K - 1) / GC_K;
+                auto fetch = [&](int s) {
+                    if (s < nst)
+                        for (int q = tid; q < own * (GC_K / 2); q += 32 * GC_WARPS) {
+                            const int row = q / (GC_K / 2), cc = 2 * (q % (GC_K / 2)), kx = s * GC_K + cc;
+                            const bool live = kx < n;
+                            cp16(&Ms[s & 1][row][cc], P.M32 + (int64_t)(i0 + row) * n + (live ? kx : 0), live);
+                        }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                };
+                c32 acc(0, 0);
+                fetch(0);
+                for (int s = 0; s < nst; ++s) {
+                    fetch(s + 1);
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    cta_sync();
+                    if (tid < own) {
+                        const int ke = min(GC_K, n - s * GC_K);   // even
+                        const float4 *xp = reinterpret_cast<const float4 *>(x32_s + s * GC_K);
+#pragma unroll 8
+                        for (int kk = 0; kk < ke; kk += 2) {
+                            const float4 xv = xp[kk >> 1], mv = *reinterpret_cast<const float4 *>(&Ms[s & 1][tid][kk]);
+                            cfma(acc, c32(xv.x, xv.y), c32(mv.x, mv.y));
+                            cfma(acc, c32(xv.z, xv.w), c32(mv.z, mv.w));
+                        }
+                    }
+                    cta_sync();   // before stage s + 2 overwrites this one
+                }
+                if (tid < own) {
+                    const z64 v((double)acc.re, (double)acc.im);
+                    w[i0 + tid] = v;
+                    s2 = fma(v.re, v.re, v.im * v.im);
+                }
+            } else {
+                for (int i = warp; i < own; i += GC_WARPS) {
+                    const z64 *mr = P.M64 + (int64_t)(i0 + i) * n;
+                    z64 a0(0, 0), a1(0, 0);
+                    int kk = lane;
+                    for (; kk + 32 < n; kk += 64) {
+                        const z64 b0 = mr[kk], b1 = mr[kk + 32];
+                        cfma(a0, x_s[kk], b0);
+                        cfma(a1, x_s[kk + 32], b1);
+                    }
+                    if (kk < n) cfma(a0, x_s[kk], mr[kk]);
+                    a0 += a1;
+                    for (int o = 16; o > 0; o >>= 1) {
+                        a0.re += __shfl_xor_sync(0xffffffffu, a0.re, o);
+                        a0.im += __shfl_xor_sync(0xffffffffu, a0.im, o);
+                    }
+                    if (lane == 0) {
+                        w[i0 + i] = a0;
+                        s2 += fma(a0.re, a0.re, a0.im * a0.im);
+                    }
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+            if (lane == 0) s_red[warp] = s2;
+            cta_sync();
+            if (tid == 0) {
+                double t = 0.0;
+                for (int q = 0; q < GC_WARPS; ++q) t += s_red[q];
+                part[c] = t;
+            }
+            cl_arrive_all();
+            cl_wait_all();
+            // h_j = V[j]^H w
+            for (int pass = 0;; ++pass) {
+                z64 *h = pass == 0 ? h1 : h2;
+                for (int j = c * GC_WARPS + warp; j <= k; j += CC * GC_WARPS) {
+                    const z64 *v = P.V + ((int64_t)j * P.nrhs + r) * P.n;
+                    double re[2] = {0, 0}, im[2] = {0, 0};
+                    int i = lane;
+                    for (; i + 32 < n; i += 64) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const z64 a = ldcg(v + i + 32 * u), b = ldcg(w + i + 32 * u);
+                            re[u] = fma(a.im, b.im, fma(a.re, b.re, re[u]));
+                            im[u] = fma(-a.im, b.re, fma(a.re, b.im, im[u]));
+                        }
+                    }
+                    if (i < n) {
+                        const z64 a = ldcg(v + i), b = ldcg(w + i);
+                        re[0] = fma(a.im, b.im, fma(a.re, b.re, re[0]));
+                        im[0] = fma(-a.im, b.re, fma(a.re, b.im, im[0]));
+                    }
+                    double sr = re[0] + re[1], si = im[0] + im[1];
+                    for (int o = 16; o > 0; o >>= 1) {
+                        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+                        si += __shfl_xor_sync(0xffffffffu, si, o);
+                    }
+                    if (lane == 0) h[j] = z64(sr, si);
+                }
+                cl_arrive_all();
+                cl_wait_all();
+                if (pass == 0 && k > 0 && __ldcg(P.rot.done + r)) return;   // column k - 1 converged (all threads alike)
+                // own entries of w -= sum_j V[j] h_j
+                {
+                    const int i = tid % W, slot = tid / W, ns = 32 * GC_WARPS / W;
+                    double re[2] = {0, 0}, im[2] = {0, 0};
+                    if (i < own) {
+                        const z64 *v = P.V + (int64_t)r * P.n + i0 + i;
+                        const int64_t stride = (int64_t)P.nrhs * P.n;
+                        int j = slot;
+                        for (; j + ns <= k; j += 2 * ns) {
+                            const z64 a0 = ldcg(v + j * stride), a1 = ldcg(v + (j + ns) * stride);
+                            const z64 c0 = ldcg(h + j), c1 = ldcg(h + j + ns);
+                            re[0] = fma(-a0.im, c0.im, fma(a0.re, c0.re, re[0]));
+                            im[0] = fma(a0.im, c0.re, fma(a0.re, c0.im, im[0]));
+                            re[1] = fma(-a1.im, c1.im, fma(a1.re, c1.re, re[1]));
+                            im[1] = fma(a1.im, c1.re, fma(a1.re, c1.im, im[1]));
+                        }
+                        if (j <= k) {
+                            const z64 a0 = ldcg(v + j * stride), c0 = ldcg(h + j);
+                            re[0] = fma(-a0.im, c0.im, fma(a0.re, c0.re, re[0]));
+                            im[0] = fma(a0.im, c0.re, fma(a0.re, c0.im, im[0]));
+                        }
+                    }
+                    s_acc[tid] = z64(re[0] + re[1], im[0] + im[1]);
+                    cta_sync();
+                    double t2 = 0.0;
+                    if (tid < 2 * own) {
+                        const double *a = reinterpret_cast<const double *>(s_acc) + tid;
+                        double t = 0.0;
+                        for (int q = 0; q < ns; ++q) t += a[2 * W * q];
+                        double *p = reinterpret_cast<double *>(w + i0) + tid;
+                        t = __ldcg(p) - t;
+                        *p = t;
+                        t2 = t * t;
+                    }
+                    for (int o = 16; o > 0; o >>= 1) t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+                    if (lane == 0) s_red[warp] = t2;
+                    cta_sync();
+                    if (tid == 0) {
+                        double t = 0.0;
+                        for (int q = 0; q < GC_WARPS; ++q) t += s_red[q];
+                        part[16 * (1 + pass) + c] = t;
+                    }
+                }
+                cl_arrive_all();
+                cl_wait_all();
+                if (pass == 1) break;
+                // again where the first pass cancelled strongly
+                if (!(total(part + 16) < DGKS_ETA2 * total(part))) break;
+            }
+        }
+        if (rotw) {   // the same barriers and decisions as the computing warps
+            if (k > 0 && __ldcg(P.rot.done + r)) return;
+            cl_arrive_all();
+            cl_wait_all();
+        }
+        const double s1 = total(part + 16);
+        again = s1 < DGKS_ETA2 * total(part);
+        if (again && rotw)
+            for (int b = 0; b < 2; ++b) {
+                cl_arrive_all();
+                cl_wait_all();
+            }
+        nrm = sqrt(again ? total(part + 32) : s1);
+        if (again && c == 0 && tid == 0) atomicAdd(P.reo, (unsigned long long)(k + 1));
+    }
+}
+
 // Back-substitution H(0:kc,0:kc) z = g(0:kc), one block per rhs (column oriented).
 __global__ void k_backsolve(int nrhs, int m, const z64 *__restrict__ H, z64 *__restrict__ g,
                             const int *__restrict__ kconv, const int *__restrict__ active, z64 *__restrict__ z) {
@@ -507,7 +992,7 @@ __global__ void k_norms(int64_t n, int nrhs, const z64 *__restrict__ b, double *
 // out[r] = M in[r] for the rows with done[r] == 0 (NULL: all): M32 in complex64 with FP32 sums (in32: the rows rounded
 // to complex64, or NULL to round in here), else M64 in FP64
 static void apply_rows(int64_t n, const z64 *M64, const c32 *M32, const z64 *in, const c32 *in32, z64 *out, int nrhs,
-                       const int *done, cudaStream_t st) {
+                       const int *done, bool ord, cudaStream_t st) {
     DevBuf<c32> tmp;
     if (M32 && !in32) {
         tmp.alloc((size_t)nrhs * n);
@@ -521,6 +1006,9 @@ static void apply_rows(int64_t n, const z64 *M64, const c32 *M32, const z64 *in,
         // against 20 us of a half-empty 32 tile)
         if (nrhs <= 8) k_matvec32<8><<<dim3(gx, (unsigned)((nrhs + 7) / 8)), 128, 0, st>>>(n, nrhs, M32, in32, out, done);
         else k_matvec32<32><<<dim3(gx, (unsigned)((nrhs + 31) / 32)), 256, 0, st>>>(n, nrhs, M32, in32, out, done);
+    } else if (ord) {
+        const dim3 g((unsigned)((n + MV_N - 1) / MV_N), (unsigned)((nrhs + MO_R - 1) / MO_R));
+        k_matvec64_ord<<<g, 32 * MO_R, 0, st>>>(n, nrhs, M64, in, out, done);
     } else {
         const unsigned gx = (unsigned)((n + 7) / 8);
         if (nrhs == 1) k_matvec64<1><<<dim3(gx, 1), 256, 0, st>>>(n, nrhs, M64, in, out, done);
@@ -552,7 +1040,58 @@ static void apply_B(Red &rd, int pc, const z64 *in, const c32 *in32, z64 *out, i
         in32 = nullptr;
     }
     const bool mixed = rd.prec != CBFM_FP64;
-    apply_rows(rd.n, mixed ? nullptr : pc_op64(rd, pc), mixed ? pc_op32(rd, pc) : nullptr, in, in32, out, nrhs, done, st);
+    apply_rows(rd.n, mixed ? nullptr : pc_op64(rd, pc), mixed ? pc_op32(rd, pc) : nullptr, in, in32, out, nrhs, done,
+               pc != CBFM_PC_CMP, st);
+}
+
+static void set_finish_smem() {   // once per device: columns of up to 1023 entries
+    static std::atomic<bool> done[64];
+    int dev = 0;
+    CBFM_CUDA(cudaGetDevice(&dev));
+    if (dev < 64 && done[dev].load(std::memory_order_acquire)) return;
+    CBFM_CUDA(cudaFuncSetAttribute(k_finish_ord, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)finish_ord_smem(1023)));
+    if (dev < 64) done[dev].store(true, std::memory_order_release);
+}
+static cudaLaunchConfig_t gmres_cl_cfg(int nrhs, cudaStream_t st, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nrhs * GC_CL), 1, 1);
+    cfg.blockDim = dim3(GC_THREADS, 1, 1);
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = GC_CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+static void launch_gmres_cl(const GmresCl &P, bool f32, cudaStream_t st) {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = gmres_cl_cfg(P.nrhs, st, at);
+    if (f32) CBFM_CUDA(cudaLaunchKernelEx(&cfg, k_gmres_cl<true>, P));
+    else CBFM_CUDA(cudaLaunchKernelEx(&cfg, k_gmres_cl<false>, P));
+}
+// Clusters of the cycle kernel that can be resident at once on this device (0: none, the size is not portable).
+static int gmres_clusters(bool f32) {
+    static std::atomic<int> known[64][2];   // zero-initialised: 0 = not asked yet, else the count + 1
+    int dev = 0;
+    CBFM_CUDA(cudaGetDevice(&dev));
+    if (dev < 64) {
+        const int k = known[dev][f32].load(std::memory_order_acquire);
+        if (k) return k - 1;
+    }
+    int nc = 0;
+    auto ask = [&](auto *f) {
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return;
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = gmres_cl_cfg(1, 0, at);
+        if (cudaOccupancyMaxActiveClusters(&nc, f, &cfg) != cudaSuccess) nc = 0;
+    };
+    if (f32) ask(k_gmres_cl<true>);
+    else ask(k_gmres_cl<false>);
+    (void)cudaGetLastError();   // a refused non-portable size is not an error here
+    if (dev < 64) known[dev][f32].store(nc + 1, std::memory_order_release);
+    return nc;
 }
 
 GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, int restart, int pc, z64 *d_x,
@@ -614,6 +1153,20 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
     }
 
     const int hld = m + 1;
+    const RotState rot{H.p, sn.p, g.p, cs.p, resid.p, bnorm.p, done.p, flag.p, kconv.p, nact.p, tol};
+    // few right-hand sides of moderate order: a cluster each, if all are resident at once (n = 222, one: 12 us an
+    // iteration against 45 us of separate launches; at n = 1024 and 1000 steps both are bound by the FP64 pipes, of 16
+    // SMs and of all)
+    const bool ord = pc != CBFM_PC_CMP;
+    const bool cl = n <= GC_NMAX && !ord && nrhs <= gmres_clusters(rd.prec != CBFM_FP64);
+    DevBuf<z64> w2, hc;
+    DevBuf<double> partc;
+    if (cl) {
+        w2.alloc((size_t)2 * nrhs * n);
+        hc.alloc((size_t)4 * nrhs * hld);
+        partc.alloc((size_t)nrhs * 2 * 3 * 16);
+    }
+    if (ord) set_finish_smem();
     const int CHECK = 4;   // iterations between convergence polls
     std::vector<int> h_iters(nrhs, 0), h_done(nrhs, 0), h_kc(nrhs, 0), h_act(nrhs, 0);
     int total = 0;
@@ -640,7 +1193,16 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
         CBFM_CUDA(cudaMemsetAsync(nact.p, 0, sizeof(int) * (m + 1), st));
         const int mc = std::min(m, maxit - total);
         int k = 0;
-        for (; k < mc; ++k) {
+        if (cl) {
+            GmresCl P{n, nrhs, m, mc, hld, nullptr, nullptr, V.p, w2.p, hc.p, hc.p + 2 * (int64_t)nrhs * hld, partc.p, reo.p, rot};
+            P.rot.flag = P.rot.n_active = nullptr;
+            if (rd.prec != CBFM_FP64) P.M32 = pc_op32(rd, pc);
+            else P.M64 = pc_op64(rd, pc);
+            ProfScope ps_("k_gmres_cl", st);
+            launch_gmres_cl(P, rd.prec != CBFM_FP64, st);
+            launched("k_gmres_cl");
+        }
+        for (; !cl && k < mc; ++k) {
             const z64 *vk = V.p + (int64_t)k * nrhs * n;
             apply_B(rd, pc, vk, x32.p, w.p, nrhs, done.p, st);
             const dim3 gd((unsigned)((k + 1 + JB - 1) / JB), nrhs), gu((unsigned)nc, nrhs);
@@ -648,22 +1210,29 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
                 z64 *hb = pass == 0 ? hb1.p : hb2.p;
                 {
                     ProfScope ps_("k_dots", st);
-                    k_dots<<<gd, 32 * JB, 0, st>>>(n, nrhs, k, V.p, w.p, hb, hld, done.p, nrm0.p,
-                                                   pass == 0 ? nullptr : part1.p, nc, flag.p, reo.p);
+                    auto *f = ord ? k_dots<true> : k_dots<false>;
+                    f<<<gd, 32 * JB, 0, st>>>(n, nrhs, k, V.p, w.p, hb, hld, done.p, nrm0.p,
+                                              pass == 0 ? nullptr : part1.p, nc, flag.p, reo.p);
                     launched("k_dots");
                 }
                 ProfScope ps_("k_orth_update", st);
                 // the second pass on the rows k_dots flagged (a finished row's flag is zero)
-                k_combine<<<gu, 256, 0, st>>>(n, nrhs, k + 1, nullptr, V.p, hb, hld, pass == 0 ? done.p : flag.p, pass,
-                                              -1.0, w.p, pass == 0 ? part1.p : part2.p);
+                const int *mask = pass == 0 ? done.p : flag.p;
+                if (ord) k_orth_ord<<<gu, 128, 0, st>>>(n, nrhs, k, V.p, hb, hld, mask, pass, w.p);
+                else
+                    k_combine<<<gu, 256, 0, st>>>(n, nrhs, k + 1, nullptr, V.p, hb, hld, mask, pass, -1.0, w.p,
+                                                  pass == 0 ? part1.p : part2.p);
                 launched("k_orth_update");
             }
             const int last = (k + 1 == mc) ? 1 : 0;
             {
                 ProfScope ps_("k_finish", st);
-                k_finish<<<nrhs, 256, 0, st>>>(n, nrhs, k, m, last, hb1.p, hb2.p, flag.p, hld, H.p, cs.p, sn.p, g.p,
-                                               bnorm.p, tol, done.p, kconv.p, resid.p, nact.p, part1.p, part2.p, nc, w.p,
-                                               V.p, x32.p);
+                if (ord)
+                    k_finish_ord<<<nrhs, 256, finish_ord_smem(k), st>>>(n, nrhs, k, m, last, hb1.p, hb2.p, hld, rot, w.p,
+                                                                        V.p, x32.p);
+                else
+                    k_finish<<<nrhs, 256, 0, st>>>(n, nrhs, k, m, last, hb1.p, hb2.p, hld, rot, part1.p, part2.p, nc, w.p,
+                                                   V.p, x32.p);
                 launched("k_finish");
             }
             if ((k + 1) % CHECK == 0 || last) {
@@ -675,16 +1244,17 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
                 }
             }
         }
-        total += k;
         CBFM_CUDA(cudaMemcpyAsync(h_kc.data(), kconv.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaMemcpyAsync(h_done.data(), done.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaStreamSynchronize(st));
         for (int r = 0; r < nrhs; ++r)
             if (h_act[r]) {
+                if (cl) k = std::max(k, h_kc[r]);
                 h_iters[r] += h_kc[r];
                 pass1 += 0.5 * (double)h_kc[r] * (h_kc[r] + 1);
                 nmatvec += h_kc[r] + 1;
             }
+        total += k;
         {
             ProfScope ps_("k_backsolve", st);
             k_backsolve<<<nrhs, 128, 0, st>>>(nrhs, m, H.p, g.p, kconv.p, active.p, zs.p);
@@ -692,7 +1262,11 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
         }
         {
             ProfScope ps_("k_update_y", st);
-            k_combine<<<dim3((unsigned)nc, nrhs), 256, 0, st>>>(n, nrhs, 0, kconv.p, V.p, zs.p, m, active.p, 1, 1.0, y.p,
+            if (ord)
+                k_update_y<<<dim3((unsigned)((n + 255) / 256), nrhs), 256, 0, st>>>(n, nrhs, m, V.p, zs.p, kconv.p,
+                                                                                    active.p, y.p);
+            else
+                k_combine<<<dim3((unsigned)nc, nrhs), 256, 0, st>>>(n, nrhs, 0, kconv.p, V.p, zs.p, m, active.p, 1, 1.0, y.p,
                                                                 nullptr);
             launched("k_update_y");
         }
@@ -705,7 +1279,7 @@ GmresOut gmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, i
         CBFM_CUDA(cudaMemsetAsync(H.p, 0, sizeof(z64) * nrhs * (m + 1) * m, st));
     }
     // x = P y
-    if (pc == CBFM_PC_CMP) apply_rows(n, rd.Ginv.p, nullptr, y.p, nullptr, d_x, nrhs, nullptr, st);
+    if (pc == CBFM_PC_CMP) apply_rows(n, rd.Ginv.p, nullptr, y.p, nullptr, d_x, nrhs, nullptr, false, st);
     else if (pc == CBFM_PC_TDIAG) tdiag_recover(rd, y.p, d_x, nrhs, st);
     else if (pc == CBFM_PC_CMP_INEXACT) cmp_inner_apply(rd, y.p, d_x, nrhs, st);
     else CBFM_CUDA(cudaMemcpyAsync(d_x, y.p, sizeof(z64) * nrhs * n, cudaMemcpyDeviceToDevice, st));
