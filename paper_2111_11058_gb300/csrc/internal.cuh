@@ -123,6 +123,8 @@ void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> 
                   bool accumulate, cudaStream_t st, double alpha = 1.0);
 // Tensor-core form of one FP64 product (k_oz.cu): C = +-op(A) op(B) [+ C].  oz_takes: where it is the faster one.
 bool oz_takes(int64_t M, int64_t N, int64_t K);
+// one small product without tiles (k_dense.cu)
+bool dir_takes(const GemmDesc &d);
 void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z64 *C, bool accumulate, cudaStream_t st,
              bool neg);
 // Scratch and error word of the tensor-core products launched on this thread while an object is alive: the caller

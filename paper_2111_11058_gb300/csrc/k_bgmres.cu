@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <atomic>
 #include <vector>
 
@@ -537,11 +538,12 @@ GemmDesc sub_desc(GemmDesc d, int opA, int opB, int64_t r0, int64_t rows, int64_
 }
 constexpr int64_t TT = 32;   // tile edge of the FP64 product kernel
 // The splits below spare the FP64 units the zero part of a triangular or
-// Hermitian product.  A product the tensor cores take stays whole: there the second
-// packing of an operand costs more than the zeros (all operands hold them).
+// Hermitian product.  A product the tensor cores or the small kernels take stays
+// whole: a second packing of an operand or a second launch costs more than the
+// zeros (all operands hold them).
 // The block upper triangle (tiles on or above the diagonal) of a Hermitian square product
 std::vector<GemmDesc> upper_tiles(const GemmDesc &d, int opA, int opB) {
-    if (oz_takes(d.M, d.N, d.K)) return {d};
+    if (oz_takes(d.M, d.N, d.K) || dir_takes(d)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT)
         g.push_back(sub_desc(d, opA, opB, r0, std::min(TT, d.M - r0), r0, d.N - r0, 0, d.K));
@@ -549,7 +551,7 @@ std::vector<GemmDesc> upper_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(A) lower triangular (row i is zero beyond column i): row tiles summed up to their last row
 std::vector<GemmDesc> lower_a_tiles(const GemmDesc &d, int opA, int opB) {
-    if (oz_takes(d.M, d.N, d.K)) return {d};
+    if (oz_takes(d.M, d.N, d.K) || dir_takes(d)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT) {
         const int64_t rows = std::min(TT, d.M - r0);
@@ -559,7 +561,7 @@ std::vector<GemmDesc> lower_a_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(A) upper triangular (row i is zero before column i): row tiles summed from their first row
 std::vector<GemmDesc> upper_a_tiles(const GemmDesc &d, int opA, int opB) {
-    if (oz_takes(d.M, d.N, d.K)) return {d};
+    if (oz_takes(d.M, d.N, d.K) || dir_takes(d)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t r0 = 0; r0 < d.M; r0 += TT)
         if (r0 < d.K) g.push_back(sub_desc(d, opA, opB, r0, std::min(TT, d.M - r0), 0, d.N, r0, d.K - r0));
@@ -567,7 +569,7 @@ std::vector<GemmDesc> upper_a_tiles(const GemmDesc &d, int opA, int opB) {
 }
 // op(B) upper triangular (column j is zero below row j): column tiles summed up to their last column
 std::vector<GemmDesc> upper_b_tiles(const GemmDesc &d, int opA, int opB) {
-    if (oz_takes(d.M, d.N, d.K)) return {d};
+    if (oz_takes(d.M, d.N, d.K) || dir_takes(d)) return {d};
     std::vector<GemmDesc> g;
     for (int64_t c0 = 0; c0 < d.N; c0 += TT) {
         const int64_t cols = std::min(TT, d.N - c0);
@@ -578,10 +580,38 @@ std::vector<GemmDesc> upper_b_tiles(const GemmDesc &d, int opA, int opB) {
 
 inline unsigned nb(int64_t work) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 4096)); }
 
+// Small results the solver decides on: one copy to pinned memory kept per host thread, one wait, then to dst (a copy
+// to pageable memory is staged by the driver and waited for on its own, ~8 us each).
+void read_back(void *dst, const void *dev, size_t bytes, cudaStream_t st) {
+    struct Pinned {
+        void *p = nullptr;
+        size_t n = 0;
+        ~Pinned() {
+            if (p) cudaFreeHost(p);
+        }
+    };
+    static thread_local Pinned h;
+    if (h.n < bytes) {
+        if (h.p) cudaFreeHost(h.p);
+        h.p = nullptr;
+        h.n = 0;
+        CBFM_CUDA(cudaMallocHost(&h.p, std::max(bytes, (size_t)1 << 14)));
+        h.n = std::max(bytes, (size_t)1 << 14);
+    }
+    CBFM_CUDA(cudaMemcpyAsync(h.p, dev, bytes, cudaMemcpyDeviceToHost, st));
+    CBFM_CUDA(cudaStreamSynchronize(st));
+    std::memcpy(dst, h.p, bytes);
+}
+
 struct Ctx {
     cudaStream_t st;
     DevBuf<z64> M, R, Rinv, X, T1, Rf, Dinv;
-    DevBuf<int> perm, rank, err, status;
+    // one buffer, read back in one copy: rank, error word, status and the order of the last factorisation
+    DevBuf<int> info;
+    struct {
+        int *p;
+    } rank, err, status, perm;
+    static constexpr int INFO = 3 + PCHOL_MAX;
     DevBuf<double> rnrm, scale, dev;
     bool perm_id = true;   // the last factorisation kept the order (perm is the identity)
     std::vector<int> hperm;
@@ -610,8 +640,7 @@ double gram_dev(Ctx &c, int m) {
     k_gram_dev_sum<<<1, 32, 0, c.st>>>(c.dev.p + 1, c.dev.p);
     launched("k_gram_dev_sum");
     double h = 0.0;
-    CBFM_CUDA(cudaMemcpyAsync(&h, c.dev.p, sizeof(double), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaStreamSynchronize(c.st));
+    read_back(&h, c.dev.p, sizeof(double), c.st);
     return h;
 }
 
@@ -698,13 +727,9 @@ int pchol(Ctx &c, int m, double tol, bool pivot) {
         k_trinv_blk<<<m, 128, 0, c.st>>>(m, c.R.p, c.Dinv.p, c.rank.p, c.status.p, c.Rinv.p);
         launched("k_trinv_blk");
     }
-    int hr[3] = {0, 0, 0};
-    c.hperm.resize(m);
-    CBFM_CUDA(cudaMemcpyAsync(&hr[0], c.rank.p, sizeof(int), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaMemcpyAsync(&hr[1], c.err.p, sizeof(int), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaMemcpyAsync(&hr[2], c.status.p, sizeof(int), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaMemcpyAsync(c.hperm.data(), c.perm.p, sizeof(int) * m, cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaStreamSynchronize(c.st));
+    int hr[Ctx::INFO] = {};
+    read_back(hr, c.info.p, sizeof(int) * (3 + m), c.st);
+    c.hperm.assign(hr + 3, hr + 3 + m);
     if (hr[1]) throw Fail{CBFM_ETIMEOUT, "Cholesky: a cluster synchronisation expired"};
     c.perm_id = true;
     for (int i = 0; i < m; ++i) c.perm_id &= c.hperm[i] == i;
@@ -725,9 +750,7 @@ int pchol(Ctx &c, int m, double tol, bool pivot) {
         k_trinv<<<m, PCHOL_MAX, trinv_smem(m), c.st>>>(m, c.R.p, c.rank.p, c.Rinv.p);
         launched("k_trinv");
     }
-    CBFM_CUDA(cudaMemcpyAsync(&hr[0], c.rank.p, sizeof(int), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaMemcpyAsync(&hr[1], c.err.p, sizeof(int), cudaMemcpyDeviceToHost, c.st));
-    CBFM_CUDA(cudaStreamSynchronize(c.st));
+    read_back(hr, c.info.p, sizeof(int) * 2, c.st);
     if (hr[1]) throw Fail{CBFM_ETIMEOUT, "pivoted Cholesky: a cluster synchronisation expired"};
     return hr[0];
 }
@@ -745,8 +768,7 @@ int cholqr2_rows(Ctx &c, z64 *W, int m, int64_t n, z64 *Qdst, z64 *Rfull, double
     launched("k_rownorm");
     if (ref <= 0.0) {
         std::vector<double> h(m);
-        CBFM_CUDA(cudaMemcpyAsync(h.data(), c.rnrm.p, sizeof(double) * m, cudaMemcpyDeviceToHost, c.st));
-        CBFM_CUDA(cudaStreamSynchronize(c.st));
+        read_back(h.data(), c.rnrm.p, sizeof(double) * m, c.st);
         for (double v : h) ref = std::max(ref, v);
         if (ref <= 0.0) return 0;
     }
@@ -884,10 +906,11 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     c.Rinv.alloc((size_t)PCHOL_MAX * PCHOL_MAX);
     c.X.alloc((size_t)PCHOL_MAX * PCHOL_MAX);
     c.Rf.alloc((size_t)PCHOL_MAX * PCHOL_MAX);
-    c.perm.alloc(PCHOL_MAX);
-    c.rank.alloc(1);
-    c.err.alloc(1);
-    c.status.alloc(1);
+    c.info.alloc(Ctx::INFO);
+    c.rank.p = c.info.p;
+    c.err.p = c.info.p + 1;
+    c.status.p = c.info.p + 2;
+    c.perm.p = c.info.p + 3;
     c.Dinv.alloc((size_t)CH_NPAN * CH_B * CH_B);
     CBFM_CUDA(cudaMemsetAsync(c.err.p, 0, sizeof(int), st));
     OzWork oz_(c.err.p);   // scratch of the tensor-core products; their error word is read with the Cholesky's
@@ -895,13 +918,16 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     c.scale.alloc(PCHOL_MAX);
     c.dev.alloc(1 + GD_CTAS);   // the deviation and its per-CTA partials
     DevBuf<z64> V, W, HcT, Hn, Qh, Rh, Gv, E1S, Rv, Y, Z, tmp, tmp2, RinvBlk, Rw, Bm, Rout;
-    DevBuf<double> bnorm, rnorm, rnorm0, fro_col;
+    DevBuf<double> bnorm, norms, fro_col;   // norms: before, then after a pass (p each), read back together
+    struct {
+        double *p;
+    } rnorm0, rnorm;
     DevBuf<int> dmask, dsel;
     DevBuf<z64> Ws;            // the vectors of a selective second Gram-Schmidt pass
     DevBuf<c32> s_in, s_out;   // complex64 rows for the mixed-precision products
     DevBuf<c32> V32, Z32;      // complex64 basis and coefficients for the mixed-precision solution update
     DevBuf<z64> zin;           // inexact CMP: the inner GMRES's (G^CBF)^{-1} in, the input of the product with A
-    std::vector<double> h_bn, h_rn, h_w1, h_h0, h_h1, h_col;
+    std::vector<double> h_bn, h_rn, h_w1, h_h0, h_h1, h_col, h_two;
     auto setup = [&]() {
         dcap = std::max<int64_t>(2 * p, std::min<int64_t>((int64_t)std::max(restart, 2 * p), n + p));
         dcap2 = dcap + p;
@@ -922,8 +948,11 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
         RinvBlk.alloc((size_t)dcap * p);   // diagonal blocks of Rh^{-1}, stacked (p_j x p_j each, ld p)
         Rw.alloc((size_t)p * p);
         Rout.alloc((size_t)p * p);
-        rnorm.alloc(p);
-        rnorm0.alloc(p);
+        norms.alloc((size_t)2 * p);
+        CBFM_CUDA(cudaMemsetAsync(norms.p, 0, sizeof(double) * 2 * p, st));
+        rnorm0.p = norms.p;
+        rnorm.p = norms.p + p;
+        h_two.assign((size_t)2 * p, 0.0);
         fro_col.alloc((size_t)std::max<int64_t>(dcap, p));
         h_col.assign((size_t)std::max<int64_t>(dcap, p), 0.0);
         h_rn.assign(p, 0.0);
@@ -952,8 +981,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     auto fro = [&](int rows, int cols, const z64 *X, int64_t ld) {
         k_colnorm<<<cols, 256, 0, st>>>(rows, cols, X, ld, fro_col.p);
         launched("k_colnorm");
-        CBFM_CUDA(cudaMemcpyAsync(h_col.data(), fro_col.p, sizeof(double) * cols, cudaMemcpyDeviceToHost, st));
-        CBFM_CUDA(cudaStreamSynchronize(st));
+        read_back(h_col.data(), fro_col.p, sizeof(double) * cols, st);
         double a = 0.0;
         for (int c = 0; c < cols; ++c) a += h_col[c] * h_col[c];
         return std::sqrt(a);
@@ -1113,9 +1141,9 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                 launched("k_copy2d");
                 k_rownorm<<<pjc, 256, 0, st>>>(n, W.p, rnorm.p);
                 launched("k_rownorm");
-                CBFM_CUDA(cudaMemcpyAsync(h_rn.data(), rnorm0.p, sizeof(double) * pjc, cudaMemcpyDeviceToHost, st));
-                CBFM_CUDA(cudaMemcpyAsync(h_w1.data(), rnorm.p, sizeof(double) * pjc, cudaMemcpyDeviceToHost, st));
-                CBFM_CUDA(cudaStreamSynchronize(st));
+                read_back(h_two.data(), norms.p, sizeof(double) * 2 * p, st);
+                std::copy_n(h_two.begin(), pjc, h_rn.begin());
+                std::copy_n(h_two.begin() + p, pjc, h_w1.begin());
                 for (int q = 0; q < pjc; ++q) wref = std::max(wref, h_rn[q]);
             }
             std::vector<int> sel;   // vectors that need the second pass
@@ -1174,8 +1202,8 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             // row block r of the new column meets only the Q blocks i >= r - 1.
             if (d0 > 0) {
                 std::vector<GemmDesc> proj, upd;
-                // on the tensor cores one product over all blocks (Qh holds the zeros)
-                const bool whole = oz_takes(d0, pjc, d1);
+                // on the tensor cores and for small blocks one product over all blocks (Qh holds the zeros)
+                const bool whole = oz_takes(d0, pjc, d1) || dir_takes(GemmDesc{d0, pjc, d1, 0, 0, 0, 0, 0, 0});
                 if (whole) {
                     proj.push_back(GemmDesc{d0, pjc, d1, 0, dcap, 0, p, 0, p});
                     upd.push_back(GemmDesc{d1, pjc, d0, 0, dcap, 0, p, 0, p});
@@ -1203,11 +1231,9 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                     if (pass == 0) {
                         k_colnorm<<<pjc, 256, 0, st>>>((int)d2, pjc, Hn.p, p, rnorm.p);
                         launched("k_colnorm");
-                        CBFM_CUDA(cudaMemcpyAsync(h_h0.data(), rnorm0.p, sizeof(double) * pjc, cudaMemcpyDeviceToHost,
-                                                  st));
-                        CBFM_CUDA(cudaMemcpyAsync(h_h1.data(), rnorm.p, sizeof(double) * pjc, cudaMemcpyDeviceToHost,
-                                                  st));
-                        CBFM_CUDA(cudaStreamSynchronize(st));
+                        read_back(h_two.data(), norms.p, sizeof(double) * 2 * p, st);
+                        std::copy_n(h_two.begin(), pjc, h_h0.begin());
+                        std::copy_n(h_two.begin() + p, pjc, h_h1.begin());
                         if (min_ratio(h_h1, h_h0, pjc) >= GS_KEEP) break;
                     }
                 }
@@ -1227,8 +1253,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                                  -1.0);
             k_colnorm<<<p, 256, 0, st>>>((int)d2, p, Rv.p, p, rnorm.p);
             launched("k_colnorm");
-            CBFM_CUDA(cudaMemcpyAsync(h_rn.data(), rnorm.p, sizeof(double) * p, cudaMemcpyDeviceToHost, st));
-            CBFM_CUDA(cudaStreamSynchronize(st));
+            read_back(h_rn.data(), rnorm.p, sizeof(double) * p, st);
             ++J;
             ++total_blocks;
             bool all = true;

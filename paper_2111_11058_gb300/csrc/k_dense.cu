@@ -363,6 +363,119 @@ __global__ void __launch_bounds__(256) k_gemm_sk(const __grid_constant__ SkBatch
     }
 }
 
+// ------------------------------------------------------ small FP64 products
+// One small product (too small for the tensor cores' packing, mostly a block of
+// few right-hand sides): no tiles, so no FP64 instruction is spent on padding (a
+// 32 x 32 tile of 7 right-hand sides is 3/4 padding and held the FP64 pipes for 37 us with its
+// second, summing launch; these take 4 to 15 us in one).  Lanes over k where the entries are few or op(B)
+// is not contiguous along its columns (one warp per entry); else lanes over entries,
+// columns fastest, the block's warps sharing k where it is long.
+struct DirArgs {
+    const z64 *A, *B;
+    z64 *C;
+    int64_t as, ak, bk, bs, ldc;   // strides: A along rows and k, B along k and columns
+    int M, N, K;
+    int ca, cb, accumulate;        // conjugate A, B
+    double alpha;
+};
+__device__ __forceinline__ void dir_mac(z64 &acc, z64 a, z64 b) {
+    acc.re = fma(a.re, b.re, acc.re);
+    acc.im = fma(a.re, b.im, acc.im);
+    acc.re = fma(-a.im, b.im, acc.re);
+    acc.im = fma(a.im, b.re, acc.im);
+}
+__device__ __forceinline__ void dir_write(const DirArgs &P, int i, int j, z64 v) {
+    z64 *c = P.C + (int64_t)i * P.ldc + j;
+    v = P.alpha * v;
+    if (P.accumulate) *c += v;
+    else *c = v;
+}
+// one warp per entry
+__global__ void __launch_bounds__(64) k_gemm_dir_k(const __grid_constant__ DirArgs P) {
+    const int lane = threadIdx.x & 31;
+    const int64_t o = blockIdx.x * 2LL + (threadIdx.x >> 5);
+    if (o >= (int64_t)P.M * P.N) return;
+    const int i = (int)(o / P.N), j = (int)(o % P.N);
+    const z64 *a = P.A + i * P.as, *b = P.B + j * P.bs;
+    const double sa = P.ca ? -1.0 : 1.0, sb = P.cb ? -1.0 : 1.0;
+    z64 acc[2] = {z64(0, 0), z64(0, 0)};
+    int k = lane;
+    for (; k + 96 < P.K; k += 128) {
+        z64 x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u] = a[(int64_t)(k + 32 * u) * P.ak];
+            y[u] = b[(int64_t)(k + 32 * u) * P.bk];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dir_mac(acc[u & 1], z64(x[u].re, sa * x[u].im), z64(y[u].re, sb * y[u].im));
+    }
+    for (; k < P.K; k += 32) {
+        const z64 x = a[(int64_t)k * P.ak], y = b[(int64_t)k * P.bk];
+        dir_mac(acc[0], z64(x.re, sa * x.im), z64(y.re, sb * y.im));
+    }
+    z64 s = acc[0] + acc[1];
+    for (int q = 16; q > 0; q >>= 1) {
+        s.re += __shfl_xor_sync(0xffffffffu, s.re, q);
+        s.im += __shfl_xor_sync(0xffffffffu, s.im, q);
+    }
+    if (lane == 0) dir_write(P, i, j, s);
+}
+// 256 / KW entries a block, KW warps share the sum over k of 32 entries
+template <int KW>
+__global__ void __launch_bounds__(256) k_gemm_dir_n(const __grid_constant__ DirArgs P) {
+    constexpr int NE = 256 / KW;
+    __shared__ z64 s_acc[KW > 1 ? KW : 1][NE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = (warp / KW) * 32 + lane, kw = warp % KW;
+    const int64_t o = (int64_t)blockIdx.x * NE + e;
+    const bool live = o < (int64_t)P.M * P.N;
+    const int i = live ? (int)(o / P.N) : 0, j = live ? (int)(o % P.N) : 0;
+    const z64 *a = P.A + i * P.as, *b = P.B + j * P.bs;
+    const double sa = P.ca ? -1.0 : 1.0, sb = P.cb ? -1.0 : 1.0;
+    const int per = (P.K + KW - 1) / KW, k1 = min(P.K, (kw + 1) * per);
+    z64 acc[2] = {z64(0, 0), z64(0, 0)};
+    if (live) {
+        int k = kw * per;
+        for (; k + 4 <= k1; k += 4) {
+            z64 x[4], y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x[u] = a[(int64_t)(k + u) * P.ak];
+                y[u] = b[(int64_t)(k + u) * P.bk];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) dir_mac(acc[u & 1], z64(x[u].re, sa * x[u].im), z64(y[u].re, sb * y[u].im));
+        }
+        for (; k < k1; ++k) {
+            const z64 x = a[(int64_t)k * P.ak], y = b[(int64_t)k * P.bk];
+            dir_mac(acc[0], z64(x.re, sa * x.im), z64(y.re, sb * y.im));
+        }
+    }
+    z64 s = acc[0] + acc[1];
+    if constexpr (KW > 1) {
+        s_acc[kw][e] = s;
+        __syncthreads();
+        if (kw != 0) return;
+        for (int q = 1; q < KW; ++q) s += s_acc[q][e];
+    }
+    if (live) dir_write(P, i, j, s);
+}
+void gemm_dir(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z64 *C, bool accumulate, cudaStream_t st,
+              double alpha) {
+    const bool rowA = opA == 0 || opA == 3, rowB = opB == 0 || opB == 3;
+    DirArgs P{A + d.a_off, B + d.b_off, C + d.c_off, rowA ? d.lda : 1, rowA ? 1 : d.lda, rowB ? d.ldb : 1, rowB ? 1 : d.ldb,
+              d.ldc, (int)d.M, (int)d.N, (int)d.K, opA >= 2, opB >= 2, accumulate, alpha};
+    const int64_t mn = d.M * d.N;
+    ProfScope ps_("k_gemm_dir", st);
+    // a warp per entry pays five shuffle steps (20 FP64 adds) an entry: for few entries over a long sum, or
+    // where neighbouring columns of op(B) are not neighbours in memory
+    if (d.K >= 32 && (mn <= 2048 || !rowB)) k_gemm_dir_k<<<(unsigned)((mn + 1) / 2), 64, 0, st>>>(P);
+    else if (d.K >= 64) k_gemm_dir_n<8><<<(unsigned)((mn + 31) / 32), 256, 0, st>>>(P);
+    else k_gemm_dir_n<1><<<(unsigned)((mn + 255) / 256), 256, 0, st>>>(P);
+    launched("k_gemm_dir");
+}
+
 // ------------------------------------------------------ batched LU solve
 // Gaussian elimination with partial pivoting on [Z | V], then backward
 // substitution; one block per system.
@@ -1413,6 +1526,10 @@ bool gj_blocked(int64_t n, int nbatch, const z64 *Aorig, z64 *inv, cudaStream_t 
 
 }  // namespace
 
+// The product's shape as these kernels take it; false where they do not (large, or sums that keep the FP64 tiles' order).
+bool dir_takes(const GemmDesc &d) {
+    return !g_oz_hold && d.M > 0 && d.N > 0 && d.K > 0 && 1.0 * d.M * d.N * d.K <= 2.0e6 && d.M * d.N < (1 << 24);
+}
 template <typename T>
 void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> *A, const cx<T> *B, cx<T> *C,
                   bool accumulate, cudaStream_t st, double alpha) {
@@ -1431,6 +1548,12 @@ void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> 
             if (g.size() == 1 && (alpha == 1.0 || alpha == -1.0) && oz_takes(g[0].M, g[0].N, g[0].K)) {
                 ProfScope site_(g_gemm_site ? g_gemm_site : "site:other", st);
                 gemm_oz(g[0], opA, opB, A, B, C, accumulate, st, alpha < 0.0);
+                return;
+            }
+            if (g.size() == 1 && dir_takes(g[0])) {
+                prof_add_work("k_gemm_dir", fl, by);
+                ProfScope site_(g_gemm_site ? g_gemm_site : "site:other", st);
+                gemm_dir(g[0], opA, opB, A, B, C, accumulate, st, alpha);
                 return;
             }
         }

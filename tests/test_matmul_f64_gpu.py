@@ -104,3 +104,20 @@ def test_special_values(P):
     e = _err(C, _longdot(A, B))
     assert e[ok].max() <= 1e-12
     assert e[11, 2] <= 1e-300 * 1e-15 * 1e-10 + 2.0 ** -1074   # a result below the smallest normal number
+
+
+# the small kernels: entries few and many, k short and long, every storage order the solver uses (FP64 sums: the
+# usual bound K u |a| |b| with u = 2^-53, four real products)
+@pytest.mark.parametrize("M,N,K,opA,opB", [
+    (7, 7, 686, 3, 1), (7, 300, 686, 0, 2), (7, 686, 300, 0, 0), (300, 7, 330, 2, 0), (300, 7, 290, 0, 0),
+    (7, 7, 300, 2, 0), (300, 7, 7, 0, 0), (1, 1, 1, 0, 0), (45, 45, 31, 0, 1), (45, 47, 64, 1, 3), (2, 1025, 97, 0, 0),
+    (129, 17, 63, 1, 0),
+])
+def test_small_products(P, M, N, K, opA, opB):
+    rng = np.random.default_rng(M + 31 * N + 1009 * K)
+    A, B, sA, sB = _mats(rng, M, N, K, opA, opB, False)
+    C0 = rng.standard_normal((M, N)) + 1j * rng.standard_normal((M, N))
+    ref = _longdot(A, B)
+    C = P.matmul_f64(sA, sB, opA, opB, C=C0)
+    mag = np.abs(A) @ np.abs(B) + np.abs(C0)
+    assert (_err(C, (ref[0] + C0.real, ref[1] + C0.imag)) <= (2 * K + 8) * 2.0 ** -53 * mag).all()
