@@ -232,6 +232,38 @@ __global__ void k_gram_times_c(int64_t ne, int64_t nh, const int32_t *__restrict
     }
 }
 
+// |(C^J_l)^H Gf C^M_l| of every CBF l over the RWG functions of its own cell: the modulus of the diagonal of G^CBF.
+// One warp per CBF.
+__global__ void k_cbf_diag(int nc, int64_t nh, const int32_t *__restrict__ cell_off, const int64_t *__restrict__ coff,
+                           const int64_t *__restrict__ boff, const int32_t *__restrict__ Lc,
+                           const double *__restrict__ val, const int32_t *__restrict__ col,
+                           const z64 *__restrict__ CM, const z64 *__restrict__ CJ, double *__restrict__ out) {
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (q >= nh) return;
+    int lo = 0, hi = nc - 1;
+    while (lo < hi) {   // last cell with coff <= q
+        const int mid = (lo + hi + 1) / 2;
+        if (coff[mid] <= q) lo = mid;
+        else hi = mid - 1;
+    }
+    const int64_t off = cell_off[lo], end = cell_off[lo + 1], L = Lc[lo], l = q - coff[lo];
+    const z64 *cm = CM + boff[lo] + l, *cj = CJ + boff[lo] + l;
+    z64 acc(0, 0);
+    for (int64_t i = off + (threadIdx.x & 31); i < end; i += 32) {
+        z64 g(0, 0);
+        for (int sl = 0; sl < 6; ++sl) {
+            const int64_t cc = col[6 * i + sl];
+            if (cc >= off && cc < end) g += val[6 * i + sl] * cm[(cc - off) * L];
+        }
+        cfmaconj(acc, cj[(i - off) * L], g);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
+        acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+    }
+    if ((threadIdx.x & 31) == 0) out[q] = sqrt(norm2(acc));
+}
+
 // complex transpose: dst (cols x rows) = src (rows x cols)^T
 __global__ void k_transpose(int64_t rows, int64_t cols, const z64 *__restrict__ src, z64 *__restrict__ dst) {
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < rows * cols;
@@ -340,6 +372,30 @@ void cbf_make32(Cbf &c, cudaStream_t st) {
     launch_z64_to_c32(c.CJ.p, c.CJ32.p, tot, st);
 }
 
+// c.spread: largest over smallest modulus on the diagonal of G^CBF (waits for the stream)
+void cbf_spread(Cbf &c, cudaStream_t st) {
+    const Mesh &m = *c.mesh;
+    const int nc = m.h.ncell;
+    DevBuf<int32_t> dcell, dL;
+    DevBuf<int64_t> dcoff, dboff;
+    DevBuf<double> g;
+    upload(dcell, m.h.cell_off, st);
+    upload(dL, c.L, st);
+    upload(dcoff, c.coff, st);
+    upload(dboff, c.boff, st);
+    g.alloc(c.nhalf);
+    k_cbf_diag<<<nblk(c.nhalf * 32), 256, 0, st>>>(nc, c.nhalf, dcell.p, dcoff.p, dboff.p, dL.p, m.gram_val.p,
+                                                   m.gram_col.p, c.CM.p, c.CJ.p, g.p);
+    launched("k_cbf_diag");
+    std::vector<double> h(c.nhalf);
+    CBFM_CUDA(cudaMemcpyAsync(h.data(), g.p, sizeof(double) * c.nhalf, cudaMemcpyDeviceToHost, st));
+    CBFM_CUDA(cudaStreamSynchronize(st));
+    const auto mm = std::minmax_element(h.begin(), h.end());
+    c.spread = *mm.first > 0.0 ? *mm.second / *mm.first : INFINITY;
+    for (double v : h)
+        if (!(v <= *mm.second)) c.spread = INFINITY;   // a NaN among them
+}
+
 // Steps after the coefficient sets (paper Eqs. (gram_CBF), (gram_CBF_SVD), (CBF)): G'_m = (J^M)^H G_m J^J,
 // SVD, truncation sigma_i / sigma_1 >= delta_svd (at most lmax when > 0), C^M = J^M U_L, C^J = J^J V_L.
 // Vm holds, per cell, [J^M; J^J] (2 N_m x s, row-major) at voff[c].
@@ -386,6 +442,7 @@ std::unique_ptr<Cbf> dual_cbfs(Mesh *m, int s, const z64 *Vm, const std::vector<
         // G' = (J^M)^H T1
         g2.push_back(GemmDesc{s, s, N, voff[c], s, t1off[c], s, soff[c], s});
     }
+    OzHold hold_(true);   // the CBFs keep one order of sums, whatever the number of cells
     gemm_grouped<double>(g1, 0, 0, Gm.p, Vm, T1.p, false, st);
     gemm_grouped<double>(g2, 2, 0, Vm, T1.p, Gp.p, false, st);
     X.alloc((size_t)nc * s * s);
@@ -461,6 +518,7 @@ std::unique_ptr<Cbf> dual_cbfs(Mesh *m, int s, const z64 *Vm, const std::vector<
     gemm_grouped<double>(gm, 0, 0, Vm, UL.p, cb->CM.p, false, st);
     gemm_grouped<double>(gj, 0, 0, Vm, VL.p, cb->CJ.p, false, st);
     cbf_make32(*cb, st);
+    cbf_spread(*cb, st);
     return cb;
 }
 
@@ -803,7 +861,7 @@ cbfm_status cbfm_cbf_import(cbfm_mesh_t mesh, const int32_t *L_per_cell, const d
         copy_in(cb->CM.p, CM, tot * sizeof(z64), st);
         copy_in(cb->CJ.p, CJ, tot * sizeof(z64), st);
         cbf_make32(*cb, st);
-        CBFM_CUDA(cudaStreamSynchronize(st));
+        cbf_spread(*cb, st);
         *out = (cbfm_cbf_t)cb.release();
     });
 }
@@ -844,7 +902,7 @@ void project(Red &r, cudaStream_t st) {
     }
     DevBuf<cx<T>> Z;
     Z.alloc(3 * (size_t)ne * ne);
-    assemble_rwg<T>(m, Z.p, st);
+    assemble_rwg<T>(m, Z.p, st, sizeof(T) == 8 || c.spread <= SPREAD_MAX);
     if constexpr (sizeof(T) == 4) {
         if (r.prec == CBFM_MIXED || r.prec == CBFM_MIXED_UNFUSED || r.prec == CBFM_MIXED_FUSED) {
             project_tc(m, c, Z.p, A.p, st);
@@ -911,7 +969,10 @@ void gram_cbf(Red &r, cudaStream_t st) {
         // first half: (C^J)^H Gf C^M
         gJ.push_back(GemmDesc{L, nh, N, c.boff[k], L, off * nh, nh, c.coff[k] * n, n});
     }
-    gemm_grouped<double>(gJ, 2, 0, c.CJ.p, XM.p, r.G.p, false, st);
+    {
+        OzHold hold_(true);   // as many products as cells: one order of sums also for a single one
+        gemm_grouped<double>(gJ, 2, 0, c.CJ.p, XM.p, r.G.p, false, st);
+    }
     // second half (C^M)^H Gf C^J = -((C^J)^H Gf C^M)^H: the RWG Gram Gf = <f_a, n x f_b> is
     // real and antisymmetric (a . (n x b) = -b . (n x a), entry by entry in k_gram_rows)
     {
@@ -1105,13 +1166,13 @@ cbfm_status cbfm_assemble_mom(cbfm_mesh_t mesh, cbfm_precision prec, void *strea
         if (prec == CBFM_FP64) {
             DevBuf<z64> Z;
             Z.alloc(3 * (size_t)ne * ne);
-            assemble_rwg<double>(*m, Z.p, st);
+            assemble_rwg<double>(*m, Z.p, st, false);
             r->A64.alloc((size_t)r->n * r->n);
             mom_place<double>(ne, Z.p, r->A64.p, st);
         } else {
             DevBuf<c32> Z;
             Z.alloc(3 * (size_t)ne * ne);
-            assemble_rwg<float>(*m, Z.p, st);
+            assemble_rwg<float>(*m, Z.p, st, false);
             r->A32.alloc((size_t)r->n * r->n);
             mom_place<float>(ne, Z.p, r->A32.p, st);
         }
@@ -1217,7 +1278,17 @@ cbfm_status cbfm_assemble_reduced_batch(const cbfm_mesh_t *meshes, const cbfm_cb
                 Zc.push_back(Z[i - i0].p);
                 Ap.push_back(r->A32.p);
             }
-            assemble_rwg_batch<float>(wm, Zp, st);
+            // one launch per stage for the scatterers of either form of the near pairs' closed forms
+            for (int lean = 0; lean < 2; ++lean) {
+                std::vector<Mesh *> lm;
+                std::vector<c32 *> lz;
+                for (size_t k = 0; k < wm.size(); ++k)
+                    if ((wc[k]->spread <= SPREAD_MAX) == (lean == 1)) {
+                        lm.push_back(wm[k]);
+                        lz.push_back(Zp[k]);
+                    }
+                if (!lm.empty()) assemble_rwg_batch<float>(lm, lz, st, lean == 1);
+            }
             project_tc_batch(wm, wc, Zc, Ap, st);
             CBFM_CUDA(cudaStreamSynchronize(st));
             i0 = i1;
@@ -1307,20 +1378,9 @@ cbfm_status cbfm_cmp_setup(cbfm_red_t red, void *stream) {
             launched("k_place_neg_adjoint");
         }
         int hinfo = 0;
-        std::vector<std::complex<double>> hdiag(nh);   // the diagonal of the first half (the second is minus its conjugate)
         CBFM_CUDA(cudaMemcpyAsync(&hinfo, info.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CBFM_CUDA(cudaMemcpy2DAsync(hdiag.data(), sizeof(z64), r->G.p, sizeof(z64) * (n + 1), sizeof(z64), nh,
-                                    cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaStreamSynchronize(st));
         if (hinfo) throw Fail{CBFM_ESINGULAR, "G^CBF is singular"};
-        {
-            double lo = INFINITY, hi = 0.0;
-            for (const std::complex<double> &g : hdiag) {
-                lo = std::min(lo, std::abs(g));
-                hi = std::max(hi, std::abs(g));
-            }
-            r->gram_spread = lo > 0.0 ? hi / lo : INFINITY;
-        }
         // B = A (G^CBF)^{-1}: GMRES then needs one product per iteration
         std::vector<GemmDesc> gb{GemmDesc{n, n, n, 0, n, 0, n, 0, n}};
         if (r->prec != CBFM_FP64) {

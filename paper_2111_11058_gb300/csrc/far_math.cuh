@@ -4,6 +4,7 @@
 // The moment form and the reading of the T sign are described in k_assembly.cu.
 #pragma once
 
+#include "fp64_math.cuh"
 #include "internal.cuh"
 
 namespace cbfm {
@@ -176,7 +177,8 @@ __device__ __forceinline__ bool is_near_t(const T *rt_cen, const T *rt_lo, T ht,
 // SOA: the test record is stored field-major, element f at rt[f * rts] (a
 // structure-of-arrays copy whose consecutive triangles sit in consecutive
 // lanes); otherwise at rt[f].
-template <typename T, bool SOA = false>
+// LEAN: the FP64 form takes its sines, cosines and reciprocal square roots from fp64_math.cuh.
+template <typename T, bool SOA = false, bool LEAN = false>
 __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *rs, const MediaT<T> &md, cx<T> *out) {
     auto R = [&](int f) -> T { return SOA ? rt[(int64_t)f * rts] : rt[f]; };
     auto sq = [&](int i) -> T { return R(TR_Q + i); };
@@ -223,7 +225,9 @@ __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *r
         for (int q = 0; q < 7; ++q) {
             const T d0 = Dp[0] - rq[q][0], d1 = Dp[1] - rq[q][1], d2 = Dp[2] - rq[q][2];
             const T R2 = d0 * d0 + d1 * d1 + d2 * d2;
-            const T iR = rsqrt_t(R2);
+            T iR;
+            if constexpr (LEAN && sizeof(T) == 8) iR = f64::rsqrt64(R2);
+            else iR = rsqrt_t(R2);
             const T R = R2 * iR;
             const T niR2 = -(iR * iR);
             const T amp = iR * wq[q];
@@ -231,7 +235,8 @@ __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *r
             for (int i = 0; i < 2; ++i) {
                 const T kR = kr[i] * R;
                 T sn, cs_;
-                sincos_red(kR, &sn, &cs_);
+                if constexpr (LEAN && sizeof(T) == 8) f64::sincos64(kR, &sn, &cs_);
+                else sincos_red(kR, &sn, &cs_);
                 T a_i = amp;
                 if (i == 1 && lossy2) a_i *= exp_t(ki[i] * R);
                 // w G = amp (cos - j sin);  w g = -(1 + j k R) w G / R^2, j k R = -ki R + j kr R

@@ -63,9 +63,19 @@ struct Cbf : HandleBase {
     std::vector<int64_t> coff;    // CBF offsets per cell (ncell+1), within one half
     std::vector<int64_t> boff;    // block offsets sum N_m L_m (ncell+1)
     int64_t nhalf = 0;            // sum L_m
+    double spread = 0.0;          // largest over smallest modulus on the diagonal of G^CBF (the CBFs' singular values)
     DevBuf<z64> CM, CJ;           // blocks N_m x L_m row-major, cells in order
     DevBuf<c32> CM32, CJ32;
 };
+
+// Spread of the CBFs' singular values up to which a mixed-precision system takes
+// the faster forms that change the last bits of its matrix or of its basis.  With
+// tiny triangles beside large ones (1.4e4 to 1e5 on spheroids and cylinders with pole
+// triangles; 1e3 to 5e3 on cubes, spheres and even cylinders) the FP32 operator's rounding, which follows those
+// bits, moves the currents by 1e-5 of their norm and 1e-3 of their rms at single
+// edges (1.5e-6 and 6e-5 where the spread is below 5e3): those systems keep one order of operations, so that
+// their results stay reproducible.
+constexpr double SPREAD_MAX = 1e4;
 
 struct Red : HandleBase {
     Mesh *mesh;
@@ -80,7 +90,6 @@ struct Red : HandleBase {
     DevBuf<z64> B64;              // B = A (G^CBF)^{-1}, the operator GMRES iterates with
     DevBuf<c32> B32;
     bool cmp_ready = false;
-    double gram_spread = 0.0;     // largest over smallest modulus on the diagonal of G^CBF (cbfm_cmp_setup)
     // T-diagonal arrangement (Eq. (MoM_T)): Bt = A P D^{-1} (P swaps the column halves),
     // tdinv[k] = 1 / D_{p(k)}: the recovery x_k = y_{p(k)} tdinv[k]
     DevBuf<z64> Bt64;
@@ -109,7 +118,7 @@ void launch_farfield(const Mesh &m, const z64 *j, int nrhs, const double *d_obs,
 // assembly (k_assembly.cu): local blocks of all triangle pairs, then the RWG
 // matrices Z_op (op = Ks, Ta, Tb), row-major ne x ne, internal edge order.
 template <typename T>
-void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool diag_cells = false);
+void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool lean, bool diag_cells = false);
 
 // dense complex linear algebra (k_dense.cu)
 struct GemmDesc {
@@ -182,10 +191,10 @@ void jacobi_svd_batched(int nb, int s, z64 *X, z64 *V, double *sig, int *d_info,
 // diag_cells: only triangle pairs that support RWGs of a common cell are
 // evaluated (the cells' diagonal blocks of Z); every other entry is zero
 template <typename T>
-void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st,
+void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
                         bool diag_cells = false);
 // near-pair blocks only, compact (27 complex64 per pair of each mesh's near list) (k_assembly.cu)
-void near_blocks_compact(const std::vector<Mesh *> &ms, const std::vector<c32 *> &out, cudaStream_t st);
+void near_blocks_compact(const std::vector<Mesh *> &ms, const std::vector<c32 *> &out, cudaStream_t st, bool lean);
 // Fused mixed-precision assembly and projection (k_fused.cu): A[k] = (C^JM)^H Z C^MJ
 // for each mesh, with no RWG or local-block matrix in device memory.  fused_fits
 // tells whether the scatterer's cells fit the kernel's tile limits.
@@ -278,7 +287,7 @@ FusedTables &fused_tables(Mesh &m, cudaStream_t st);
 // near-pair blocks only, compact (27 complex per pair of each mesh's near list),
 // FP64 closed forms with FP32 (T = float) or FP64 (T = double) smooth remainders (k_assembly.cu)
 template <typename T>
-void near_blocks_compact_t(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &out, cudaStream_t st);
+void near_blocks_compact_t(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &out, cudaStream_t st, bool lean);
 // Z_mm of every cell in FP64, the 2 N_m x 2 N_m matrix [[Ks, Ta], [Tb, Ks]] of its RWG functions
 // (row-major, at Zmm + zoff[c]), from the triangle pairs of the cell alone (k_celldiag.cu)
 void assemble_cell_diag(Mesh &m, z64 *Zmm, const std::vector<int64_t> &zoff, cudaStream_t st);

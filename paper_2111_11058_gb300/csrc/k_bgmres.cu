@@ -628,10 +628,6 @@ constexpr double ORTH_TOL = 1e-12;
 // under ORTH_TOL); otherwise its coefficients are formed and applied when
 // they exceed ORTH_TOL of the block.
 constexpr double GS_KEEP = 0.1;
-// Spread of the diagonal of G^CBF (the CBFs' singular values) up to which a mixed-precision solve forms its basis
-// on the tensor cores; measured 1e3 to 5e3 on cubes, spheres and cylinders with even triangles, 1.4e4 to 1e5 on
-// spheroids and cylinders with pole triangles.
-constexpr double SPREAD_MAX = 1e4;
 
 // ||M - I||_F of the m x m Gram matrix in ctx.M (host sync).
 double gram_dev(Ctx &c, int m) {
@@ -1002,13 +998,10 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     CBFM_CUDA(cudaMemcpyAsync(h_bn.data(), bnorm.p, sizeof(double) * p, cudaMemcpyDeviceToHost, st));
     CBFM_CUDA(cudaStreamSynchronize(st));
 
-    // Where the operator's product is FP32, its rounding errors depend on the last bits of the basis, and the
-    // reduced system amplifies them: with the CBFs' singular values spread over SPREAD_MAX and more (tiny triangles
-    // beside large ones) the currents move by 1e-5 of their norm and 1e-3 of their rms at single edges when the
-    // sums of the basis are only reordered (1.5e-6 and 6e-5 where the spread is below 5e3).  Those systems keep the FP64 units' sums for the basis
-    // and the FP32 solution update, so that their results stay reproducible, and so do the slowly converging
-    // systems without the CMP; everything else goes to the tensor cores.
-    const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.gram_spread <= SPREAD_MAX);
+    // The basis (Gram-Schmidt and its Cholesky QR) on the tensor cores, except where the FP32 operator would carry a change
+    // of its last bits into the currents (SPREAD_MAX), and in the slowly converging systems without the CMP: there the
+    // FP64 units' order of sums and the FP32 solution update stay.
+    const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.cbf->spread <= SPREAD_MAX);
     OzMat op;   // FP64 operator cut into digits once per solve
     auto applyB = [&](const z64 *in, z64 *out, int rows) {
         if (pc == CBFM_PC_CMP_INEXACT) {

@@ -110,7 +110,7 @@ void assemble_cell_diag(Mesh &m, z64 *Zmm, const std::vector<int64_t> &zoff, cud
     // FP64 near-pair blocks, compact
     DevBuf<z64> nearv;
     nearv.alloc((size_t)std::max<int64_t>(1, m.n_near) * NCOMP);
-    near_blocks_compact_t<double>({&m}, {nearv.p}, st);
+    near_blocks_compact_t<double>({&m}, {nearv.p}, st, false);   // the CBFs keep the general functions
     std::vector<int64_t> poff(nc + 1, 0);
     for (int c = 0; c < nc; ++c) {
         const int64_t nT = ft.tl_off[c + 1] - ft.tl_off[c];
