@@ -900,16 +900,20 @@ void project(Red &r, cudaStream_t st) {
             return;
         }
     }
-    DevBuf<cx<T>> Z;
-    Z.alloc(3 * (size_t)ne * ne);
-    assemble_rwg<T>(m, Z.p, st, sizeof(T) == 8 || c.spread <= SPREAD_MAX);
+    const bool lean = sizeof(T) == 8 || c.spread <= SPREAD_MAX;
     if constexpr (sizeof(T) == 4) {
         if (r.prec == CBFM_MIXED || r.prec == CBFM_MIXED_UNFUSED || r.prec == CBFM_MIXED_FUSED) {
-            project_tc(m, c, Z.p, A.p, st);
+            DevBuf<float> Zs;
+            Zs.alloc(tc_planes(ne));
+            assemble_rwg_split({&m}, {Zs.p}, st, lean);
+            project_tc(m, c, Zs, A.p, st);
             A.give(r.A32);
             return;
         }
     }
+    DevBuf<cx<T>> Z;
+    Z.alloc(3 * (size_t)ne * ne);
+    assemble_rwg<T>(m, Z.p, st, lean);
     const cx<T> *CM, *CJ;
     if constexpr (sizeof(T) == 8) { CM = c.CM.p; CJ = c.CJ.p; }
     else { CM = c.CM32.p; CJ = c.CJ32.p; }
@@ -1254,7 +1258,7 @@ cbfm_status cbfm_assemble_reduced_batch(const cbfm_mesh_t *meshes, const cbfm_cb
         auto transient = [&](int k) {
             const double nt = (double)ms[k]->h.nt, ne = (double)ms[k]->h.ne, nh = (double)cs[k]->nhalf;
             const double ldz = std::ceil(2.0 * ne / 32.0) * 32.0;
-            return 27.0 * nt * nt * 8 + 3.0 * ne * ne * 8 + 6.0 * ne * ldz * 4 + 8.0 * 2 * nh * ldz * 4 +
+            return 27.0 * nt * nt * 8 + 6.0 * ne * ldz * 4 + 8.0 * 2 * nh * ldz * 4 +
                    4.0 * nh * nh * 8;
         };
         size_t i0 = 0;
@@ -1264,32 +1268,28 @@ cbfm_status cbfm_assemble_reduced_batch(const cbfm_mesh_t *meshes, const cbfm_cb
             while (i1 < rest.size() && (i1 == i0 || used + transient(rest[i1]) <= budget)) used += transient(rest[i1++]);
             std::vector<Mesh *> wm;
             std::vector<Cbf *> wc;
-            std::vector<DevBuf<c32>> Z(i1 - i0);
-            std::vector<c32 *> Zp, Ap;
-            std::vector<const c32 *> Zc;
+            std::vector<DevBuf<float>> Zs(i1 - i0);
+            std::vector<c32 *> Ap;
             for (size_t i = i0; i < i1; ++i) {
                 const int32_t k = rest[i];
                 Red *r = make(k);
                 wm.push_back(ms[k]);
                 wc.push_back(cs[k]);
-                const int64_t ne = ms[k]->h.ne;
-                Z[i - i0].alloc((size_t)3 * ne * ne);
-                Zp.push_back(Z[i - i0].p);
-                Zc.push_back(Z[i - i0].p);
+                Zs[i - i0].alloc(tc_planes(ms[k]->h.ne));
                 Ap.push_back(r->A32.p);
             }
             // one launch per stage for the scatterers of either form of the near pairs' closed forms
             for (int lean = 0; lean < 2; ++lean) {
                 std::vector<Mesh *> lm;
-                std::vector<c32 *> lz;
+                std::vector<float *> lz;
                 for (size_t k = 0; k < wm.size(); ++k)
                     if ((wc[k]->spread <= SPREAD_MAX) == (lean == 1)) {
                         lm.push_back(wm[k]);
-                        lz.push_back(Zp[k]);
+                        lz.push_back(Zs[k].p);
                     }
-                if (!lm.empty()) assemble_rwg_batch<float>(lm, lz, st, lean == 1);
+                if (!lm.empty()) assemble_rwg_split(lm, lz, st, lean == 1);
             }
-            project_tc_batch(wm, wc, Zc, Ap, st);
+            project_tc_batch(wm, wc, Zs, Ap, st);
             CBFM_CUDA(cudaStreamSynchronize(st));
             i0 = i1;
         }

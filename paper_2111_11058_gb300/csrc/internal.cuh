@@ -193,6 +193,10 @@ void jacobi_svd_batched(int nb, int s, z64 *X, z64 *V, double *sig, int *d_info,
 template <typename T>
 void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
                         bool diag_cells = false);
+// the RWG operators of several meshes as split-TF32 planes Zs[plane][op][i][f], row pitch tc_ldz(ne) floats (k_assembly.cu)
+void assemble_rwg_split(const std::vector<Mesh *> &ms, const std::vector<float *> &Zs, cudaStream_t st, bool lean);
+inline int64_t tc_ldz(int64_t ne) { return (2 * ne + 31) / 32 * 32; }
+inline size_t tc_planes(int64_t ne) { return (size_t)2 * 3 * ne * tc_ldz(ne); }
 // near-pair blocks only, compact (27 complex64 per pair of each mesh's near list) (k_assembly.cu)
 void near_blocks_compact(const std::vector<Mesh *> &ms, const std::vector<c32 *> &out, cudaStream_t st, bool lean);
 // Fused mixed-precision assembly and projection (k_fused.cu): A[k] = (C^JM)^H Z C^MJ
@@ -208,9 +212,10 @@ void assemble_project_fused(const std::vector<Mesh *> &ms, const std::vector<Cbf
 // tuned launch parameters, per key (api.cu); 0 when not tuned yet
 int tuning_get(const std::string &key);
 void tuning_set(const std::string &key, int value);
-// tensor-core projection of Z (3 x ne x ne, c32) onto the CBFs into A (k_tc.cu)
-void project_tc(Mesh &m, Cbf &c, const c32 *Z, c32 *A, cudaStream_t st);
-void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &cs, const std::vector<const c32 *> &Z,
+// tensor-core projection of the operators in Zs (assemble_rwg_split) onto the CBFs into A (k_tc.cu); Zs is released
+// as soon as it has been read
+void project_tc(Mesh &m, Cbf &c, DevBuf<float> &Zs, c32 *A, cudaStream_t st);
+void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &cs, std::vector<DevBuf<float>> &Zs,
                       const std::vector<c32 *> &A, cudaStream_t st);
 void gauss_jordan_inverse(int64_t n, int nbatch, z64 *Aug, z64 *inv, int *d_info, cudaStream_t st);
 

@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "far_math.cuh"
+#include "tc_ptx.cuh"
 
 namespace cbfm {
 
@@ -531,6 +532,8 @@ struct AsmJob {
     const int32_t *vid, *pairs, *edge_tri, *edge_loc;
     const int32_t *tri_cell;   // non-null: evaluate only pairs of triangles that share a cell
     cx<T> *Zloc, *Z;
+    float *Zs;                 // non-null (FP32): the RWG rows as hi/lo planes instead of Z, row pitch ldz floats
+    int64_t ldz;
     cx<T> *nearblk;            // non-null: near-pair blocks in compact form, 27 per pair of the near list
     MediaT<T> mdt;
     Media md;
@@ -779,7 +782,12 @@ __global__ void __launch_bounds__(256) k_mirror(const AsmJob<T> *__restrict__ jo
     }
 }
 
-// Gather of all meshes: one block per RWG row, grid-stride over the rows of all meshes.
+// Gather of all meshes: one block per RWG row, grid-stride over the rows of all
+// meshes.  With J.Zs the row leaves as the split-TF32 planes the tensor-core
+// projection reads, Zs[plane][op][i][f] (interleaved floats, zero up to the pitch ldz),
+// so that Z itself is neither written nor read again.  Bound: HBM, the 27 planes
+// of local blocks read once and the planes written once (9216-unknown cube: 0.50 ms
+// of gather and 0.34 ms of splitting -> GATHER_MS ms in one pass).
 template <typename T>
 __global__ void k_gather(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t nrows) {
     for (int64_t row = blockIdx.x; row < nrows; row += gridDim.x) {
@@ -787,14 +795,32 @@ __global__ void k_gather(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t 
         const int64_t i = row - J.row0, ne = J.ne;
         const int64_t plane = (int64_t)J.nt * J.nt;
         const int ti[2] = {J.edge_tri[2 * i], J.edge_tri[2 * i + 1]}, ai[2] = {J.edge_loc[2 * i], J.edge_loc[2 * i + 1]};
-        for (int64_t j = threadIdx.x; j < ne; j += blockDim.x) {
-            const int tj[2] = {J.edge_tri[2 * j], J.edge_tri[2 * j + 1]};
-            const int aj[2] = {J.edge_loc[2 * j], J.edge_loc[2 * j + 1]};
+        const int64_t cols = J.Zs ? J.ldz / 2 : ne;
+        for (int64_t j = threadIdx.x; j < cols; j += blockDim.x) {
+            int tj[2] = {0, 0}, aj[2] = {0, 0};
+            if (j < ne) {
+                tj[0] = J.edge_tri[2 * j];
+                tj[1] = J.edge_tri[2 * j + 1];
+                aj[0] = J.edge_loc[2 * j];
+                aj[1] = J.edge_loc[2 * j + 1];
+            }
             for (int op = 0; op < 3; ++op) {
                 cx<T> v(0, 0);
-                for (int a = 0; a < 2; ++a)
-                    for (int b = 0; b < 2; ++b)
-                        v += J.Zloc[(op * 9 + 3 * ai[a] + aj[b]) * plane + (int64_t)ti[a] * J.nt + tj[b]];
+                if (j < ne)
+                    for (int a = 0; a < 2; ++a)
+                        for (int b = 0; b < 2; ++b)
+                            v += J.Zloc[(op * 9 + 3 * ai[a] + aj[b]) * plane + (int64_t)ti[a] * J.nt + tj[b]];
+                if constexpr (sizeof(T) == 4) {
+                    if (J.Zs) {
+                        float2 hi, lo;
+                        tc::split(v.re, hi.x, lo.x);
+                        tc::split(v.im, hi.y, lo.y);
+                        float *d = J.Zs + (op * ne + i) * J.ldz + 2 * j;
+                        *reinterpret_cast<float2 *>(d) = hi;
+                        *reinterpret_cast<float2 *>(d + 3 * ne * J.ldz) = lo;
+                        continue;
+                    }
+                }
                 J.Z[(op * ne + i) * ne + j] = v;
             }
         }
@@ -804,8 +830,17 @@ __global__ void k_gather(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t 
 }  // namespace
 
 template <typename T>
+static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
+                           cudaStream_t st, bool lean, bool diag_cells);
+template <typename T>
 void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
-                        bool diag_cells);
+                        bool diag_cells) {
+    assemble_batch<T>(ms, Z, {}, st, lean, diag_cells);
+}
+// The RWG operators as the split-TF32 planes of the tensor-core projection (k_tc.cu: row pitch tc_ldz).
+void assemble_rwg_split(const std::vector<Mesh *> &ms, const std::vector<float *> &Zs, cudaStream_t st, bool lean) {
+    assemble_batch<float>(ms, {}, Zs, st, lean, false);
+}
 
 // One mesh: the batched stages with a batch of one (one code path, so a
 // mesh assembled alone and in a batch gets the same bits).
@@ -826,8 +861,8 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
 // long restarted solves carry a last bit of Z into the currents, and mixed
 // systems beyond SPREAD_MAX keep the general ones.
 template <typename T>
-void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
-                        bool diag_cells) {
+static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
+                           cudaStream_t st, bool lean, bool diag_cells) {
     const int nj = (int)ms.size();
     if (nj == 0) return;
     std::vector<DevBuf<cx<T>>> Zloc(nj);
@@ -849,7 +884,9 @@ void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *
         J.edge_loc = m.edge_loc.p;
         J.tri_cell = diag_cells ? m.tri_cell.p : nullptr;
         J.Zloc = Zloc[k].p;
-        J.Z = Z[k];
+        J.Z = Z.empty() ? nullptr : Z[k];
+        J.Zs = Zs.empty() ? nullptr : Zs[k];
+        J.ldz = tc_ldz(m.h.ne);
         J.mdt = media_t<T>(md);
         J.md = md;
         J.alpha = m.alpha;
@@ -864,7 +901,7 @@ void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *
         ntiles += tb * (tb + 1) / 2;
         mir_bytes += 2.0 * NCOMP * (0.5 * nt * (nt - 1.0)) * sizeof(cx<T>);   // pairs s < t read and written
         // the gather reads every local block once and writes the three RWG planes
-        gat_bytes += ((double)NCOMP * nt * nt + 3.0 * (double)m.h.ne * m.h.ne) * sizeof(cx<T>);
+        gat_bytes += ((double)NCOMP * nt * nt + (Zs.empty() ? 1.0 : 2.0) * 3.0 * (double)m.h.ne * m.h.ne) * sizeof(cx<T>);
         const double upper = 0.5 * nt * (nt + 1.0);   // pairs t <= s
         far_flop += (upper - (double)m.n_near) * 49.0 * FAR_FLOP_PER_POINT_PAIR;
         far_bytes += (double)NCOMP * upper * sizeof(cx<T>);

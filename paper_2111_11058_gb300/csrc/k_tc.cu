@@ -250,25 +250,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_gemm(const __grid_constant
 }
 
 // ----------------------------------------------------------- operand builders
-// Z planes: Zs[plane][op][e][f] = hi/lo of the interleaved float f of row e
-// of Z_op (f < 2 ne), zero in the padding up to ldz.
-__global__ void k_split_z(int64_t ne, int64_t ldz, const c32 *__restrict__ Z, float *__restrict__ Zs) {
-    const int64_t rows = 3 * ne, per = ldz / 2;   // complex slots per row
-    const int64_t plane = rows * ldz;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows * per;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / per, c = i - r * per;
-        float2 hi = make_float2(0.f, 0.f), lo = hi;
-        if (c < ne) {
-            const c32 z = Z[r * ne + c];
-            split(z.re, hi.x, lo.x);
-            split(z.im, hi.y, lo.y);
-        }
-        *reinterpret_cast<float2 *>(Zs + r * ldz + 2 * c) = hi;
-        *reinterpret_cast<float2 *>(Zs + plane + r * ldz + 2 * c) = lo;
-    }
-}
-
 // GEMM1 B panels: for cell k, rows [0, P_k) expand C^M_k, rows [P_k, 2 P_k)
 // expand C^J_k ((j, re) row then (j, im) row per CBF j; zero rows up to P_k),
 // columns kk of the cell's K frame: float kk0_k + kk of a Z row.
@@ -414,7 +395,7 @@ namespace {
 // Per-scatterer operands of the projection (split planes, panels, index
 // tables), its tensor maps and launch parameters, and its work counts.
 struct TcPrep {
-    DevBuf<float> Zs, Bp, Cp, YT;
+    DevBuf<float> Bp, Cp, YT;
     DevBuf<int32_t> dLs, dPk, dprow, dkk0, dcell_off, dcell_of_cbf, dks;
     DevBuf<int64_t> dboff, dcoff;
     TcMaps maps;
@@ -424,24 +405,14 @@ struct TcPrep {
 
 // Builds the operands and appends the scatterer's GEMM1 and GEMM2 tasks
 // (tagged sidx).  Returns false when the scatterer has no CBFs.
-bool tc_prepare(Mesh &m, Cbf &c, const c32 *Z, c32 *A, int sidx, int *errp, TcPrep &pp, std::vector<TcTask> &t1,
+bool tc_prepare(Mesh &m, Cbf &c, float *Zs, c32 *A, int sidx, int *errp, TcPrep &pp, std::vector<TcTask> &t1,
                 std::vector<TcTask> &t2, cudaStream_t st) {
     const int nc = m.h.ncell;
 
     const int64_t ne = m.h.ne, nh = c.nhalf, nred = 2 * nh;
     if (nh == 0) return false;
-    const int64_t ldz = up(2 * ne, TC_KB);
+    const int64_t ldz = tc_ldz(ne);
     CBFM_REQUIRE(ne < (1ll << 30) / 2 && ldz < (1ll << 31), "mesh too large for 32-bit tile coordinates");
-
-    // --- Z hi/lo planes
-    DevBuf<float> &Zs = pp.Zs;
-    Zs.alloc((size_t)2 * 3 * ne * ldz);
-    {
-        ProfScope ps_("k_split_z", st);
-        k_split_z<<<4 * sm_count(), 256, 0, st>>>(ne, ldz, Z, Zs.p);
-        launched("k_split_z");
-        prof_add_work("k_split_z", 0.0, (double)3 * ne * ne * 8 + (double)2 * 3 * ne * ldz * 4);
-    }
 
     // --- GEMM1 B panels (per cell K frame, aligned to 32 floats)
     std::vector<int32_t> Ls(nc), Pk(nc), prow(nc), kk0(nc);
@@ -510,7 +481,7 @@ bool tc_prepare(Mesh &m, Cbf &c, const c32 *Z, c32 *A, int sidx, int *errp, TcPr
         CBFM_CUDA(cudaMemset2DAsync(YT.p + 2 * ne, ldz * 4, 0, (ldz - 2 * ne) * 4, (size_t)2 * 4 * 2 * nh, st));
 
     TcMaps &maps = pp.maps;
-    make_map(&maps.m[MAP_Z], Zs.p, ldz, ne, 3, 2, TC_M);
+    make_map(&maps.m[MAP_Z], Zs, ldz, ne, 3, 2, TC_M);
     make_map(&maps.m[MAP_BP], Bp.p, ldb, brows, 1, 2, TC_BROWS);
     make_map(&maps.m[MAP_CP], Cp.p, ldc, (int64_t)ntile * TC_M, 2, 2, TC_M);
     make_map(&maps.m[MAP_YT], YT.p, ldz, 2 * nh, 4, 2, TC_BROWS);
@@ -578,18 +549,18 @@ void check_err(const int *errp, cudaStream_t st) {
 
 }  // namespace
 
-// A (nred x nred, c32) = the four CBF projections of Z (3 x ne x ne, c32) on
-// the tensor cores.  Z is consumed (released by the caller afterwards).
-void project_tc(Mesh &m, Cbf &c, const c32 *Z, c32 *A, cudaStream_t st) {
+// A (nred x nred, c32) = the four CBF projections of the operators in Zs on the
+// tensor cores.
+void project_tc(Mesh &m, Cbf &c, DevBuf<float> &Zs, c32 *A, cudaStream_t st) {
     DevBuf<int> err;
     err.alloc(1);
     CBFM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
     TcPrep pp;
     std::vector<TcTask> t1, t2;
-    if (!tc_prepare(m, c, Z, A, 0, err.p, pp, t1, t2, st)) return;
+    if (!tc_prepare(m, c, Zs.p, A, 0, err.p, pp, t1, t2, st)) return;
     launch_tc(pp.maps, nullptr, nullptr, t1, pp.P, st, "k_tc_gemm1");
     prof_add_work("k_tc_gemm1", pp.fl1, pp.by1);
-    pp.Zs.release();
+    Zs.release();
     launch_tc(pp.maps, nullptr, nullptr, t2, pp.P, st, "k_tc_gemm2");
     prof_add_work("k_tc_gemm2", pp.fl2, pp.by2);
     check_err(err.p, st);
@@ -597,7 +568,7 @@ void project_tc(Mesh &m, Cbf &c, const c32 *Z, c32 *A, cudaStream_t st) {
 
 // The same for several scatterers: one GEMM1 launch and one GEMM2 launch over
 // the tasks of all of them (tensor maps and parameters in global memory).
-void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &cs, const std::vector<const c32 *> &Z,
+void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &cs, std::vector<DevBuf<float>> &Zs,
                       const std::vector<c32 *> &A, cudaStream_t st) {
     DevBuf<int> err;
     err.alloc(1);
@@ -609,7 +580,7 @@ void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &c
     double fl1 = 0, fl2 = 0, by1 = 0, by2 = 0;
     for (size_t k = 0; k < ms.size(); ++k) {
         std::unique_ptr<TcPrep> pp(new TcPrep());
-        if (!tc_prepare(*ms[k], *cs[k], Z[k], A[k], (int)hmaps.size(), err.p, *pp, t1, t2, st)) continue;
+        if (!tc_prepare(*ms[k], *cs[k], Zs[k].p, A[k], (int)hmaps.size(), err.p, *pp, t1, t2, st)) continue;
         hmaps.push_back(pp->maps);
         hpar.push_back(pp->P);
         fl1 += pp->fl1;
@@ -628,7 +599,7 @@ void project_tc_batch(const std::vector<Mesh *> &ms, const std::vector<Cbf *> &c
     CBFM_CUDA(cudaMemcpyAsync(dpar.p, hpar.data(), sizeof(TcParams) * hpar.size(), cudaMemcpyHostToDevice, st));
     launch_tc(hmaps[0], dmaps.p, dpar.p, t1, hpar[0], st, "k_tc_gemm1");
     prof_add_work("k_tc_gemm1", fl1, by1);
-    for (auto &pp : preps) pp->Zs.release();
+    for (auto &z : Zs) z.release();
     launch_tc(hmaps[0], dmaps.p, dpar.p, t2, hpar[0], st, "k_tc_gemm2");
     prof_add_work("k_tc_gemm2", fl2, by2);
     check_err(err.p, st);
