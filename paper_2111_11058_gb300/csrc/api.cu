@@ -652,6 +652,8 @@ cbfm_status cbfm_mesh(const double *verts, int64_t nv, const int32_t *tris, int6
         upload(m->edge_cell, ecell, st);
         m->tri64.alloc((size_t)h.nt * TRI_REC);
         m->tri32.alloc((size_t)h.nt * TRI_REC);
+        m->far64.alloc((size_t)h.nt * FB_REC);
+        m->far32.alloc((size_t)h.nt * FB_REC);
         launch_tri_records(*m, dv.p, dt.p, st);
         launch_near_pairs(*m, st);
         launch_gram_rows(*m, st);

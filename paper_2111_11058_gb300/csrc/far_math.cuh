@@ -11,6 +11,9 @@ namespace cbfm {
 namespace fm {
 
 constexpr int NCOMP = 27;   // 3 operators x 3 x 3
+// Far record of a triangle (FB_REC values, far_bary.cuh): vertices relative to the centroid, c_a times
+// the area, centroid (FP32: hi + lo parts, relative to the mesh centre), longest edge.
+constexpr int FB_P = 0, FB_C = 9, FB_CEN = 12, FB_CLO = 15, FB_H = 18;
 // Algorithmic work of one quadrature point pair, both media, counting an FMA
 // as 2: the direct evaluation of G and g (distance, R, 1/R, e^{-jkR}, the
 // (1 + jkR)/R^2 factor) and of the 14 complex moment sums of the far pair
@@ -177,8 +180,7 @@ __device__ __forceinline__ bool is_near_t(const T *rt_cen, const T *rt_lo, T ht,
 // SOA: the test record is stored field-major, element f at rt[f * rts] (a
 // structure-of-arrays copy whose consecutive triangles sit in consecutive
 // lanes); otherwise at rt[f].
-// LEAN: the FP64 form takes its sines, cosines and reciprocal square roots from fp64_math.cuh.
-template <typename T, bool SOA = false, bool LEAN = false>
+template <typename T, bool SOA = false>
 __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *rs, const MediaT<T> &md, cx<T> *out) {
     auto R = [&](int f) -> T { return SOA ? rt[(int64_t)f * rts] : rt[f]; };
     auto sq = [&](int i) -> T { return R(TR_Q + i); };
@@ -225,9 +227,7 @@ __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *r
         for (int q = 0; q < 7; ++q) {
             const T d0 = Dp[0] - rq[q][0], d1 = Dp[1] - rq[q][1], d2 = Dp[2] - rq[q][2];
             const T R2 = d0 * d0 + d1 * d1 + d2 * d2;
-            T iR;
-            if constexpr (LEAN && sizeof(T) == 8) iR = f64::rsqrt64(R2);
-            else iR = rsqrt_t(R2);
+            const T iR = rsqrt_t(R2);
             const T R = R2 * iR;
             const T niR2 = -(iR * iR);
             const T amp = iR * wq[q];
@@ -235,8 +235,7 @@ __device__ __forceinline__ void far_entries(const T *rt, int64_t rts, const T *r
             for (int i = 0; i < 2; ++i) {
                 const T kR = kr[i] * R;
                 T sn, cs_;
-                if constexpr (LEAN && sizeof(T) == 8) f64::sincos64(kR, &sn, &cs_);
-                else sincos_red(kR, &sn, &cs_);
+                sincos_red(kR, &sn, &cs_);
                 T a_i = amp;
                 if (i == 1 && lossy2) a_i *= exp_t(ki[i] * R);
                 // w G = amp (cos - j sin);  w g = -(1 + j k R) w G / R^2, j k R = -ki R + j kr R

@@ -43,6 +43,8 @@ struct Mesh : HandleBase {
     z64 k1, k2, eta1, eta2;
     DevBuf<double> tri64;        // nt * TRI_REC
     DevBuf<float> tri32;         // nt * TRI_REC (centred coordinates)
+    DevBuf<double> far64;        // nt * FB_REC (far_bary.cuh)
+    DevBuf<float> far32;
     DevBuf<int32_t> tri_vid;     // nt*3 vertex ids
     DevBuf<int32_t> tri_edge;    // nt*3 internal edge id
     DevBuf<int32_t> tri_cell;    // nt*3 cell of each of the triangle's RWGs

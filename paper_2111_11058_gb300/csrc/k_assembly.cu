@@ -33,9 +33,10 @@
 //   the 2 x 2 triangle pairs of the two supports.
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
-#include "far_math.cuh"
+#include "far_bary.cuh"
 #include "tc_ptx.cuh"
 
 namespace cbfm {
@@ -56,6 +57,16 @@ struct FarStage {
     T trial[32][TRI_REC + 1];
 };
 
+// The same for the barycentric quadrature (far_bary.cuh); the row pitch keeps 16-byte loads of consecutive rows apart.
+template <typename T>
+struct BaryStage {
+    T trec[FB_REC];
+    int32_t tv[4];
+    T trial[32][FB_REC + (sizeof(T) == 8 ? 2 : 0)];
+};
+template <typename T, bool LEAN>
+using StageOf = std::conditional_t<LEAN, BaryStage<T>, FarStage<T>>;
+
 template <int B>
 __device__ __forceinline__ void cp_async(void *dst_smem, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst_smem)),
@@ -73,7 +84,7 @@ __device__ __forceinline__ void cp_async(void *dst_smem, const void *src) {
 
 // One far triangle pair (t, s), t <= s (a near one is left to the near stage, which runs beside this one); rs is the
 // record of the trial triangle s.
-template <typename T, bool LEAN>
+template <typename T>
 __device__ __forceinline__ void far_pair(const FarStage<T> &S, int nt, const T *rs,
                                          const double *__restrict__ rec64, const int32_t *__restrict__ vid,
                                          double alpha, const MediaT<T> &md, cx<T> *__restrict__ Zloc, int t, int s) {
@@ -84,7 +95,20 @@ __device__ __forceinline__ void far_pair(const FarStage<T> &S, int nt, const T *
                      vs, alpha))
         return;
     cx<T> out[NCOMP];
-    far_entries<T, false, LEAN>(S.trec, 1, rs, md, out);
+    far_entries<T, false>(S.trec, 1, rs, md, out);
+    for (int c = 0; c < NCOMP; ++c) Zloc[c * plane + base] = out[c];
+}
+template <typename T>
+__device__ __forceinline__ void far_pair(const BaryStage<T> &S, int nt, const T *rs,
+                                         const double *__restrict__ rec64, const int32_t *__restrict__ vid,
+                                         double alpha, const MediaT<T> &md, cx<T> *__restrict__ Zloc, int t, int s) {
+    const int64_t plane = (int64_t)nt * nt;
+    const int64_t base = (int64_t)t * nt + s;
+    int32_t vs[3] = {vid[3 * s], vid[3 * s + 1], vid[3 * s + 2]};
+    T dc[3];
+    if (is_near_b<T>(S.trec, rs, rec64 + (int64_t)t * TRI_REC, rec64 + (int64_t)s * TRI_REC, S.tv, vs, alpha, dc)) return;
+    cx<T> out[NCOMP];
+    far_bary<T>(S.trec + FB_P, S.trec + FB_C, rs + FB_P, rs + FB_C, dc, md, out);
     for (int c = 0; c < NCOMP; ++c) Zloc[c * plane + base] = out[c];
 }
 
@@ -527,7 +551,7 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
 // the job of an item by binary search over the jobs' first item.
 template <typename T>
 struct AsmJob {
-    const T *rec;
+    const T *rec, *frec;
     const double *rec64;
     const int32_t *vid, *pairs, *edge_tri, *edge_loc;
     const int32_t *tri_cell;   // non-null: evaluate only pairs of triangles that share a cell
@@ -614,8 +638,8 @@ __global__ void __launch_bounds__(128) k_near_blocks(const AsmJob<T> *__restrict
 // memory.
 template <typename T>
 __host__ __device__ constexpr int far_warps() { return sizeof(T) == 4 ? 4 : 2; }
-template <typename T>
-constexpr size_t far_smem() { return (size_t)2 * far_warps<T>() * sizeof(FarStage<T>); }
+template <typename T, bool LEAN>
+constexpr size_t far_smem() { return (size_t)2 * far_warps<T>() * sizeof(StageOf<T, LEAN>); }
 
 template <typename T>
 __device__ __forceinline__ void far_stage(FarStage<T> &S, const AsmJob<T> &J, int t, int s0, int cnt, int lane) {
@@ -628,6 +652,17 @@ __device__ __forceinline__ void far_stage(FarStage<T> &S, const AsmJob<T> &J, in
 #pragma unroll 4
     for (int idx = lane; idx < cnt * TRI_REC; idx += 32)
         cp_async<sizeof(T)>(&S.trial[idx / TRI_REC][idx % TRI_REC], src + idx);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <typename T>
+__device__ __forceinline__ void far_stage(BaryStage<T> &S, const AsmJob<T> &J, int t, int s0, int cnt, int lane) {
+    constexpr int V = 16 / sizeof(T), NV = FB_REC / V;   // records are whole 16-byte pieces
+    if (lane < NV) cp_async<16>(&S.trec[lane * V], J.frec + (int64_t)t * FB_REC + lane * V);
+    if (lane >= 16 && lane < 19) cp_async<4>(&S.tv[lane - 16], J.vid + 3 * (int64_t)t + lane - 16);
+    const T *src = J.frec + (int64_t)s0 * FB_REC;
+#pragma unroll
+    for (int idx = lane; idx < 32 * NV; idx += 32)
+        if (idx < cnt * NV) cp_async<16>(&S.trial[idx / NV][idx % NV * V], src + idx * V);
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
@@ -657,7 +692,8 @@ __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
           int64_t npairs, int near_ctas) {
     extern __shared__ __align__(16) unsigned char far_raw[];
     const int lane = threadIdx.x & 31;
-    FarStage<T> *stage = reinterpret_cast<FarStage<T> *>(far_raw) + 2 * (threadIdx.x >> 5);
+    using Stage = StageOf<T, LEAN>;
+    Stage *stage = reinterpret_cast<Stage *>(far_raw) + 2 * (threadIdx.x >> 5);
     // the task being staged: job, test triangle, end of its strip
     int tj = 0, tt = 0, tse = 0;
     auto grab = [&](int &s0) -> bool {
@@ -689,7 +725,7 @@ __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
     for (int phase = 0; phase < 2; ++phase) {
     if ((phase == 0) == near_first) {
         if constexpr (sizeof(T) == 4) {
-            static_assert(sizeof(NearShared<T>) <= 2 * sizeof(FarStage<T>), "a warp's far stages hold its near scratch");
+            static_assert(sizeof(NearShared<T>) <= 2 * sizeof(Stage), "a warp's far stages hold its near scratch");
             if (npairs > 0) {
                 __syncwarp();
                 near_loop<T, LEAN>(jobs, njobs, npairs, 0, 0, *reinterpret_cast<NearShared<T> *>(stage), counter + 1);
@@ -722,7 +758,7 @@ __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
                     const int64_t plane = (int64_t)J.nt * J.nt, base = (int64_t)ct * J.nt + s;
                     for (int c = 0; c < NCOMP; ++c) J.Zloc[c * plane + base] = cx<T>(0, 0);
                 } else {
-                    far_pair<T, LEAN>(stage[b], J.nt, stage[b].trial[lane], J.rec64, J.vid, J.alpha, J.mdt, J.Zloc, ct, s);
+                    far_pair(stage[b], J.nt, stage[b].trial[lane], J.rec64, J.vid, J.alpha, J.mdt, J.Zloc, ct, s);
                 }
             }
         }
@@ -787,7 +823,7 @@ __global__ void __launch_bounds__(256) k_mirror(const AsmJob<T> *__restrict__ jo
 // projection reads, Zs[plane][op][i][f] (interleaved floats, zero up to the pitch ldz),
 // so that Z itself is neither written nor read again.  Bound: HBM, the 27 planes
 // of local blocks read once and the planes written once (9216-unknown cube: 0.50 ms
-// of gather and 0.34 ms of splitting -> GATHER_MS ms in one pass).
+// of gather and 0.34 ms of splitting -> 0.59 ms in one pass).
 template <typename T>
 __global__ void k_gather(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t nrows) {
     for (int64_t row = blockIdx.x; row < nrows; row += gridDim.x) {
@@ -855,9 +891,9 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
 // per stage.  The far stage's strip width (trial triangles per task) is
 // picked once per device and precision by timing the candidates, twice each,
 // on the first batch (every candidate writes the same values, so the batch
-// is not run again afterwards).  lean: the near pairs' closed forms and the
-// FP64 quadrature with the short elementary functions (near pairs of the
-// 9216-unknown cube 1.73 -> 1.15 ms by themselves); the conventional MoM, whose
+// is not run again afterwards).  lean: the near pairs' closed forms with the
+// short elementary functions (near pairs of the 9216-unknown cube 1.73 -> 1.15 ms
+// by themselves) and the far pairs in barycentric moments (far_bary.cuh); the conventional MoM, whose
 // long restarted solves carry a last bit of Z into the currents, and mixed
 // systems beyond SPREAD_MAX keep the general ones.
 template <typename T>
@@ -875,8 +911,8 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         Zloc[k].alloc((size_t)NCOMP * nt * nt);
         const Media md = media_full(m.k1, m.k2, m.eta1, m.eta2);
         AsmJob<T> &J = jobs[k];
-        if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p;
-        else J.rec = (const T *)m.tri32.p;
+        if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p, J.frec = (const T *)m.far64.p;
+        else J.rec = (const T *)m.tri32.p, J.frec = (const T *)m.far32.p;
         J.rec64 = m.tri64.p;
         J.vid = m.tri_vid.p;
         J.pairs = m.near_pairs.p;
@@ -921,6 +957,7 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
     // a first-launch delay or one noisy timing does not decide
     const int reps = tuned > 0 ? 1 : 2;
     auto *far = lean ? k_far<T, true> : k_far<T, false>;
+    const size_t far_sm = lean ? far_smem<T, true>() : far_smem<T, false>();
     auto *near = lean ? k_near_blocks<T, true> : k_near_blocks<T, false>;
     bool near_done = false;
     for (int rep = 0; rep < reps; ++rep)
@@ -936,15 +973,15 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         CBFM_CUDA(cudaMemcpyAsync(djobs.p, jobs.data(), sizeof(AsmJob<T>) * nj, cudaMemcpyHostToDevice, st));
         CBFM_CUDA(cudaMemsetAsync(counter.p, 0, 2 * sizeof(unsigned long long), st));
         constexpr int FB = 32 * far_warps<T>();
-        CBFM_CUDA(cudaFuncSetAttribute(far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)far_smem<T>()));
+        CBFM_CUDA(cudaFuncSetAttribute(far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)far_sm));
         int occ = 0;
-        CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, far, FB, far_smem<T>()));
+        CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, far, FB, far_sm));
         const unsigned grid = (unsigned)std::max(1, occ) * (unsigned)nsm;
         if (tuned > 0) {   // the near pairs beside the far ones (FP32 form)
             const bool both = sizeof(T) == 4 && npairs > 0;
             near_done = both;
             ProfScope ps_("k_far", st);
-            far<<<grid, FB, far_smem<T>(), st>>>(djobs.p, nj, ntask, counter.p, npairs, both ? 2 * nsm : 0);
+            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, npairs, both ? 2 * nsm : 0);
             launched("k_far");
             break;
         }
@@ -954,7 +991,7 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         CBFM_CUDA(cudaEventRecord(e0, st));
         {
             ProfScope ps_("k_far", st);
-            far<<<grid, FB, far_smem<T>(), st>>>(djobs.p, nj, ntask, counter.p, 0, 0);
+            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, 0, 0);
             launched("k_far");
         }
         CBFM_CUDA(cudaEventRecord(e1, st));
@@ -1011,8 +1048,8 @@ void near_blocks_compact_t(const std::vector<Mesh *> &ms, const std::vector<cx<T
         Mesh &m = *ms[k];
         AsmJob<T> &J = jobs[k];
         J = AsmJob<T>{};
-        if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p;
-        else J.rec = (const T *)m.tri32.p;
+        if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p, J.frec = (const T *)m.far64.p;
+        else J.rec = (const T *)m.tri32.p, J.frec = (const T *)m.far32.p;
         J.rec64 = m.tri64.p;
         J.vid = m.tri_vid.p;
         J.pairs = m.near_pairs.p;

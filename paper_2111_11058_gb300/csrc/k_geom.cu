@@ -3,6 +3,7 @@
 // Eq. (v); monostatic/bistatic RCS after Knott).
 #include <vector>
 
+#include "far_math.cuh"
 #include "internal.cuh"
 
 namespace cbfm {
@@ -34,7 +35,8 @@ __device__ inline double norm3_rn(double x, double y, double z) {
 __global__ void k_tri_records(int64_t nt, const double *__restrict__ V, const int32_t *__restrict__ tris,
                               const int32_t *__restrict__ tri_edge, const int32_t *__restrict__ tri_sign,
                               const double *__restrict__ edge_len, double cx, double cy, double cz,
-                              double *__restrict__ rec64, float *__restrict__ rec32) {
+                              double *__restrict__ rec64, float *__restrict__ rec32, double *__restrict__ far64,
+                              float *__restrict__ far32) {
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= nt) return;
     double v[3][3];
@@ -84,6 +86,20 @@ __global__ void k_tri_records(int64_t nt, const double *__restrict__ V, const in
         double x = r[TR_CEN + d] - c[d];
         float hi = (float)x;
         rec32[t * TRI_REC + TR_CLO + d] = (float)(x - (double)hi);
+    }
+    // records of the barycentric far quadrature, rounded once from FP64
+    double f[FB_REC];
+    for (int i = 0; i < FB_REC; ++i) f[i] = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        for (int d = 0; d < 3; ++d) f[fm::FB_P + 3 * a + d] = v[a][d] - r[TR_CEN + d];
+        f[fm::FB_C + a] = r[TR_C + a] * area;
+        f[fm::FB_CEN + a] = r[TR_CEN + a];
+    }
+    f[fm::FB_H] = h;
+    for (int i = 0; i < FB_REC; ++i) {
+        far64[t * FB_REC + i] = f[i];
+        const bool cen = i >= fm::FB_CEN && i < fm::FB_H;   // hi and lo parts as in the FP32 record above
+        far32[t * FB_REC + i] = cen ? rec32[t * TRI_REC + TR_CEN + (i - fm::FB_CEN) + (i >= fm::FB_CLO ? 1 : 0)] : (float)f[i];
     }
 }
 
@@ -371,7 +387,7 @@ void launch_tri_records(Mesh &m, const double *d_verts, const int32_t *d_tris, c
         ProfScope ps_("k_tri_records", st);
         k_tri_records<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>(nt, d_verts, d_tris, m.tri_edge.p, d_sign.p, d_len.p,
                                                                     m.centre[0], m.centre[1], m.centre[2], m.tri64.p,
-                                                                    m.tri32.p);
+                                                                    m.tri32.p, m.far64.p, m.far32.p);
         launched("k_tri_records");
     }
     CBFM_CUDA(cudaStreamSynchronize(st));
