@@ -50,13 +50,13 @@ __device__ __forceinline__ PF pmk(float a, float b) {
 }
 __device__ __forceinline__ PD pmk(double a, double b) { return PD{a, b}; }
 __device__ __forceinline__ float plo(PF x) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    float a;
+    asm("{\n .reg .f32 t;\n mov.b64 {%0, t}, %1;\n}" : "=f"(a) : "l"(x.v));
     return a;
 }
 __device__ __forceinline__ float phi(PF x) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    float b;
+    asm("{\n .reg .f32 t;\n mov.b64 {t, %0}, %1;\n}" : "=f"(b) : "l"(x.v));
     return b;
 }
 __device__ __forceinline__ double plo(PD x) { return x.a; }
@@ -106,12 +106,11 @@ __device__ __forceinline__ double brsqrt(double x) { return f64::rsqrt64(x); }
 constexpr double Q7_S15 = 3.87298334620741688517926539978;
 constexpr double Q7_B1 = (6.0 - Q7_S15) / 21.0, Q7_B2 = (6.0 + Q7_S15) / 21.0;
 constexpr double Q7_W0 = 9.0 / 40.0, Q7_W1 = (155.0 - Q7_S15) / 1200.0, Q7_W2 = (155.0 + Q7_S15) / 1200.0;
-constexpr double Q7_T1 = 1.0 - 3.0 * Q7_B1, Q7_T2 = 1.0 - 3.0 * Q7_B2;   // point = T p_k from the centroid
 
-// barycentric coordinates (rows 0-2) and weighted ones (3-5) of point p
+// barycentric coordinates of point p, plain and weighted; per orbit: distance factor T, weight times b, weight times T
 template <typename T>
 struct Q7Tab {
-    T l[7][3], wl[7][3];
+    T l[7][3], wl[7][3], orb[2][3];
 };
 template <typename T>
 constexpr Q7Tab<T> q7_tab() {
@@ -124,6 +123,12 @@ constexpr Q7Tab<T> q7_tab() {
             t.l[p][j] = (T)l;
             t.wl[p][j] = (T)(w * l);
         }
+    for (int o = 0; o < 2; ++o) {
+        const double b = o == 0 ? Q7_B1 : Q7_B2, w = o == 0 ? Q7_W1 : Q7_W2;
+        t.orb[o][0] = (T)(1.0 - 3.0 * b);
+        t.orb[o][1] = (T)(w * b);
+        t.orb[o][2] = (T)(w * (1.0 - 3.0 * b));
+    }
     return t;
 }
 static __constant__ Q7Tab<float> q7f = q7_tab<float>();
@@ -151,10 +156,13 @@ __device__ __forceinline__ bool is_near_b(const T *rt, const T *rs, const double
 
 // The 27 local entries (op x 3 x 3, op = Ks, Ta, Tb) of a far pair: pt, ps the
 // vertices of the test and trial triangle relative to their centroids, at, as
-// the coefficients c_a times the area, dc the centroid difference.
-// PS: anything indexable by 0..8 (registers or shared memory).
-template <typename T, typename PT, typename PS>
-__device__ __forceinline__ void far_bary(const PT &pt, const PT &at, const PS &ps, const PS &as, const T dc[3],
+// the coefficients c_a times the area, dc the centroid difference.  ROLL keeps the
+// two orbits in one loop body (fewer instructions to fetch, a few more to execute):
+// the FP32 far kernel is faster without (0.85 against 0.96 ms on the 9216-unknown
+// cube), FP64 (3.37 against 3.44 ms) and the fused kernel, whose warps run in
+// different places of a longer program (31 against 38 ms), with it.
+template <typename T, bool ROLL>
+__device__ __forceinline__ void far_bary(const T *pt, const T *at, const T *ps, const T *as, const T dc[3],
                                          const MediaT<T> &md, cx<T> *out) {
     using P = typename PairOf<T>::type;
     const bool lossy2 = md.ki[1] != (T)0;
@@ -174,20 +182,13 @@ __device__ __forceinline__ void far_bary(const PT &pt, const PT &at, const PS &p
         for (int d = 0; d < 3; ++d)
             Dp[d] = dc[d] + (tab.l[p][0] * pt[d] + tab.l[p][1] * pt[3 + d] + tab.l[p][2] * pt[6 + d]);
         P U[4][3], S[4];   // sums of w G lambda_k, w g lambda_k; the part common to the three k
-#pragma unroll
-        for (int q = 0; q < 7; ++q) {
-            const int k = (q + 2) % 3;   // vertex of an orbit point
-            const T tau = (T)(q < 4 ? Q7_T1 : Q7_T2);
-            T d[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) d[c] = q == 0 ? Dp[c] : Dp[c] - tau * ps[3 * k + c];
+        auto point = [&](const T d[3], P G[4]) {
             const T R2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
             const T iR = brsqrt(R2), R = R2 * iR, h = iR * iR;
             const P RR = pmk(R, R), hh = pmk(h, h);
             const P kR = pmul(RR, kk), nkR = pmul(RR, nk);
             P sn, cs;
             psincos(kR, sn, cs);
-            P G[4];
             if (lossy2) {
                 const P aa = pmk(iR, iR * exp_t(md.ki[1] * R));
                 const P o = pmk((T)1, (T)1 - md.ki[1] * R);
@@ -202,12 +203,34 @@ __device__ __forceinline__ void far_bary(const PT &pt, const PT &at, const PS &p
                 G[2] = pmul(hh, pfma(kR, G[1], G[0]));
                 G[3] = pmul(hh, pfma(nkR, G[0], G[1]));
             }
-            const T wc = (T)(q == 0 ? Q7_W0 / 3.0 : q < 4 ? Q7_W1 * Q7_B1 : Q7_W2 * Q7_B2);
-            const T wk = (T)(q < 4 ? Q7_W1 * Q7_T1 : Q7_W2 * Q7_T2);
+        };
+        {
+            P G[4];
+            point(Dp, G);
+            const P wc = pmk((T)(Q7_W0 / 3.0), (T)(Q7_W0 / 3.0));
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
-                S[x] = q == 0 ? pmul(pmk(wc, wc), G[x]) : pfma(pmk(wc, wc), G[x], S[x]);
-                if (q >= 1) U[x][k] = q < 4 ? pmul(pmk(wk, wk), G[x]) : pfma(pmk(wk, wk), G[x], U[x][k]);
+                S[x] = pmul(wc, G[x]);
+                U[x][0] = U[x][1] = U[x][2] = pmk((T)0, (T)0);
+            }
+        }
+        // ROLL: the two orbits share one body
+#pragma unroll(ROLL ? 1 : 2)
+        for (int o = 0; o < 2; ++o) {
+            const T tau = ROLL ? tab.orb[o][0] : (T)(1.0 - 3.0 * (o == 0 ? Q7_B1 : Q7_B2));
+            const T wcs = ROLL ? tab.orb[o][1] : (T)(o == 0 ? Q7_W1 * Q7_B1 : Q7_W2 * Q7_B2);
+            const T wks = ROLL ? tab.orb[o][2] : (T)(o == 0 ? Q7_W1 * (1.0 - 3.0 * Q7_B1) : Q7_W2 * (1.0 - 3.0 * Q7_B2));
+            const P wc = pmk(wcs, wcs), wk = pmk(wks, wks);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                P G[4];
+                const T d[3] = {Dp[0] - tau * ps[3 * k], Dp[1] - tau * ps[3 * k + 1], Dp[2] - tau * ps[3 * k + 2]};
+                point(d, G);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    S[x] = pfma(wc, G[x], S[x]);
+                    U[x][k] = !ROLL && o == 0 ? pmul(wk, G[x]) : pfma(wk, G[x], U[x][k]);
+                }
             }
         }
 #pragma unroll

@@ -277,12 +277,11 @@ void noalloc_prepare();
 // every cell the triangles that carry one of its RWG functions (spatially
 // ordered), the fused kernel's chunks of them, and the near list as a CSR.
 struct FusedTables {
-    std::vector<int32_t> tl_off, ch_off;   // per cell: offsets into tl and into the chunk table (host)
-    DevBuf<int4> tl;                       // per list entry: {triangle, rows a0 | a1 << 16, row a2 | cols b0, b1 << 24, col b2}
-    DevBuf<int32_t> dtl_off, dch_off;
-    DevBuf<int2> chunk;                    // per chunk: [begin, end) into tl
-    DevBuf<int16_t> chunk_cols;            // per chunk: the fused kernel's cell-local RWG columns (-1: padding)
-    DevBuf<float> recT;                    // FP32 triangle records of the list entries, field-major (48 x entries)
+    std::vector<int32_t> tl_off;           // per cell: offsets into tl (host)
+    DevBuf<int4> tl;                       // per list entry: {triangle, rows a0 | a1 << 16, row a2 | sides << 16, 0}
+    DevBuf<int32_t> dtl_off, tl_cell;      // offsets; cell of each entry
+    DevBuf<float> farT;                    // FP32 far records of the list entries, field-major (FB_REC x entries)
+    DevBuf<float> trial;                   // per entry: far record, vertex ids, triangle (the fused kernel's FuTrial)
     DevBuf<int32_t> vidT;                  // vertex ids of the list entries, field-major (3 x entries)
     DevBuf<int2> rwg_pos;                  // per internal edge: list positions (in its cell's list) of its + and - triangles
     DevBuf<int32_t> near_row;              // nt + 1: CSR of the near list over test triangles

@@ -108,7 +108,7 @@ __device__ __forceinline__ void far_pair(const BaryStage<T> &S, int nt, const T 
     T dc[3];
     if (is_near_b<T>(S.trec, rs, rec64 + (int64_t)t * TRI_REC, rec64 + (int64_t)s * TRI_REC, S.tv, vs, alpha, dc)) return;
     cx<T> out[NCOMP];
-    far_bary<T>(S.trec + FB_P, S.trec + FB_C, rs + FB_P, rs + FB_C, dc, md, out);
+    far_bary<T, sizeof(T) == 8>(S.trec + FB_P, S.trec + FB_C, rs + FB_P, rs + FB_C, dc, md, out);
     for (int c = 0; c < NCOMP; ++c) Zloc[c * plane + base] = out[c];
 }
 

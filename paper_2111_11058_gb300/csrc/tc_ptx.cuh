@@ -143,5 +143,15 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
+// The same with the 32-byte swizzle (8 floats per row, one K step): 16-byte chunk index XOR address bit 7,
+// 8-row groups 256 bytes apart, swizzle mode 6.
+__device__ __forceinline__ uint32_t swz32(int r, int f) {
+    return (uint32_t)r * 32u + ((((uint32_t)(f >> 2)) ^ (((uint32_t)r >> 2) & 1u)) << 4) + ((uint32_t)(f & 3) << 2);
+}
+__device__ __forceinline__ uint64_t sdesc32(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256u >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+
 }  // namespace tc
 }  // namespace cbfm

@@ -46,3 +46,21 @@ def test_identity_blocks_are_the_rwg_matrix(P, shape, eps):
         A = P.assemble_reduced(gm, cb, prec).export()
         assert A.shape == Z.shape
         assert np.abs(A - Z).max() < tol * np.abs(Z).max(), prec
+
+
+# fused form: many cells with fewer triangles than a warp has lanes, single CBFs, cell pairs with the
+# conjugate lanes (L <= 16) up to their limit and beyond it, one cell, tiles close to N = 256
+@pytest.mark.parametrize("shape,nc,L", [("cube4", 60, 1), ("cube4", 24, 3), ("ico2", 9, 16), ("ico2", 4, 17),
+                                        ("ico2", 2, 8), ("cube3", 1, 16), ("ico2", 6, 32)])
+def test_fused_cell_pairs(P, shape, nc, L):
+    """Fused against unfused, both FP32 quadrature and split TF32: 5e-6 of the largest entry (above)."""
+    n = int(shape[-1])
+    g = W.cube(n, 0.8) if shape.startswith("cube") else W.icosphere(n, 0.5)
+    gm = P.mesh(g.verts, g.tris, nc, 3.0 - 0.1j, partition="rcb")
+    Ns = np.bincount(gm.cells(), minlength=nc)
+    CM, CJ = W.random_cbfs(Ns, [min(L, k) for k in Ns], seed=3)
+    cb = P.cbf_import(gm, CM, CJ)
+    Af = P.assemble_reduced(gm, cb, P.MIXED_FUSED).export()
+    Au = P.assemble_reduced(gm, cb, P.MIXED_UNFUSED).export()
+    assert np.isfinite(Af).all()
+    assert np.abs(Af - Au).max() < 5e-6 * np.abs(Au).max()
