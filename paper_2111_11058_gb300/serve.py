@@ -21,6 +21,9 @@ The service
   (a batch building or solving it) joins that group -- appended while the
   entry is built, and handed to the running block GMRES session otherwise,
   which takes it at its next block-iteration boundary (`cbfm_session_join`);
+  the group stays open after its solve, up to as long as the batch took, while
+  its worker has nothing else to do: a request that comes then is solved at
+  once as part of the batch;
   only when no group is open, or the group is full, does it wait;
 * runs batches on several CUDA streams at once (one worker thread per
   stream; the library releases the GIL during its calls and its scratch
@@ -46,6 +49,7 @@ from typing import Any, Dict, List, Optional, Tuple
 import numpy as np
 
 MAX_BLOCK_RHS = 128   # block GMRES groups (the library's block width)
+KEEP_OPEN_S = 0.05    # longest time a solved group stays open for joins on an otherwise idle worker
 
 
 @dataclasses.dataclass(frozen=True)
@@ -252,7 +256,9 @@ class _Group:
         self.hit = hit
         self.members: List[list] = []     # [request, future, first slot or None]
         self.nrhs = 0
-        self.state = "pending"            # pending (joins append) -> running (joins go to the session) -> done
+        # pending (joins append) -> running (joins go to the session) -> idle (solved, its worker has nothing else to
+        # do: joins append and are solved next) -> done
+        self.state = "pending"
         self.session: Any = None
         self.scratch = 0                  # solve scratch accounted for this group
         self.joined = 0                   # requests that joined after the batch started
@@ -279,6 +285,8 @@ class Server:
         self.rid = itertools.count()
         self.bid = itertools.count()
         self.running = True
+        self.draining = 0                                      # callers in drain()
+        self.idle = 0                                          # workers that only keep a solved group open
         self.log: List[dict] = []                              # one record per finished batch
         self.hits = self.misses = self.evictions = 0
         self.streams = [backend.make_stream() for _ in range(n_streams)]
@@ -299,14 +307,19 @@ class Server:
             if not self._try_join(req, fut):
                 self.waiting.append((req, fut))
                 self._dispatch()
+                if self.waiting:
+                    self.lock.notify_all()     # a worker that keeps an idle group open takes it
         return fut
 
     def drain(self, timeout: float = 600.0) -> None:
         """Wait until nothing waits or runs (every finished batch is in the log)."""
         end = time.perf_counter() + timeout
         with self.lock:
+            self.draining += 1
+            self.lock.notify_all()
             while (self.waiting or any(self.busy)) and time.perf_counter() < end:
                 self.lock.wait(timeout=0.05)
+            self.draining -= 1
 
     def close(self) -> None:
         with self.lock:
@@ -349,7 +362,35 @@ class Server:
         g.scratch += delta
         g.joined += 1
         self._account(delta)
+        if g.state == "idle":
+            self.lock.notify_all()
         return True
+
+    def _keep_open(self, g: _Group, seconds: float) -> bool:
+        """Keep a solved group open for joins while nothing else waits, for as long
+        as its batch took; true if a request joined.  A request that comes just
+        after a short solve is then solved at once on the resident entry."""
+        end = time.perf_counter() + seconds
+        with self.lock:
+            if g.key in self.open or not self.joins:
+                return False
+            g.members, g.nrhs, g.state, g.session = [], 0, "idle", None
+            self.inflight -= g.scratch
+            g.scratch = 0
+            self.open[g.key] = g
+            self.idle += 1
+            while self.running and not self.draining and not self.waiting and not g.members:
+                left = end - time.perf_counter()
+                if left <= 0:
+                    break
+                self.lock.wait(left)
+            self.idle -= 1
+            if g.members:
+                g.state = "pending"
+                return True
+            g.state = "done"
+            del self.open[g.key]
+            return False
 
     def _footprint(self, req: Request, nrhs: int) -> Tuple[int, bool]:
         """(bytes the batch adds, whether its entry is already resident or being built)."""
@@ -425,7 +466,7 @@ class Server:
                     # a cache miss: when this is the last free worker, other waiting misses of other
                     # keys are built in the same batch (idle workers would rather take them in parallel)
                     todo = [(req.key, group, nrhs, need)]
-                    gather = self.busy.count(False) == 1
+                    gather = self.busy.count(False) + self.idle == 1
                     for r3, _f3 in list(self.waiting):
                         if not gather or len(todo) >= self.max_build_keys:
                             break
@@ -462,6 +503,51 @@ class Server:
                 return
 
     # ---- workers
+    def _solve_group(self, g: _Group, st, bid: int) -> Tuple[int, int]:
+        """Solves an open group and delivers its results; returns the requests and right-hand sides served."""
+        err: Optional[BaseException] = g.entry.error
+        rcs = iters = None
+        if err is None:
+            try:
+                with self.lock:
+                    exc = np.concatenate([m[0].exc for m in g.members], axis=0)
+                    ofs = 0
+                    for m in g.members:
+                        m[2] = ofs
+                        ofs += m[0].nrhs
+                    if hasattr(self.be, "open_session"):
+                        g.session = self.be.open_session(g.entry.handle, exc, st)
+                        g.state = "running"
+                    else:
+                        g.state = "done"
+                        del self.open[g.key]
+                if g.session is not None:
+                    rcs, iters = g.session.run()
+                else:
+                    rcs, iters = self.be.solve(g.entry.handle, exc, st)
+            except BaseException as e:  # delivered to the requests of the group
+                err = e
+        t_end = time.perf_counter()
+        with self.lock:
+            if g.state != "done":
+                g.state = "done"
+                if self.open.get(g.key) is g:
+                    del self.open[g.key]
+            requeue = []
+            nsolved = 0 if rcs is None else int(rcs.shape[0])
+            for req, fut, slot in g.members:
+                if err is not None:
+                    fut.set_exception(err)
+                elif slot is not None and slot + req.nrhs <= nsolved:
+                    fut.set_result(Result(req.rid, rcs[slot:slot + req.nrhs], iters[slot:slot + req.nrhs],
+                                          t_end - req.arrival, bid, nsolved, g.hit))
+                else:
+                    requeue.append((req, fut))   # joined too late for the solve: wait again
+            if g.session is not None and hasattr(g.session, "free"):
+                g.session.free()
+            self.waiting[0:0] = requeue
+            return len(g.members), g.nrhs
+
     def _worker(self, w: int) -> None:
         st = self.streams[w]
         while True:
@@ -500,66 +586,32 @@ class Server:
                 if g.hit:
                     g.entry.ready.wait()
             # the solves, one session per key; joins reach a session while it runs
-            for g in groups:
-                err: Optional[BaseException] = g.entry.error
-                rcs = iters = None
-                if err is None:
-                    try:
-                        with self.lock:
-                            exc = np.concatenate([m[0].exc for m in g.members], axis=0)
-                            ofs = 0
-                            for m in g.members:
-                                m[2] = ofs
-                                ofs += m[0].nrhs
-                            if hasattr(self.be, "open_session"):
-                                g.session = self.be.open_session(g.entry.handle, exc, st)
-                                g.state = "running"
-                            else:
-                                g.state = "done"
-                                del self.open[g.key]
-                        if g.session is not None:
-                            rcs, iters = g.session.run()
-                        else:
-                            rcs, iters = self.be.solve(g.entry.handle, exc, st)
-                    except BaseException as e:  # delivered to the requests of the group
-                        err = e
-                t_end = time.perf_counter()
-                with self.lock:
-                    if g.state != "done":
-                        g.state = "done"
-                        if self.open.get(g.key) is g:
-                            del self.open[g.key]
-                    requeue = []
-                    nsolved = 0 if rcs is None else int(rcs.shape[0])
-                    for req, fut, slot in g.members:
-                        if err is not None:
-                            fut.set_exception(err)
-                        elif slot is not None and slot + req.nrhs <= nsolved:
-                            fut.set_result(Result(req.rid, rcs[slot:slot + req.nrhs], iters[slot:slot + req.nrhs],
-                                                  t_end - req.arrival, bid, nsolved, g.hit))
-                        else:
-                            requeue.append((req, fut))   # joined too late for the solve: wait again
-                    if g.session is not None and hasattr(g.session, "free"):
-                        g.session.free()
-                    self.waiting[0:0] = requeue
-            ev1 = self.be.event(st) if ev0 is not None else None
-            t_end = time.perf_counter()
-            rec = {"batch": bid, "worker": w, "keys": [g.key for g in groups],
-                   "requests": sum(len(g.members) for g in groups), "joined": sum(g.joined for g in groups),
-                   "rhs": sum(g.nrhs for g in groups), "hit": all(g.hit for g in groups), "t_start": t_start,
-                   "t_end": t_end, "error": any(g.entry.error is not None for g in groups)}
-            if ev0 is not None:
-                rec["dev_ms"] = (self.be.elapsed_ms(self.t0_event, ev0), self.be.elapsed_ms(self.t0_event, ev1))
+            rec = {"batch": bid, "worker": w, "keys": [g.key for g in groups], "requests": 0, "joined": 0, "rhs": 0,
+                   "hit": all(g.hit for g in groups), "t_start": t_start}
+
+            def served(counts):   # the batch's record so far
+                ev1 = self.be.event(st) if ev0 is not None else None
+                rec.update(requests=rec["requests"] + sum(c[0] for c in counts), rhs=rec["rhs"] + sum(c[1] for c in counts),
+                           joined=sum(g.joined for g in groups), t_end=time.perf_counter(),
+                           error=any(g.entry.error is not None for g in groups))
+                if ev0 is not None:
+                    rec["dev_ms"] = (self.be.elapsed_ms(self.t0_event, ev0), self.be.elapsed_ms(self.t0_event, ev1))
+
+            served([self._solve_group(g, st, bid) for g in groups])
+            with self.lock:
+                self.log.append(rec)
+            if len(groups) == 1 and not rec["error"] and hasattr(self.be, "open_session"):
+                while self._keep_open(groups[0], min(time.perf_counter() - t_start, KEEP_OPEN_S)):
+                    served([self._solve_group(groups[0], st, bid)])
             with self.lock:
                 for g in groups:
                     g.entry.users -= 1
-                    g.entry.last_used = t_end
+                    g.entry.last_used = rec["t_end"]
                     if g.entry.error is not None and self.cache.get(g.entry.key) is g.entry:
                         del self.cache[g.entry.key]               # a failed build is not cached
                     self.inflight -= g.scratch
                 self.busy[w] = False
                 self.work[w] = None
-                self.log.append(rec)
                 self._dispatch()
                 self.lock.notify_all()
 
