@@ -755,8 +755,11 @@ cbfm_status cbfm_build_cbfs(cbfm_mesh_t mesh, const double *waves, int32_t s, do
         std::vector<int> hinfo(nc);
         CBFM_CUDA(cudaMemcpyAsync(hinfo.data(), info.p, sizeof(int) * nc, cudaMemcpyDeviceToHost, st));
         CBFM_CUDA(cudaStreamSynchronize(st));
-        for (int c = 0; c < nc; ++c)
+        for (int c = 0; c < nc; ++c) {
+            if (hinfo[c] == 2)
+                throw Fail{CBFM_ETIMEOUT, "Z_mm solve: a cluster synchronisation expired in cell " + std::to_string(c)};
             if (hinfo[c]) throw Fail{CBFM_ESINGULAR, "singular Z_mm in cell " + std::to_string(c)};
+        }
         Zmm.release();
         std::unique_ptr<Cbf> cb = dual_cbfs(m, s, Vm.p, voff, delta_svd, lmax, L_per_cell, sigma_out, st);
         CBFM_CUDA(cudaStreamSynchronize(st));

@@ -478,24 +478,75 @@ void gemm_dir(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z
 
 // ------------------------------------------------------ batched LU solve
 // Gaussian elimination with partial pivoting on [Z | V], then backward
-// substitution; one block per system.
-__global__ void __launch_bounds__(256) k_lu_solve(const int64_t *__restrict__ zoff, const int64_t *__restrict__ voff,
-                                                  const int *__restrict__ nsz, int s, z64 *__restrict__ Zall,
-                                                  z64 *__restrict__ Vall, int *__restrict__ info) {
-    const int b = blockIdx.x;
+// substitution.  One cluster of LU_CL CTAs per system, the columns of Z and V in
+// blocks of eight dealt to the CTAs: a step's pivot, row exchange and
+// multipliers need only column k, which every CTA reads (through L2) and works
+// through by itself, so a step takes one cluster synchronisation, and the
+// substitution, whose right-hand sides are independent, takes none.  Every entry
+// goes through the operations of the plain elimination in the same order.
+//
+// Bound: the FP64 pipes, of eight SMs instead of one (16 systems of 147 unknowns
+// with 128 right-hand sides: 8.3 ms -> 2.1 ms), then the step's serial chain (the
+// column through L2, the pivot search, one division).  col, dinv: n entries each
+// per CTA, in shared memory where they fit.  info[b] = 1: singular; 2: a cluster
+// synchronisation expired.
+constexpr int LU_CL = 8;
+
+// FP64 products with the rounding written out, in this and the next kernel: the CBFs they
+// give decide, through solves that amplify a last bit, the digits of every later result, so
+// their operations do not follow the compiler's choice of which product of a sum is fused.
+__device__ __forceinline__ double norm2_rn(z64 a) { return __fma_rn(a.re, a.re, __dmul_rn(a.im, a.im)); }
+__device__ __forceinline__ z64 mul_rn(z64 a, z64 b) {   // Im: Im a Re b fused
+    return z64(__fma_rn(a.re, b.re, -__dmul_rn(a.im, b.im)), __fma_rn(a.im, b.re, __dmul_rn(a.re, b.im)));
+}
+__device__ __forceinline__ z64 mul2_rn(z64 a, z64 b) {  // Im: Re a Im b fused
+    return z64(__fma_rn(a.re, b.re, -__dmul_rn(a.im, b.im)), __fma_rn(a.re, b.im, __dmul_rn(a.im, b.re)));
+}
+__device__ __forceinline__ z64 sub_rn(z64 a, z64 b) { return z64(__dsub_rn(a.re, b.re), __dsub_rn(a.im, b.im)); }
+__device__ __forceinline__ z64 inv_rn(z64 d) {
+    const double n = norm2_rn(d);
+    return n > 0.0 ? z64(__ddiv_rn(d.re, n), __ddiv_rn(-d.im, n)) : z64(0, 0);
+}
+
+__device__ __forceinline__ z64 ldcg64(const z64 *p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+    return z64(v.x, v.y);
+}
+
+__global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
+    k_lu_solve(const int64_t *__restrict__ zoff, const int64_t *__restrict__ voff, const int *__restrict__ nsz, int s,
+               z64 *__restrict__ Zall, z64 *__restrict__ Vall, int *__restrict__ info, z64 *__restrict__ scratch,
+               int nmax) {
+    extern __shared__ __align__(16) unsigned char lu_raw[];
+    cg::cluster_group cl = cg::this_cluster();
+    const int me = (int)cl.block_rank(), b = blockIdx.x / LU_CL;
     const int n = nsz[b];
     z64 *Z = Zall + zoff[b];
     z64 *V = Vall + voff[b];
-    __shared__ int piv;
+    z64 *col = scratch ? scratch + (int64_t)blockIdx.x * 2 * nmax : reinterpret_cast<z64 *>(lu_raw);
+    z64 *dinv = col + nmax;
+    __shared__ uint64_t cbar[2];
+    __shared__ int piv, s_abort;
     __shared__ z64 pinv;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < n; ++k) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c8 = tid & 7, r32 = tid >> 3;   // column within a block of eight, row within 32
+    const int nbz = (n + 7) >> 3, nbv = (s + 7) >> 3;
+    if (tid == 0) {
+        cl_bar_init(cbar, LU_CL);
+        s_abort = 0;
+    }
+    __syncthreads();
+    cl.sync();   // barriers initialised in every CTA (unconditional)
+    bool ok = true;
+    for (int k = 0; k < n && ok; ++k) {
+        for (int i = k + tid; i < n; i += blockDim.x) col[i] = ldcg64(Z + (int64_t)i * n + k);
+        __syncthreads();
         // pivot search by warp 0: largest |Z[i][k]|^2 (first on ties), bit patterns compared as integers
         if (warp == 0) {
             long long best = -1;
             int bi = k;
             for (int i = k + lane; i < n; i += 32) {
-                const long long v = __double_as_longlong(norm2(Z[(int64_t)i * n + k]));
+                const long long v = __double_as_longlong(norm2_rn(col[i]));
                 if (v > best) {
                     best = v;
                     bi = i;
@@ -511,65 +562,84 @@ __global__ void __launch_bounds__(256) k_lu_solve(const int64_t *__restrict__ zo
             }
             if (lane == 0) {
                 piv = bi;
-                if (best <= 0) info[b] = 1;
+                if (best <= 0 && me == 0) info[b] = 1;
+                const z64 d = col[bi];
+                col[bi] = col[k];
+                col[k] = d;
+                pinv = inv_rn(d);
             }
         }
         __syncthreads();
         const int p = piv;
+        // the multipliers once per row
+        for (int i = k + 1 + tid; i < n; i += blockDim.x) col[i] = mul_rn(col[i], pinv);
+        // row exchange in this CTA's columns (of column k only the diagonal is used again)
         if (p != k) {
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                z64 t = Z[(int64_t)k * n + j];
-                Z[(int64_t)k * n + j] = Z[(int64_t)p * n + j];
-                Z[(int64_t)p * n + j] = t;
+            for (int jb = me + LU_CL * r32; jb < nbz; jb += LU_CL * 32) {
+                const int j = 8 * jb + c8;
+                if (j > k && j < n) {
+                    z64 t = Z[(int64_t)k * n + j];
+                    Z[(int64_t)k * n + j] = Z[(int64_t)p * n + j];
+                    Z[(int64_t)p * n + j] = t;
+                }
             }
-            for (int j = threadIdx.x; j < s; j += blockDim.x) {
-                z64 t = V[(int64_t)k * s + j];
-                V[(int64_t)k * s + j] = V[(int64_t)p * s + j];
-                V[(int64_t)p * s + j] = t;
+            for (int jb = me + LU_CL * r32; jb < nbv; jb += LU_CL * 32) {
+                const int j = 8 * jb + c8;
+                if (j < s) {
+                    z64 t = V[(int64_t)k * s + j];
+                    V[(int64_t)k * s + j] = V[(int64_t)p * s + j];
+                    V[(int64_t)p * s + j] = t;
+                }
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            z64 d = Z[(int64_t)k * n + k];
-            pinv = (norm2(d) > 0.0) ? cdiv(z64(1, 0), d) : z64(0, 0);
-        }
-        __syncthreads();
-        // multipliers once per row, kept in column k
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) Z[(int64_t)i * n + k] = Z[(int64_t)i * n + k] * pinv;
-        __syncthreads();
+        if (tid == 0) dinv[k] = pinv;
         // eliminate below
-        const int rows = n - k - 1;
-        const int wcols = (n - k - 1) + s;
-        for (int64_t idx = threadIdx.x; idx < (int64_t)rows * wcols; idx += blockDim.x) {
-            int i = k + 1 + (int)(idx / wcols);
-            int c = (int)(idx % wcols);
-            const z64 l = Z[(int64_t)i * n + k];
-            if (c < n - k - 1) {
-                int j = k + 1 + c;
-                Z[(int64_t)i * n + j] -= l * Z[(int64_t)k * n + j];
-            } else {
-                int j = c - (n - k - 1);
-                V[(int64_t)i * s + j] -= l * V[(int64_t)k * s + j];
+        for (int jb = me + LU_CL * ((((k + 1) >> 3) + LU_CL - 1 - me) / LU_CL); jb < nbz; jb += LU_CL) {
+            const int j = 8 * jb + c8;
+            if (j <= k || j >= n) continue;
+            const z64 u = Z[(int64_t)k * n + j];
+#pragma unroll 4
+            for (int i = k + 1 + r32; i < n; i += 32) {
+                z64 &z = Z[(int64_t)i * n + j];
+                z = sub_rn(z, mul_rn(col[i], u));
+            }
+        }
+        for (int jb = me; jb < nbv; jb += LU_CL) {
+            const int j = 8 * jb + c8;
+            if (j >= s) continue;
+            const z64 u = V[(int64_t)k * s + j];
+#pragma unroll 4
+            for (int i = k + 1 + r32; i < n; i += 32) {
+                z64 &v = V[(int64_t)i * s + j];
+                v = sub_rn(v, mul_rn(col[i], u));
+            }
+        }
+        ok = cl_sync(cbar, k, LU_CL, &s_abort, info + b);
+    }
+    // backward substitution, column oriented, on this CTA's right-hand sides
+    for (int k = n - 1; k >= 0 && ok; --k) {
+        for (int i = tid; i < k; i += blockDim.x) col[i] = ldcg64(Z + (int64_t)i * n + k);
+        const z64 di = dinv[k];
+        for (int jb = me + LU_CL * r32; jb < nbv; jb += LU_CL * 32) {
+            const int j = 8 * jb + c8;
+            if (j < s) V[(int64_t)k * s + j] = mul2_rn(V[(int64_t)k * s + j], di);
+        }
+        __syncthreads();
+        for (int jb = me; jb < nbv; jb += LU_CL) {
+            const int j = 8 * jb + c8;
+            if (j >= s) continue;
+            const z64 u = V[(int64_t)k * s + j];
+#pragma unroll 4
+            for (int i = r32; i < k; i += 32) {
+                z64 &v = V[(int64_t)i * s + j];
+                v = sub_rn(v, mul_rn(col[i], u));
             }
         }
         __syncthreads();
     }
-    // backward substitution, column oriented
-    for (int k = n - 1; k >= 0; --k) {
-        if (threadIdx.x == 0) {
-            const z64 d = Z[(int64_t)k * n + k];
-            pinv = (norm2(d) > 0.0) ? cdiv(z64(1, 0), d) : z64(0, 0);
-        }
-        __syncthreads();
-        const z64 dinv = pinv;
-        for (int j = threadIdx.x; j < s; j += blockDim.x) V[(int64_t)k * s + j] = V[(int64_t)k * s + j] * dinv;
-        __syncthreads();
-        for (int64_t idx = threadIdx.x; idx < (int64_t)k * s; idx += blockDim.x) {
-            int i = (int)(idx / s), j = (int)(idx % s);
-            V[(int64_t)i * s + j] -= Z[(int64_t)i * n + k] * V[(int64_t)k * s + j];
-        }
-        __syncthreads();
-    }
+    if (!ok && tid == 0) atomicExch(info + b, 2);
+    cl.sync();   // no CTA leaves while another may still arrive on its barriers
 }
 
 // ---------------------------------------------- one-sided Jacobi SVD
@@ -585,10 +655,19 @@ __global__ void __launch_bounds__(256) k_lu_solve(const int64_t *__restrict__ zo
 // (flags exchanged through distributed shared memory), so all CTAs run the
 // same number of rounds and sweeps.  info[mat] = 2: no convergence in 60
 // sweeps; 1: a cluster synchronisation expired.
-constexpr int JS_CL = 8;
+//
+// A round of a CTA's eight pairs: each warp forms the products of its pair, the
+// first warp works out all eight rotations side by side (the chain of square roots
+// and divisions, about 150 FP64 instructions, costs as much as the vector work when
+// every warp issues it for one pair), each warp rotates its columns.  HELD
+// (s <= 32 JS_E): the columns stay in registers between the two, and those of V are
+// loaded before the rotation is known.  Bound: the FP64 pipes (16 matrices of
+// s = 128: 46 -> 36 ms; FP64 pipe 57 % active).
+constexpr int JS_CL = 8, JS_E = 4;
 
 __device__ __forceinline__ double norm2d(double2 a) { return a.x * a.x + a.y * a.y; }
 
+template <bool HELD>
 __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
     k_jacobi_svd(int s, z64 *__restrict__ Xall, z64 *__restrict__ Vall, double *__restrict__ sig,
                  int *__restrict__ info, double tol, double keep) {
@@ -601,6 +680,8 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
     __shared__ uint64_t cbar[2];
     __shared__ int s_abort, rot_local, rotflag[JS_CL];
     __shared__ double s_wmax[32], s_big;
+    __shared__ double s_dot[8][4], s_rot[8][5];   // per warp: |x_i|^2, |x_j|^2, x_i^H x_j; c, sem, sep
+    __shared__ int s_do[8];
     for (int64_t i = (int64_t)me * blockDim.x + threadIdx.x; i < (int64_t)s * s; i += (int64_t)JS_CL * blockDim.x)
         V[i] = z64((i % s) == (i / s) ? 1.0 : 0.0, 0.0);
     if (threadIdx.x == 0) {
@@ -642,49 +723,110 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
         __syncthreads();
         const double floor_abs = fmax(tol * tol, 1e-10 * keep * keep) * s_big;
         for (int round = 0; round < n2 - 1 && ok; ++round) {
-            for (int pr = gw; pr < n2 / 2; pr += ngw) {
+            for (int p0 = me * nw; p0 < n2 / 2; p0 += ngw) {
+                const int pr = p0 + warp;
                 // round-robin: position 0 fixed, others rotate
-                int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (n2 - 1);
-                int b = 1 + (n2 - 2 - pr + round) % (n2 - 1);
-                int i = min(a, b), j = max(a, b);
-                if (j >= s) continue;   // dummy column of odd sizes
+                const int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (n2 - 1);
+                const int b = 1 + (n2 - 2 - pr + round) % (n2 - 1);
+                const int i = min(a, b), j = max(a, b);
+                const bool pair = pr < n2 / 2 && j < s;   // j == s: dummy column of odd sizes
                 z64 *xi = X + (int64_t)i * s, *xj = X + (int64_t)j * s;
+                z64 *vi = V + (int64_t)i * s, *vj = V + (int64_t)j * s;
+                z64 xu[JS_E], xv[JS_E], wu[JS_E], wv[JS_E];
                 double al = 0, be = 0;
                 z64 ga(0, 0);
-                for (int r = lane; r < s; r += 32) {
-                    const double2 u2 = __ldcg(reinterpret_cast<const double2 *>(xi) + r);
-                    const double2 v2 = __ldcg(reinterpret_cast<const double2 *>(xj) + r);
-                    const z64 u(u2.x, u2.y), v(v2.x, v2.y);
-                    al += norm2(u);
-                    be += norm2(v);
-                    cfmaconj(ga, u, v);
+                auto add = [&](z64 u, z64 v) {
+                    al = __dadd_rn(al, norm2_rn(u));
+                    be = __dadd_rn(be, norm2_rn(v));
+                    ga.re = __fma_rn(u.im, v.im, __fma_rn(u.re, v.re, ga.re));
+                    ga.im = __fma_rn(-u.im, v.re, __fma_rn(u.re, v.im, ga.im));
+                };
+                if (pair) {
+                    if constexpr (HELD) {
+#pragma unroll
+                        for (int e = 0; e < JS_E; ++e) {
+                            const int r = lane + 32 * e;
+                            if (r < s) {
+                                xu[e] = ldcg64(xi + r);
+                                xv[e] = ldcg64(xj + r);
+                            }
+                        }
+#pragma unroll
+                        for (int e = 0; e < JS_E; ++e) {
+                            const int r = lane + 32 * e;
+                            if (r < s) {
+                                wu[e] = ldcg64(vi + r);
+                                wv[e] = ldcg64(vj + r);
+                            }
+                        }
+#pragma unroll
+                        for (int e = 0; e < JS_E; ++e) {
+                            if (lane + 32 * e < s) add(xu[e], xv[e]);
+                        }
+                    } else {
+                        for (int r = lane; r < s; r += 32) add(ldcg64(xi + r), ldcg64(xj + r));
+                    }
+                    for (int o = 16; o > 0; o >>= 1) {
+                        al += __shfl_xor_sync(0xffffffffu, al, o);
+                        be += __shfl_xor_sync(0xffffffffu, be, o);
+                        ga.re += __shfl_xor_sync(0xffffffffu, ga.re, o);
+                        ga.im += __shfl_xor_sync(0xffffffffu, ga.im, o);
+                    }
                 }
-                for (int o = 16; o > 0; o >>= 1) {
-                    al += __shfl_xor_sync(0xffffffffu, al, o);
-                    be += __shfl_xor_sync(0xffffffffu, be, o);
-                    ga.re += __shfl_xor_sync(0xffffffffu, ga.re, o);
-                    ga.im += __shfl_xor_sync(0xffffffffu, ga.im, o);
+                if (lane == 0) {
+                    s_dot[warp][0] = al;
+                    s_dot[warp][1] = be;
+                    s_dot[warp][2] = ga.re;
+                    s_dot[warp][3] = ga.im;
                 }
-                double ag = sqrt(norm2(ga));
-                if (ag <= tol * sqrt(al * be) || ag <= floor_abs || ag == 0.0) continue;
-                if (lane == 0) rot_local = 1;
-                double zeta = (be - al) / (2.0 * ag);
-                double t = 1.0 / (zeta + copysign(sqrt(1.0 + zeta * zeta), zeta));
-                double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
-                z64 e(ga.re / ag, ga.im / ag);   // e^{i phi}
-                z64 sem = sn * conj(e), sep = sn * e;
-                z64 *vi = V + (int64_t)i * s, *vj = V + (int64_t)j * s;
-                for (int r = lane; r < s; r += 32) {
-                    const double2 u2 = __ldcg(reinterpret_cast<const double2 *>(xi) + r);
-                    const double2 v2 = __ldcg(reinterpret_cast<const double2 *>(xj) + r);
-                    const z64 u(u2.x, u2.y), v(v2.x, v2.y);
-                    xi[r] = c * u - sem * v;
-                    xj[r] = sep * u + c * v;
-                    const double2 p2 = __ldcg(reinterpret_cast<const double2 *>(vi) + r);
-                    const double2 q2 = __ldcg(reinterpret_cast<const double2 *>(vj) + r);
-                    const z64 vu(p2.x, p2.y), vv(q2.x, q2.y);
-                    vi[r] = c * vu - sem * vv;
-                    vj[r] = sep * vu + c * vv;
+                __syncthreads();
+                if (warp == 0) {
+                    // lane 8 q + w: pair w of the CTA; the independent roots and quotients of a pair on its lanes q
+                    const int w = lane & 7, q = lane >> 3;
+                    const double pal = s_dot[w][0], pbe = s_dot[w][1];
+                    const z64 pga(s_dot[w][2], s_dot[w][3]);
+                    const double root = sqrt(q == 1 ? pal * pbe : norm2(pga));
+                    const double ag = __shfl_sync(0xffffffffu, root, w), sab = __shfl_sync(0xffffffffu, root, w + 8);
+                    const bool rot = !(ag <= tol * sab || ag <= floor_abs || ag == 0.0);
+                    const double quo = (q == 0 ? pbe - pal : q == 1 ? pga.re : pga.im) / (q == 0 ? 2.0 * ag : ag);
+                    const double zeta = __shfl_sync(0xffffffffu, quo, w);
+                    const z64 e(__shfl_sync(0xffffffffu, quo, w + 8), __shfl_sync(0xffffffffu, quo, w + 16));   // e^{i phi}
+                    const double t = 1.0 / (zeta + copysign(sqrt(1.0 + zeta * zeta), zeta));
+                    const double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
+                    const z64 sem = sn * conj(e), sep = sn * e;
+                    if (q == 0) {
+                        s_do[w] = rot;
+                        s_rot[w][0] = c;
+                        s_rot[w][1] = sem.re;
+                        s_rot[w][2] = sem.im;
+                        s_rot[w][3] = sep.re;
+                        s_rot[w][4] = sep.im;
+                        if (rot) rot_local = 1;
+                    }
+                }
+                __syncthreads();
+                if (!pair || !s_do[warp]) continue;
+                const double c = s_rot[warp][0];
+                const z64 sem(s_rot[warp][1], s_rot[warp][2]), sep(s_rot[warp][3], s_rot[warp][4]);
+                auto turn = [&](z64 u, z64 v, z64 *pu, z64 *pv) {   // c u - sem v, sep u + c v
+                    const z64 a_ = mul2_rn(sem, v), b_ = mul2_rn(sep, u);
+                    *pu = z64(__fma_rn(c, u.re, -a_.re), __fma_rn(c, u.im, -a_.im));
+                    *pv = z64(__fma_rn(c, v.re, b_.re), __fma_rn(c, v.im, b_.im));
+                };
+                if constexpr (HELD) {
+#pragma unroll
+                    for (int e = 0; e < JS_E; ++e) {
+                        const int r = lane + 32 * e;
+                        if (r < s) {
+                            turn(xu[e], xv[e], xi + r, xj + r);
+                            turn(wu[e], wv[e], vi + r, vj + r);
+                        }
+                    }
+                } else {
+                    for (int r = lane; r < s; r += 32) {
+                        turn(ldcg64(xi + r), ldcg64(xj + r), xi + r, xj + r);
+                        turn(ldcg64(vi + r), ldcg64(vj + r), vi + r, vj + r);
+                    }
                 }
             }
             ok = cl_sync(cbar, step++, JS_CL, &s_abort, info + mat);
@@ -1632,9 +1774,19 @@ void lu_solve_batched(int nb, const int64_t *h_zoff, const int64_t *h_voff, cons
     CBFM_CUDA(cudaMemcpyAsync(zo.p, h_zoff, nb * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     CBFM_CUDA(cudaMemcpyAsync(vo.p, h_voff, nb * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     CBFM_CUDA(cudaMemcpyAsync(nn.p, h_n, nb * sizeof(int), cudaMemcpyHostToDevice, st));
+    int nmax = 1;
+    for (int k = 0; k < nb; ++k) nmax = std::max(nmax, h_n[k]);
+    size_t smem = sizeof(z64) * 2 * (size_t)nmax;
+    DevBuf<z64> scratch;
+    if (smem > 160 * 1024) {
+        scratch.alloc((size_t)nb * LU_CL * 2 * nmax);
+        smem = 0;
+    } else {
+        CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    }
     {
         ProfScope ps_("k_lu_solve", st);
-        k_lu_solve<<<nb, 256, 0, st>>>(zo.p, vo.p, nn.p, s, Z, V, d_info);
+        k_lu_solve<<<nb * LU_CL, 256, smem, st>>>(zo.p, vo.p, nn.p, s, Z, V, d_info, scratch.p, nmax);
         launched("k_lu_solve");
     }
     CBFM_CUDA(cudaStreamSynchronize(st));
@@ -1644,7 +1796,9 @@ void jacobi_svd_batched(int nb, int s, z64 *X, z64 *V, double *sig, int *d_info,
     // rotation threshold: a few units of round-off in the column dot products
     {
         ProfScope ps_("k_jacobi_svd", st);
-        k_jacobi_svd<<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, 1e-15 * (s > 8 ? s : 8), keep);
+        const double tol = 1e-15 * (s > 8 ? s : 8);
+        if (s <= 32 * JS_E) k_jacobi_svd<true><<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, tol, keep);
+        else k_jacobi_svd<false><<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, tol, keep);
         launched("k_jacobi_svd");
     }
 }
