@@ -654,7 +654,9 @@ cbfm_status cbfm_mesh(const double *verts, int64_t nv, const int32_t *tris, int6
         m->tri32.alloc((size_t)h.nt * TRI_REC);
         m->far64.alloc((size_t)h.nt * FB_REC);
         m->far32.alloc((size_t)h.nt * FB_REC);
+        m->geo.alloc((size_t)h.nt * GEO_REC);
         launch_tri_records(*m, dv.p, dt.p, st);
+        launch_tri_geo(*m, st);
         launch_near_pairs(*m, st);
         launch_gram_rows(*m, st);
         CBFM_CUDA(cudaStreamSynchronize(st));

@@ -122,6 +122,7 @@ constexpr double K0 = 2.0 * PI;          // lengths in free-space wavelengths
 //   [44,47) FP32 copy only: low parts of the centroid (centroid = hi + lo)
 //   [47]    padding
 constexpr int TRI_REC = 48;
+constexpr int GEO_REC = 25;  // doubles of a triangle's TriGeo (k_assembly.cu)
 constexpr int FB_REC = 20;   // record of the barycentric far quadrature (far_bary.cuh)
 constexpr int TR_Q = 0, TR_W = 21, TR_P = 28, TR_C = 37, TR_CEN = 40, TR_H = 43, TR_CLO = 44;
 

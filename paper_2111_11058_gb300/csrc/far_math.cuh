@@ -27,14 +27,16 @@ struct Media {
     double e1r, e1i, e2r, e2i;   // eta1, eta2
     double f1r, f1i, f2r, f2i;   // 4 / k1^2, 4 / k2^2
     double i1r, i1i, i2r, i2i;   // 1 / eta1, 1 / eta2
+    double kk1r, kk1i, kk2r, kk2i;   // k1^2, k2^2
 };
 
 // the derived constants of a Media from k1, k2, eta1, eta2 (host)
 inline Media media_full(z64 k1, z64 k2, z64 e1, z64 e2) {
+    const z64 q1 = k1 * k1, q2 = k2 * k2;
     const z64 f1 = cdiv(z64(4.0, 0.0), k1 * k1), f2 = cdiv(z64(4.0, 0.0), k2 * k2);
     const z64 i1 = cdiv(z64(1.0, 0.0), e1), i2 = cdiv(z64(1.0, 0.0), e2);
     return Media{k1.re, k1.im, k2.re, k2.im, e1.re, e1.im, e2.re, e2.im,
-                 f1.re, f1.im, f2.re, f2.im, i1.re, i1.im, i2.re, i2.im};
+                 f1.re, f1.im, f2.re, f2.im, i1.re, i1.im, i2.re, i2.im, q1.re, q1.im, q2.re, q2.im};
 }
 
 // Per-medium constants in the arithmetic type of the far-pair kernel,

@@ -45,6 +45,7 @@ struct Mesh : HandleBase {
     DevBuf<float> tri32;         // nt * TRI_REC (centred coordinates)
     DevBuf<double> far64;        // nt * FB_REC (far_bary.cuh)
     DevBuf<float> far32;
+    DevBuf<double> geo;          // nt * GEO_REC (unit vectors of the near pairs' closed forms)
     DevBuf<int32_t> tri_vid;     // nt*3 vertex ids
     DevBuf<int32_t> tri_edge;    // nt*3 internal edge id
     DevBuf<int32_t> tri_cell;    // nt*3 cell of each of the triangle's RWGs
@@ -109,6 +110,7 @@ struct Red : HandleBase {
 
 // ------------------------------------------------------------- kernels
 // geometry (k_geom.cu)
+void launch_tri_geo(Mesh &m, cudaStream_t st);   // k_assembly.cu
 void launch_tri_records(Mesh &m, const double *d_verts, const int32_t *d_tris, cudaStream_t st);
 void launch_near_pairs(Mesh &m, cudaStream_t st);
 void launch_gram_rows(Mesh &m, cudaStream_t st);

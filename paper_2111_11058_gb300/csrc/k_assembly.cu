@@ -196,8 +196,8 @@ __device__ void potentials(const double *V, const double *r, double &I1, double 
 
 // The same closed forms with fewer FP64 operations (~260 a test point instead of
 // ~700), for the near pairs of the reduced systems:
-//   * the trial triangle's unit vectors and lengths (TriGeo), the same for its
-//     seven test points, come from three lanes per triangle through shared memory;
+//   * the trial triangle's unit vectors and lengths (TriGeo) are formed once per
+//     mesh and come through shared memory;
 //   * the sum of the edges' arctangents is the solid angle of the triangle, one
 //     arctangent instead of three (A. van Oosterom, J. Strackee, "The solid angle of
 //     a plane triangle", IEEE Trans. Biomed. Eng. 30, 1983): tan(Omega / 2) = |h| 2A / (R0 R1 R2 +
@@ -228,6 +228,11 @@ __device__ __forceinline__ void tri_geo(const double *V, int i, TriGeo &g) {   /
         for (int d = 0; d < 3; ++d) g.n[d] = n[d];
         g.nl = nl2 * inl;
     }
+}
+static_assert(sizeof(TriGeo) == GEO_REC * sizeof(double), "TriGeo record");
+__global__ void k_tri_geo(int64_t nt, const double *__restrict__ rec, double *__restrict__ geo) {
+    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, t = x / 3;
+    if (t < nt) tri_geo(rec + t * TRI_REC + TR_P, (int)(x - 3 * t), reinterpret_cast<TriGeo *>(geo)[t]);
 }
 __device__ __forceinline__ void potentials_lean(const double *V, const TriGeo &g, const double *r, double &I1,
                                                 double Iv[3], double I3[3]) {
@@ -284,11 +289,13 @@ __device__ __forceinline__ void potentials_lean(const double *V, const TriGeo &g
 //   gr = -jk/(4 pi)      sum_{j>=0} (-y)^j / (j+1)!
 //   hr = -(jk)^3/(4 pi)  sum_{j>=0} (-1)^j (j+2)/(j+3)! y^j
 // where 12 terms leave < 1e-19 relative.
+// LEAN: the reciprocal iR of R (any value at R = 0) comes with it, from one
+// reciprocal square root for both media.
 template <bool LEAN>
-__device__ inline void green_rems(z64 k, double R, z64 &gr, z64 &hr) {
+__device__ inline void green_rems(z64 k, double R, double iR, z64 &gr, z64 &hr) {
     const z64 jk(-k.im, k.re);
     const z64 y = jk * R;
-    if (sqrt(norm2(y)) < 0.2) {
+    if (LEAN ? norm2(y) < 0.2 * 0.2 : sqrt(norm2(y)) < 0.2) {
         z64 pw(1, 0), s1(0, 0), s2(0, 0);
         double f1 = 1.0, f3 = 6.0;   // (j+1)!, (j+3)!
         for (int j = 0; j < 12; ++j) {
@@ -305,10 +312,9 @@ __device__ inline void green_rems(z64 k, double R, z64 &gr, z64 &hr) {
         hr = (jk * jk * jk) * s2 * (-1.0 / (4.0 * PI));
         return;
     }
-    double sn, cs, iR;
+    double sn, cs;
     if constexpr (LEAN) {
         f64::sincos64(k.re * R, &sn, &cs);
-        iR = f64::rcp64(R);
     } else {
         sincos(k.re * R, &sn, &cs);
         iR = 1.0 / R;
@@ -396,6 +402,8 @@ constexpr double near_fp64_ops() {
 
 template <typename T, bool LEAN>
 __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *__restrict__ rec, const Media &md,
+                                           const MediaT<T> &mdt, const T *__restrict__ recT,
+                                           const T *__restrict__ frec, const double *__restrict__ tgeo,
                                            cx<T> *__restrict__ Zloc, cx<T> (*sm)[2][2][NEAR_MOM], TriGeo *geo,
                                            cx<T> *__restrict__ blk) {
     // (t, s): the pair of this lane's slot (t < 0: none); every lane reads only
@@ -404,7 +412,9 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
     const int slot = lane >> 4, o = (lane >> 3) & 1, p = lane & 7;
     __syncwarp();   // the slot's previous readers are done
     if constexpr (LEAN) {
-        if (p < 3 && t >= 0) tri_geo(rec + (int64_t)(o == 0 ? s : t) * TRI_REC + TR_P, p, geo[lane >> 3]);
+        if (t >= 0)
+            for (int i = p; i < GEO_REC; i += 8)
+                reinterpret_cast<double *>(geo + (lane >> 3))[i] = tgeo[(int64_t)(o == 0 ? s : t) * GEO_REC + i];
         __syncwarp();
     }
     // the test-point moments and the entries are the outer quadrature of the
@@ -421,35 +431,54 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
         double I1, Iv[3], I3[3];
         if constexpr (LEAN) potentials_lean(B + TR_P, geo[lane >> 3], r, I1, Iv, I3);
         else potentials(B + TR_P, r, I1, Iv, I3);
-        const T wp = (T)A[TR_W + p];
+        // LEAN: the potentials over 4 pi by one product each (a quotient is some 15 FP64 instructions)
+        if constexpr (LEAN) {
+            constexpr double C4 = 1.0 / (4.0 * PI);
+            I1 *= C4;
+            for (int d = 0; d < 3; ++d) {
+                Iv[d] *= C4;
+                I3[d] *= C4;
+            }
+        }
+        // LEAN: FP32 weights and media constants as stored, P from the far record (the same values; conversions
+        // take the FP64 pipe)
+        const T *wB = recT + (int64_t)(o == 0 ? s : t) * TRI_REC + TR_W;
+        const T wp = LEAN ? recT[(int64_t)(o == 0 ? t : s) * TRI_REC + TR_W + p] : (T)A[TR_W + p];
         const T rr[3] = {(T)(r[0] - A[TR_CEN]), (T)(r[1] - A[TR_CEN + 1]), (T)(r[2] - A[TR_CEN + 2])};
         const T r2 = rr[0] * rr[0] + rr[1] * rr[1] + rr[2] * rr[2];
         // trial points: d = r - r', R, weights; shared by the two media.  On the
         // mixed path the smooth remainders, their 7-point sums and the moments
         // are FP32 and only the closed forms FP64.
-        T dq[7][3], Rq[7], wq[7];
+        T dq[7][3], Rq[7], iRq[7], wq[7];
 #pragma unroll
         for (int q = 0; q < 7; ++q) {
             double dv[3];
             sub3(r, B + TR_Q + 3 * q, dv);
             for (int d = 0; d < 3; ++d) dq[q][d] = (T)dv[d];
             if constexpr (sizeof(T) == 4) Rq[q] = sqrtf(dq[q][0] * dq[q][0] + dq[q][1] * dq[q][1] + dq[q][2] * dq[q][2]);
-            else Rq[q] = sqrt(dot3(dv, dv));
-            wq[q] = (T)B[TR_W + q];
+            else if constexpr (LEAN) {
+                const double R2 = dot3(dv, dv);
+                iRq[q] = R2 > 0.0 ? f64::rsqrt64(R2) : 0.0;
+                Rq[q] = R2 * iRq[q];
+            } else {
+                Rq[q] = sqrt(dot3(dv, dv));
+            }
+            wq[q] = LEAN ? wB[q] : (T)B[TR_W + q];
         }
 #pragma unroll
         for (int med = 0; med < 2; ++med) {
             const z64 k = med == 0 ? z64(md.k1r, md.k1i) : z64(md.k2r, md.k2i);
-            const z64 kk = k * k;
+            const z64 kk = LEAN ? (med == 0 ? z64(md.kk1r, md.kk1i) : z64(md.kk2r, md.kk2i)) : k * k;
             cx<T> g0(0, 0), gr[3], hw[3];   // sum w g, sum w g (-d), sum w h d over the trial points
             for (int d = 0; d < 3; ++d) gr[d] = hw[d] = cx<T>(0, 0);
 #pragma unroll
             for (int q = 0; q < 7; ++q) {
                 cx<T> gs, hs;
                 if constexpr (sizeof(T) == 4) {
-                    green_rems_f((float)k.re, (float)k.im, Rq[q], gs, hs);
+                    if constexpr (LEAN) green_rems_f(mdt.kr[med], mdt.ki[med], Rq[q], gs, hs);
+                    else green_rems_f((float)k.re, (float)k.im, Rq[q], gs, hs);
                 } else {
-                    green_rems<LEAN>(k, Rq[q], gs, hs);
+                    green_rems<LEAN>(k, Rq[q], iRq[q], gs, hs);
                 }
                 gs = gs * wq[q];
                 hs = hs * wq[q];
@@ -459,12 +488,12 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
                     hw[d] += hs * dq[q][d];
                 }
             }
-            const cx<T> S0((T)(I1 / (4.0 * PI)) + g0.re, g0.im);
+            const cx<T> S0((T)(LEAN ? I1 : I1 / (4.0 * PI)) + g0.re, g0.im);
             cx<T> Sr[3], Wv[3];
             for (int d = 0; d < 3; ++d) {
-                Sr[d] = cx<T>((T)(Iv[d] / (4.0 * PI)) + gr[d].re, gr[d].im);
-                const z64 kI = kk * (Iv[d] / (8.0 * PI));
-                Wv[d] = cx<T>((T)(kI.re - I3[d] / (4.0 * PI)), (T)kI.im) + hw[d];
+                Sr[d] = cx<T>((T)(LEAN ? Iv[d] : Iv[d] / (4.0 * PI)) + gr[d].re, gr[d].im);
+                const z64 kI = kk * (LEAN ? 0.5 * Iv[d] : Iv[d] / (8.0 * PI));
+                Wv[d] = cx<T>((T)(kI.re - (LEAN ? I3[d] : I3[d] / (4.0 * PI))), (T)kI.im) + hw[d];
             }
             cx<T> *m = mom[med];
             const cx<T> wS0 = wp * S0;
@@ -508,7 +537,8 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
         const int ia = oo == 0 ? a : b, ib = oo == 0 ? b : a;   // test vertex, trial vertex
         T P[3], Q[3];
         for (int d = 0; d < 3; ++d) {
-            P[d] = (T)(A[TR_P + 3 * ia + d] - A[TR_CEN + d]);
+            P[d] = LEAN ? frec[(int64_t)(oo == 0 ? t : s) * FB_REC + FB_P + 3 * ia + d]
+                        : (T)(A[TR_P + 3 * ia + d] - A[TR_CEN + d]);
             Q[d] = (T)(B[TR_P + 3 * ib + d] - A[TR_CEN + d]);
         }
         const T cc = (T)(0.5 * A[TR_C + ia] * B[TR_C + ib]);
@@ -520,14 +550,22 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
 #pragma unroll
         for (int med = 0; med < 2; ++med) {
             const cx<T> *m = sm[slot][oo][med];
-            const cx<T> k = med == 0 ? cx<T>((T)md.k1r, (T)md.k1i) : cx<T>((T)md.k2r, (T)md.k2i);
-            const cx<T> eta = med == 0 ? cx<T>((T)md.e1r, (T)md.e1i) : cx<T>((T)md.e2r, (T)md.e2i);
-            const cx<T> f4k2 = med == 0 ? cx<T>((T)md.f1r, (T)md.f1i) : cx<T>((T)md.f2r, (T)md.f2i);   // 4 / k^2
-            const cx<T> ieta = med == 0 ? cx<T>((T)md.i1r, (T)md.i1i) : cx<T>((T)md.i2r, (T)md.i2i);   // 1 / eta
+            cx<T> k, meta, f4k2, ieta;   // k, -eta, 4 / k^2, 1 / eta
+            if constexpr (LEAN) {
+                k = cx<T>(mdt.kr[med], mdt.ki[med]);
+                meta = cx<T>(mdt.wTar[med], mdt.wTai[med]);
+                f4k2 = cx<T>(mdt.fk2r[med], mdt.fk2i[med]);
+                ieta = cx<T>(mdt.wTbr[med], mdt.wTbi[med]);
+            } else {
+                k = med == 0 ? cx<T>((T)md.k1r, (T)md.k1i) : cx<T>((T)md.k2r, (T)md.k2i);
+                meta = -(med == 0 ? cx<T>((T)md.e1r, (T)md.e1i) : cx<T>((T)md.e2r, (T)md.e2i));
+                f4k2 = med == 0 ? cx<T>((T)md.f1r, (T)md.f1i) : cx<T>((T)md.f2r, (T)md.f2i);
+                ieta = med == 0 ? cx<T>((T)md.i1r, (T)md.i1i) : cx<T>((T)md.i2r, (T)md.i2i);
+            }
             cx<T> br = m[8] + m[4] - (P[0] * m[5] + P[1] * m[6] + P[2] * m[7]) -
                        (PpQ[0] * m[1] + PpQ[1] * m[2] + PpQ[2] * m[3]) + PQ * m[0] - f4k2 * m[0];
             const cx<T> Tv = cc * (cx<T>(k.im, -k.re) * br);
-            ta += -eta * Tv;
+            ta += meta * Tv;
             tb += Tv * ieta;
             if (t != s)
                 ks += cc * (QmP[0] * m[12] + QmP[1] * m[13] + QmP[2] * m[14] + QxP[0] * m[9] + QxP[1] * m[10] +
@@ -552,7 +590,7 @@ __device__ __forceinline__ void near_pair2(int t, int s, int nt, const double *_
 template <typename T>
 struct AsmJob {
     const T *rec, *frec;
-    const double *rec64;
+    const double *rec64, *geo;
     const int32_t *vid, *pairs, *edge_tri, *edge_loc;
     const int32_t *tri_cell;   // non-null: evaluate only pairs of triangles that share a cell
     cx<T> *Zloc, *Z;
@@ -618,7 +656,7 @@ __device__ __forceinline__ void near_loop(const AsmJob<T> *__restrict__ jobs, in
             if (J->tri_cell && !share_cell(J->tri_cell, t, s)) t = s = -1;   // stays zero (written by the far stage)
         }
         cx<T> *blk = (J->nearblk && t >= 0) ? J->nearblk + (pid - J->near0) * NCOMP : nullptr;
-        near_pair2<T, LEAN>(t, s, J->nt, J->rec64, J->md, J->Zloc, sh.mom, sh.geo, blk);
+        near_pair2<T, LEAN>(t, s, J->nt, J->rec64, J->md, J->mdt, J->rec, J->frec, J->geo, J->Zloc, sh.mom, sh.geo, blk);
     }
 }
 template <typename T, bool LEAN>
@@ -865,6 +903,13 @@ __global__ void k_gather(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t 
 
 }  // namespace
 
+void launch_tri_geo(Mesh &m, cudaStream_t st) {
+    const int64_t nt = m.h.nt;
+    if (nt <= 0) return;
+    k_tri_geo<<<(unsigned)((3 * nt + 127) / 128), 128, 0, st>>>(nt, m.tri64.p, m.geo.p);
+    launched("k_tri_geo");
+}
+
 template <typename T>
 static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
                            cudaStream_t st, bool lean, bool diag_cells);
@@ -914,6 +959,7 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p, J.frec = (const T *)m.far64.p;
         else J.rec = (const T *)m.tri32.p, J.frec = (const T *)m.far32.p;
         J.rec64 = m.tri64.p;
+        J.geo = m.geo.p;
         J.vid = m.tri_vid.p;
         J.pairs = m.near_pairs.p;
         J.edge_tri = m.edge_tri.p;
@@ -1051,6 +1097,7 @@ void near_blocks_compact_t(const std::vector<Mesh *> &ms, const std::vector<cx<T
         if constexpr (sizeof(T) == 8) J.rec = (const T *)m.tri64.p, J.frec = (const T *)m.far64.p;
         else J.rec = (const T *)m.tri32.p, J.frec = (const T *)m.far32.p;
         J.rec64 = m.tri64.p;
+        J.geo = m.geo.p;
         J.vid = m.tri_vid.p;
         J.pairs = m.near_pairs.p;
         J.nearblk = out[k];
