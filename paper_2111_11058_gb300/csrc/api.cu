@@ -907,7 +907,7 @@ void project(Red &r, cudaStream_t st) {
             return;
         }
     }
-    const bool lean = sizeof(T) == 8 || c.spread <= SPREAD_MAX;
+    const bool lean = sizeof(T) == 8 || c.spread <= SPREAD_ASM;
     if constexpr (sizeof(T) == 4) {
         if (r.prec == CBFM_MIXED || r.prec == CBFM_MIXED_UNFUSED || r.prec == CBFM_MIXED_FUSED) {
             DevBuf<float> Zs;
@@ -1285,12 +1285,12 @@ cbfm_status cbfm_assemble_reduced_batch(const cbfm_mesh_t *meshes, const cbfm_cb
                 Zs[i - i0].alloc(tc_planes(ms[k]->h.ne));
                 Ap.push_back(r->A32.p);
             }
-            // one launch per stage for the scatterers of either form of the near pairs' closed forms
+            // one launch per stage for the scatterers of either form of the entries
             for (int lean = 0; lean < 2; ++lean) {
                 std::vector<Mesh *> lm;
                 std::vector<float *> lz;
                 for (size_t k = 0; k < wm.size(); ++k)
-                    if ((wc[k]->spread <= SPREAD_MAX) == (lean == 1)) {
+                    if ((wc[k]->spread <= SPREAD_ASM) == (lean == 1)) {
                         lm.push_back(wm[k]);
                         lz.push_back(Zs[k].p);
                     }

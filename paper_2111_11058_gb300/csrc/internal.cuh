@@ -79,6 +79,12 @@ struct Cbf : HandleBase {
 // edges (1.5e-6 and 6e-5 where the spread is below 5e3): those systems keep one order of operations, so that
 // their results stay reproducible.
 constexpr double SPREAD_MAX = 1e4;
+// The same for the assembly's shorter forms (near pairs' closed forms, barycentric far pairs): their entries
+// round differently (1.4e-7 of the matrix).  CBFs kept to sigma / sigma_1 >= 1e-3 spread over 1e3, and
+// currents on coarse meshes carry such a difference up to 300 times (69 solves drawn from spheres, cubes,
+// cylinders and spheroids: 4.4e-5 of the currents' norm with these forms everywhere, 2.3e-5 with the near
+// pairs' alone, 4.5e-6 where only spreads below this line take them).
+constexpr double SPREAD_ASM = 300.0;
 
 struct Red : HandleBase {
     Mesh *mesh;

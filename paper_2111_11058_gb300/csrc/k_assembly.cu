@@ -997,7 +997,7 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
 // short elementary functions (near pairs of the 9216-unknown cube 1.73 -> 1.15 ms
 // by themselves) and the far pairs in barycentric moments (far_bary.cuh); the conventional MoM, whose
 // long restarted solves carry a last bit of Z into the currents, and mixed
-// systems beyond SPREAD_MAX keep the general ones.
+// systems beyond SPREAD_ASM keep the general ones.
 template <typename T>
 static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
                            cudaStream_t st, bool lean, bool diag_cells) {

@@ -947,9 +947,7 @@ void assemble_project_fused(const std::vector<Mesh *> &ms, const std::vector<Cbf
         nearv[k].alloc((size_t)std::max<int64_t>(1, ms[k]->n_near) * NCOMP);
         nearp[k] = nearv[k].p;
     }
-    bool lean = true;   // the shorter closed forms, unless one of the systems keeps its bits
-    for (const Cbf *c : cs) lean &= c->spread <= SPREAD_MAX;
-    near_blocks_compact(ms, nearp, st, lean);
+    near_blocks_compact(ms, nearp, st, true);
     std::vector<FusedJob> jobs(nj);
     std::vector<std::pair<double, int4>> items;
     std::vector<DevBuf<int32_t>> dL(nj), dcoff32(nj);
