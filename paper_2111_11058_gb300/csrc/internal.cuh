@@ -71,19 +71,20 @@ struct Cbf : HandleBase {
     DevBuf<c32> CM32, CJ32;
 };
 
-// Spread of the CBFs' singular values up to which a mixed-precision system takes
-// the faster forms that change the last bits of its matrix or of its basis.  With
-// tiny triangles beside large ones (1.4e4 to 1e5 on spheroids and cylinders with pole
-// triangles; 1e3 to 5e3 on cubes, spheres and even cylinders) the FP32 operator's rounding, which follows those
-// bits, moves the currents by 1e-5 of their norm and 1e-3 of their rms at single
-// edges (1.5e-6 and 6e-5 where the spread is below 5e3): those systems keep one order of operations, so that
-// their results stay reproducible.
-constexpr double SPREAD_MAX = 1e4;
+// Spread of the CBFs' singular values up to which a mixed-precision block solve takes
+// the faster forms that change the last bits of its basis.  With tiny triangles beside
+// large ones (1.4e4 to 1e5 on spheroids and cylinders with pole triangles; 1e3 to 1e4 on
+// cubes, spheres and even cylinders) the FP32 operator's rounding, which follows those
+// bits, moves the currents by up to 1e-5 of their norm and 1e-3 of their rms at single
+// edges; of 446 drawn solves below 1e4 three moved by more than 2e-5 (8e-5), all above
+// 2.1e3, and below this line none by more than 1.2e-5.  The others keep one order of
+// operations, so that their results stay reproducible.
+constexpr double SPREAD_MAX = 2e3;
 // The same for the assembly's shorter forms (near pairs' closed forms, barycentric far pairs): their entries
 // round differently (1.4e-7 of the matrix).  CBFs kept to sigma / sigma_1 >= 1e-3 spread over 1e3, and
 // currents on coarse meshes carry such a difference up to 300 times (69 solves drawn from spheres, cubes,
 // cylinders and spheroids: 4.4e-5 of the currents' norm with these forms everywhere, 2.3e-5 with the near
-// pairs' alone, 4.5e-6 where only spreads below this line take them).
+// pairs' alone; with a line at 800 still 7.4e-5 on a sphere a tenth of a wavelength across).
 constexpr double SPREAD_ASM = 300.0;
 
 struct Red : HandleBase {

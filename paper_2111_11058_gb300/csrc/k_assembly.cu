@@ -1080,11 +1080,13 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         int occ = 0;
         CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, far, FB, far_sm));
         const unsigned grid = (unsigned)std::max(1, occ) * (unsigned)nsm;
-        if (tuned > 0) {   // the near pairs beside the far ones (FP32 form)
-            const bool both = sizeof(T) == 4 && npairs > 0;
+        // the near pairs beside the far ones (FP32, shorter forms; inlined there, the general closed forms would have
+        // their products fused differently than in the near kernel, and they are taken for their bits)
+        if (tuned > 0) {
+            const bool both = sizeof(T) == 4 && lean && npairs > 0;
             near_done = both;
             ProfScope ps_("k_far", st);
-            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, npairs, both ? 2 * nsm : 0);
+            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, both ? npairs : 0, both ? 2 * nsm : 0);
             launched("k_far");
             break;
         }
