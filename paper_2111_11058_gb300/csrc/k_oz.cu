@@ -592,10 +592,12 @@ void launch_pack(const OzPack *p, int np, int64_t K, cudaStream_t st) {
     launched("k_oz_pack");
 }
 void launch_gemm(OzArgs g, int64_t mt, cudaStream_t st) {
-    // CTAs per tile: the K stages are shared while the tiles leave SMs idle, down to one drain's worth of stages
+    // CTAs per tile: the K stages are shared while the tiles leave SMs idle, down to half a drain's worth of stages
+    // (block solve of the 9216-unknown cube: 120 products 3.45 -> 3.20 ms against a whole one, 3.13 ms with clusters of
+    // 16, which cost the 2304-unknown cube's more than they give; the sums are integers, so the split has no say in them)
     const int64_t tiles = mt * g.tn;
     int cs = 1;
-    while (cs < 8 && tiles * cs * 2 <= sm_count() && g.nkb >= 2 * OZ_CHUNK * cs) cs *= 2;
+    while (cs < 8 && tiles * cs * 2 <= sm_count() && g.nkb >= OZ_CHUNK * cs) cs *= 2;
     g.cs = cs;
     set_smem_once(k_oz_gemm, OZ_SMEM);
     cudaLaunchConfig_t cfg = {};
