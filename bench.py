@@ -118,7 +118,10 @@ DEV = {"n_sm": 152, "sm_max_mhz": 2070.0}
 def fp32_peak_tflops() -> float:
     return DEV["n_sm"] * FP32_LANES_PER_SM * 2 * DEV["sm_max_mhz"] * 1e6 / 1e12
 FP64_KERNELS = {"k_dots", "k_orth_update", "k_near_blocks", "k_finish", "k_lu_solve", "k_jacobi_svd",
-                "k_gemm_z64", "k_pchol", "k_trinv", "k_gj_sweep", "k_gjb_inv", "k_gjb_persistent"}
+                "k_gemm_z64", "k_gemm_dir", "k_gmres_cl", "k_pchol", "k_trinv", "k_gj_sweep", "k_gjb_inv",
+                "k_gjb_persistent"}
+# FP64 products on the FP16 tensor cores: 28 exact digit products for one FP64 one
+OZ_KERNELS, OZ_PRODUCTS = {"k_oz_gemm"}, 28
 FP32_KERNELS = {"k_far", "k_fused", "k_matvec", "k_gemm_c32"}
 
 
@@ -137,6 +140,12 @@ def roofline(name, rec, peaks, peak_src):
                     "peak_source": ("nominal FP64 1.25 TFLOP/s (FP64 units, 2070 MHz)" if fp64 else
                                     f"derived: {DEV['n_sm']} SM x 128 FP32 lanes x 2 flop x "
                                     f"{DEV['sm_max_mhz']:.0f} MHz")})
+    elif name in OZ_KERNELS:
+        peak = (peaks.get("bf16_tflops") or 0.0) / OZ_PRODUCTS or None
+        ach = rec.get("flop", 0.0) / secs / 1e12 if secs > 0 and rec.get("flop") else None
+        out.update({"bound": "tensor", "unit": "TFLOP/s", "peak": peak, "achieved": ach,
+                    "frac": (ach / peak) if ach and peak else None,
+                    "peak_source": f"{peak_src}: 16-bit tensor rate over {OZ_PRODUCTS} digit products per FP64 product"})
     else:
         peak = peaks.get("hbm_gbs")
         ach = rec.get("bytes", 0.0) / secs / 1e9 if secs > 0 and rec.get("bytes") else None
