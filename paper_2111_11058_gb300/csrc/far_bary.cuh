@@ -23,7 +23,7 @@
 // cycles and 3.2e3 issue slots per 32 pairs against 4.9e3 of both before.  In FP64
 // the pipe is the bound and the shorter sums are the gain.  Far pairs of the
 // 9216-unknown cube by themselves 1.2 -> 0.8 ms, with the near pairs beside them
-// 2.15 -> 1.80 ms; FP64, 2304 unknowns: 4.8 -> 3.4 ms.
+// 2.15 -> 1.80 ms (1.51 with the near pairs' present form); FP64, 2304 unknowns: 4.8 -> 3.4 ms.
 #pragma once
 
 #include "far_math.cuh"

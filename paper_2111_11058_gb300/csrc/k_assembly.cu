@@ -994,7 +994,7 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
 // picked once per device and precision by timing the candidates, twice each,
 // on the first batch (every candidate writes the same values, so the batch
 // is not run again afterwards).  lean: the near pairs' closed forms with the
-// short elementary functions (near pairs of the 9216-unknown cube 1.73 -> 1.15 ms
+// short elementary functions (near pairs of the 9216-unknown cube 1.73 -> 0.89 ms
 // by themselves) and the far pairs in barycentric moments (far_bary.cuh); the conventional MoM, whose
 // long restarted solves carry a last bit of Z into the currents, and mixed
 // systems beyond SPREAD_ASM keep the general ones.
@@ -1138,7 +1138,8 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         for (const auto &J : jobs) ntmax = std::max(ntmax, J.nt);
         const size_t sm = (size_t)6 * ntmax * sizeof(cx<T>);
         if (sizeof(T) == 4 && sm <= GATHER_SM) {
-            CBFM_CUDA(cudaFuncSetAttribute(k_gather_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            // the same limit from every thread: a smaller one set in between would fail the other's launch
+            CBFM_CUDA(cudaFuncSetAttribute(k_gather_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GATHER_SM));
             int occ = 0;
             CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gather_rows<T>, 256, sm));
             const unsigned grid = (unsigned)std::min<int64_t>(nrows, (int64_t)std::max(1, occ) * nsm);

@@ -1778,11 +1778,13 @@ void lu_solve_batched(int nb, const int64_t *h_zoff, const int64_t *h_voff, cons
     for (int k = 0; k < nb; ++k) nmax = std::max(nmax, h_n[k]);
     size_t smem = sizeof(z64) * 2 * (size_t)nmax;
     DevBuf<z64> scratch;
-    if (smem > 160 * 1024) {
+    constexpr size_t LU_SM = 160 * 1024;
+    if (smem > LU_SM) {
         scratch.alloc((size_t)nb * LU_CL * 2 * nmax);
         smem = 0;
     } else {
-        CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // the same limit from every thread: a smaller one set in between would fail the other's launch
+        CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LU_SM));
     }
     {
         ProfScope ps_("k_lu_solve", st);

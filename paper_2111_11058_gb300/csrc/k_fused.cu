@@ -888,7 +888,7 @@ void fused_launch(std::vector<FusedJob> &jobs, const std::vector<std::pair<doubl
     std::stable_sort(items.begin(), items.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
     std::vector<int4> hit(items.size());
     for (size_t i = 0; i < items.size(); ++i) hit[i] = items[i].second;
-    CBFM_REQUIRE(plan.total <= FU_SMEM, "fused assembly: shared-memory plan too large");
+    CBFM_REQUIRE(plan.total + FU_STATIC <= FU_SMEM, "fused assembly: shared-memory plan too large");
     const uint32_t tcols = plan.nacc * plan.acol <= 256 ? 256u : 512u;
     const int nj = j1 - j0;
     DevBuf<FusedJob> djobs;
@@ -904,7 +904,9 @@ void fused_launch(std::vector<FusedJob> &jobs, const std::vector<std::pair<doubl
     CBFM_CUDA(cudaMemsetAsync(counter.p, 0, sizeof(unsigned int), st));
     CBFM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
     const size_t smem = plan.total + 1024;
-    CBFM_CUDA(cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the same limit from every thread: a smaller one set in between would fail the other's launch
+    CBFM_CUDA(cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)(FU_SMEM + 1024 - FU_STATIC)));
     const unsigned grid = (unsigned)std::min<int64_t>((int64_t)hit.size(), sm_count());
     {
         ProfScope ps_("k_fused", st);
