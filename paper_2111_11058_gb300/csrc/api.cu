@@ -652,9 +652,10 @@ cbfm_status cbfm_mesh(const double *verts, int64_t nv, const int32_t *tris, int6
         upload(m->edge_cell, ecell, st);
         m->tri64.alloc((size_t)h.nt * TRI_REC);
         m->tri32.alloc((size_t)h.nt * TRI_REC);
-        m->far64.alloc((size_t)h.nt * FB_REC);
-        m->far32.alloc((size_t)h.nt * FB_REC);
-        m->geo.alloc((size_t)h.nt * GEO_REC);
+        m->shape.alloc((size_t)h.nt * (3 * FB_REC + 2 * GEO_REC));
+        m->far32.p = m->shape.p;
+        m->far64.p = reinterpret_cast<double *>(m->far32.p + (size_t)h.nt * FB_REC);
+        m->geo.p = m->far64.p + (size_t)h.nt * FB_REC;
         launch_tri_records(*m, dv.p, dt.p, st);
         launch_tri_geo(*m, st);
         launch_near_pairs(*m, st);

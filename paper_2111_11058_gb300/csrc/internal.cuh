@@ -43,9 +43,10 @@ struct Mesh : HandleBase {
     z64 k1, k2, eta1, eta2;
     DevBuf<double> tri64;        // nt * TRI_REC
     DevBuf<float> tri32;         // nt * TRI_REC (centred coordinates)
-    DevBuf<double> far64;        // nt * FB_REC (far_bary.cuh)
-    DevBuf<float> far32;
-    DevBuf<double> geo;          // nt * GEO_REC (unit vectors of the near pairs' closed forms)
+    DevBuf<float> shape;         // one allocation: far32 and far64 (nt * FB_REC each, far_bary.cuh; 16-byte pieces),
+                                 // geo (nt * GEO_REC, unit vectors of the near pairs' closed forms)
+    struct { float *p = nullptr; } far32;
+    struct { double *p = nullptr; } far64, geo;
     DevBuf<int32_t> tri_vid;     // nt*3 vertex ids
     DevBuf<int32_t> tri_edge;    // nt*3 internal edge id
     DevBuf<int32_t> tri_cell;    // nt*3 cell of each of the triangle's RWGs
