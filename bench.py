@@ -118,7 +118,7 @@ DEV = {"n_sm": 152, "sm_max_mhz": 2070.0}
 def fp32_peak_tflops() -> float:
     return DEV["n_sm"] * FP32_LANES_PER_SM * 2 * DEV["sm_max_mhz"] * 1e6 / 1e12
 FP64_KERNELS = {"k_dots", "k_orth_update", "k_near_blocks", "k_finish", "k_lu_solve", "k_jacobi_svd",
-                "k_gemm_z64", "k_gemm_dir", "k_gmres_cl", "k_pchol", "k_trinv", "k_gj_sweep", "k_gjb_inv",
+                "k_gemm_z64", "k_gemm_dir", "k_gmres_cl", "k_pchol", "k_chol_blk", "k_trinv", "k_trinv_blk", "k_gj_sweep", "k_gjb_inv",
                 "k_gjb_persistent"}
 # FP64 products on the FP16 tensor cores: 28 exact digit products for one FP64 one
 OZ_KERNELS, OZ_PRODUCTS = {"k_oz_gemm"}, 28
