@@ -910,6 +910,11 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     c.Dinv.alloc((size_t)CH_NPAN * CH_B * CH_B);
     CBFM_CUDA(cudaMemsetAsync(c.err.p, 0, sizeof(int), st));
     OzWork oz_(c.err.p);   // scratch of the tensor-core products; their error word is read with the Cholesky's
+    // Without the CMP a restarted solve runs for hundreds of block iterations and its last digits decide whether it
+    // stagnates: every product keeps the FP64 units' sums, the operator's and the Hessenberg matrix's among them (MoM of a
+    // 408-unknown cylinder, 10 right-hand sides, restart 200: 1577 block iterations, more than 4000 with those two on
+    // the tensor cores and in the small kernels).
+    OzHold plain_(pc != CBFM_PC_CMP);
     c.rnrm.alloc(PCHOL_MAX);
     c.scale.alloc(PCHOL_MAX);
     c.dev.alloc(1 + GD_CTAS);   // the deviation and its per-CTA partials
@@ -999,8 +1004,8 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     CBFM_CUDA(cudaStreamSynchronize(st));
 
     // The basis (Gram-Schmidt and its Cholesky QR) on the tensor cores, except where the FP32 operator would carry a change
-    // of its last bits into the currents (SPREAD_MAX), and in the slowly converging systems without the CMP: there the
-    // FP64 units' order of sums and the FP32 solution update stay.
+    // of its last bits into the currents (SPREAD_MAX), and in the systems without the CMP (above): there the FP64 units'
+    // order of sums and the FP32 solution update stay.
     const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.cbf->spread <= SPREAD_MAX);
     OzMat op;   // FP64 operator cut into digits once per solve
     auto applyB = [&](const z64 *in, z64 *out, int rows) {

@@ -1,0 +1,66 @@
+"""Which products of a solve may be cut into digits of row-scaled fixed point (the tensor-core FP64 form), and what
+depends on it.
+
+A digit product is off by about 2^-56 of the largest entries of a row and a column, an FP64 sum by 2^-53 of the
+products it adds: rows whose entries differ by orders of magnitude lose digits in the first form that
+the second keeps.
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.init()
+    from paper_2111_11058_gb300 import build as B
+    B.build()
+    import paper_2111_11058_gb300 as pkg
+    return pkg
+
+
+def _launches(P, call):
+    """Kernels launched by a call, name -> launches."""
+    P.profile(True)
+    P.profile_read()
+    try:
+        call()
+        return {k: v["launches"] for k, v in P.profile_read().items()}
+    finally:
+        P.profile(False)
+
+
+def test_mom_block_solve_converges(P):
+    """Restarted block GMRES on the conventional MoM system (924 unknowns, 16 right-hand sides): about 1000 block
+    iterations with FP64 sums, more than 3000 where the operator's and the Hessenberg matrix's products lose digits."""
+    g = W.cylinder(0.2, 0.5, 14, 8, 2)
+    mom = P.assemble_mom(P.mesh(g.verts, g.tris, 2, 3.0), P.FP64)
+    P.tdiag_setup(mom, jacobi=True)
+    exc = W.plane_wave_set(W.fibonacci_dirs(8))
+    s = P.solve(mom, exc, tol=1e-6, maxit=2000, restart=200, precond=P.PC_TDIAG, solver=P.BLOCK, monostatic=True,
+                allow_noconv=True)
+    assert s.resid.max() <= 1e-6 and (s.iters > 0).all()
+
+
+@pytest.mark.parametrize("pc", ["none", "inexact", "tdiag"])
+def test_fp64_sums_without_the_cmp(P, pc):
+    g = W.cube(5, 0.6)
+    m = P.mesh(g.verts, g.tris, 3, 2.5)
+    exc = W.plane_wave_set(W.fibonacci_dirs(20))
+    kw = dict(tol=1e-6, maxit=20, restart=300, solver=P.BLOCK, monostatic=True, allow_noconv=True)
+    if pc == "tdiag":
+        r = P.assemble_mom(m, P.FP64)
+        P.tdiag_setup(r, jacobi=True)
+        kw["precond"] = P.PC_TDIAG
+    else:
+        r = P.assemble_reduced(m, P.build_cbfs(m, W.plane_wave_set(W.fibonacci_dirs(24))), P.FP64)
+        P.cmp_setup(r, inexact=pc == "inexact", inner_tol=1e-5)
+        kw["precond"] = P.PC_NONE if pc == "none" else P.PC_CMP_INEXACT
+    n = _launches(P, lambda: P.solve(r, exc, **kw))
+    assert n.get("k_oz_gemm", 0) == 0 and n.get("k_gemm_dir", 0) == 0
