@@ -925,6 +925,9 @@ void project(Red &r, cudaStream_t st) {
     const cx<T> *CM, *CJ;
     if constexpr (sizeof(T) == 8) { CM = c.CM.p; CJ = c.CJ.p; }
     else { CM = c.CM32.p; CJ = c.CJ32.p; }
+    // as many products as cells: FP64 sums also for a single one, whose rows (near and far entries of Z) differ by orders
+    // of magnitude (one cell of 336 RWGs: relative error of the T blocks 2e-16, cut into digits 1.1e-15)
+    OzHold hold_(true);
     // chains: (operator, coefficient side of the columns, row test side, A row block, A column block)
     struct Chain { int op; bool colM; bool rowJ; int64_t r0, c0; };
     const Chain ch[4] = {{0, true, true, 0, 0}, {1, false, true, 0, nh}, {2, true, false, nh, 0}, {0, false, false, nh, nh}};
@@ -1033,6 +1036,7 @@ void reduced_rhs_rows(Red &r, const double *d_exc, int nrhs, z64 *b, cudaStream_
             gemm_grouped<float>(gH, 2, 0, c.CM32.p, h32.p, b32.p, false, st);
             launch_c32_to_z64(b32.p, bt.p, n * nrhs, st);
         } else {
+            OzHold hold_(true);   // as many products as cells: FP64 sums also for a single one
             gemm_grouped<double>(gE, 2, 0, c.CJ.p, vE.p, bt.p, false, st);
             gemm_grouped<double>(gH, 2, 0, c.CM.p, vH.p, bt.p, false, st);
         }
@@ -1074,6 +1078,7 @@ void recover_currents(Red &r, const z64 *x, int nrhs, z64 *jint, cudaStream_t st
         gemm_grouped<float>(jJ, 0, 1, c.CJ32.p, x32.p, j32.p, false, st);
         launch_c32_to_z64(j32.p, jint, 2 * ne * nrhs, st);
     } else {
+        OzHold hold_(true);   // as many products as cells: FP64 sums also for a single one
         gemm_grouped<double>(jM, 0, 1, c.CM.p, x, jint, false, st);
         gemm_grouped<double>(jJ, 0, 1, c.CJ.p, x, jint, false, st);
     }

@@ -64,3 +64,23 @@ def test_fp64_sums_without_the_cmp(P, pc):
         kw["precond"] = P.PC_NONE if pc == "none" else P.PC_CMP_INEXACT
     n = _launches(P, lambda: P.solve(r, exc, **kw))
     assert n.get("k_oz_gemm", 0) == 0 and n.get("k_gemm_dir", 0) == 0
+
+
+def test_one_cell_products_keep_fp64_sums(P):
+    """FP64 products with identity CBF blocks are exact (one term of every sum is not zero), so A is Z entry by entry
+    whatever the number of cells, also where the entries of a row differ by 1e5."""
+    g = W.cube(4, 0.8)
+    A = []
+    for nc in (1, 3):
+        m = P.mesh(g.verts, g.tris, nc, 2.5 - 0.1j)
+        cell = m.cells()
+        blocks = [np.eye(k, dtype=complex) for k in np.bincount(cell, minlength=nc)]
+        r = P.assemble_reduced(m, P.cbf_import(m, blocks, blocks), P.FP64)
+        order = np.argsort(np.argsort(cell, kind="stable"))   # CBFs follow the cells, RWG functions the mesh
+        order = np.concatenate([order, len(cell) + order])
+        A.append(r.export()[np.ix_(order, order)])
+        if nc == 1:   # right-hand sides and currents of the one cell
+            exc = W.plane_wave_set(W.fibonacci_dirs(20))
+            n = _launches(P, lambda: P.solve(r, exc, maxit=2, precond=P.PC_NONE, monostatic=True, allow_noconv=True))
+    assert np.array_equal(A[0], A[1])
+    assert n.get("k_oz_gemm", 0) == 0
