@@ -442,7 +442,7 @@ std::unique_ptr<Cbf> dual_cbfs(Mesh *m, int s, const z64 *Vm, const std::vector<
         // G' = (J^M)^H T1
         g2.push_back(GemmDesc{s, s, N, voff[c], s, t1off[c], s, soff[c], s});
     }
-    OzHold hold_(true);   // the CBFs keep one order of sums, whatever the number of cells
+    OzHold hold_(OZ_ONE_ORDER);   // the CBFs keep one order of sums, whatever the number of cells
     gemm_grouped<double>(g1, 0, 0, Gm.p, Vm, T1.p, false, st);
     gemm_grouped<double>(g2, 2, 0, Vm, T1.p, Gp.p, false, st);
     X.alloc((size_t)nc * s * s);
@@ -927,7 +927,7 @@ void project(Red &r, cudaStream_t st) {
     else { CM = c.CM32.p; CJ = c.CJ32.p; }
     // as many products as cells: FP64 sums also for a single one, whose rows (near and far entries of Z) differ by orders
     // of magnitude (one cell of 336 RWGs: relative error of the T blocks 2e-16, cut into digits 1.1e-15)
-    OzHold hold_(true);
+    OzHold hold_(OZ_FP64_SUMS);
     // chains: (operator, coefficient side of the columns, row test side, A row block, A column block)
     struct Chain { int op; bool colM; bool rowJ; int64_t r0, c0; };
     const Chain ch[4] = {{0, true, true, 0, 0}, {1, false, true, 0, nh}, {2, true, false, nh, 0}, {0, false, false, nh, nh}};
@@ -985,7 +985,7 @@ void gram_cbf(Red &r, cudaStream_t st) {
         gJ.push_back(GemmDesc{L, nh, N, c.boff[k], L, off * nh, nh, c.coff[k] * n, n});
     }
     {
-        OzHold hold_(true);   // as many products as cells: one order of sums also for a single one
+        OzHold hold_(OZ_ONE_ORDER);   // as many products as cells: one order of sums also for a single one
         gemm_grouped<double>(gJ, 2, 0, c.CJ.p, XM.p, r.G.p, false, st);
     }
     // second half (C^M)^H Gf C^J = -((C^J)^H Gf C^M)^H: the RWG Gram Gf = <f_a, n x f_b> is
@@ -1036,7 +1036,7 @@ void reduced_rhs_rows(Red &r, const double *d_exc, int nrhs, z64 *b, cudaStream_
             gemm_grouped<float>(gH, 2, 0, c.CM32.p, h32.p, b32.p, false, st);
             launch_c32_to_z64(b32.p, bt.p, n * nrhs, st);
         } else {
-            OzHold hold_(true);   // as many products as cells: FP64 sums also for a single one
+            OzHold hold_(OZ_FP64_SUMS);   // as many products as cells: FP64 sums also for a single one
             gemm_grouped<double>(gE, 2, 0, c.CJ.p, vE.p, bt.p, false, st);
             gemm_grouped<double>(gH, 2, 0, c.CM.p, vH.p, bt.p, false, st);
         }
@@ -1078,7 +1078,7 @@ void recover_currents(Red &r, const z64 *x, int nrhs, z64 *jint, cudaStream_t st
         gemm_grouped<float>(jJ, 0, 1, c.CJ32.p, x32.p, j32.p, false, st);
         launch_c32_to_z64(j32.p, jint, 2 * ne * nrhs, st);
     } else {
-        OzHold hold_(true);   // as many products as cells: FP64 sums also for a single one
+        OzHold hold_(OZ_FP64_SUMS);   // as many products as cells: FP64 sums also for a single one
         gemm_grouped<double>(jM, 0, 1, c.CM.p, x, jint, false, st);
         gemm_grouped<double>(jJ, 0, 1, c.CJ.p, x, jint, false, st);
     }
@@ -1403,6 +1403,7 @@ cbfm_status cbfm_cmp_setup(cbfm_red_t red, void *stream) {
             gemm_grouped<float>(gb, 0, 0, r->A32.p, r->Ginv32.p, r->B32.p, false, st);
         } else {
             r->B64.alloc((size_t)n * n);
+            OzHold plain_(OZ_FP64_SUMS);   // FP64 sums: the columns of the inverse differ by the CBFs' spread (k_bgmres.cu)
             gemm_grouped<double>(gb, 0, 0, r->A64.p, r->Ginv.p, r->B64.p, false, st);
         }
         CBFM_CUDA(cudaStreamSynchronize(st));

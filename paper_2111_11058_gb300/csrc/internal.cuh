@@ -162,21 +162,24 @@ struct OzWork {
     OzWork(const OzWork &) = delete;
     OzWork &operator=(const OzWork &) = delete;
 };
-// While an object made with true is alive, oz_takes() answers no on this thread (products stay on the FP64 units).
-extern thread_local bool g_oz_hold;
+// What the FP64 products of this thread do without while an object is alive: OZ_FP64_SUMS the tensor cores' digits
+// (oz_takes() answers no), OZ_ONE_ORDER the small kernels too (dir_takes()): one order of sums whatever the sizes.
+constexpr int OZ_FREE = 0, OZ_FP64_SUMS = 1, OZ_ONE_ORDER = 2;
+extern thread_local int g_oz_hold;
 struct OzHold {
-    bool prev;
-    explicit OzHold(bool hold) : prev(g_oz_hold) { g_oz_hold = prev || hold; }
+    int prev;
+    explicit OzHold(int level) : prev(g_oz_hold) {
+        if (level > prev) g_oz_hold = level;
+    }
     ~OzHold() { g_oz_hold = prev; }
     OzHold(const OzHold &) = delete;
     OzHold &operator=(const OzHold &) = delete;
 };
-// A matrix cut into digits once and multiplied many times (the operator of an iterative solve): n_rows x n_k,
-// row-major, complex64 (widened exactly) or complex128.
+// A complex64 matrix (n_rows x n_k, row-major) cut into digits, its entries widened exactly.
 struct OzMat {
     DevBuf<unsigned char> buf;
     int64_t rows = 0, K = 0;
-    void pack(const void *X, bool f32, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st);
+    void pack(const c32 *X, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st);
 };
 // out[r] = M in[r] for n rows of leading dimensions ldi and ldo, FP64
 void gemm_oz_rows(const OzMat &M, const z64 *in, int64_t ldi, z64 *out, int64_t ldo, int64_t n, cudaStream_t st);

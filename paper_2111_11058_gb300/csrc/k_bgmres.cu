@@ -914,7 +914,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     // stagnates: every product keeps the FP64 units' sums, the operator's and the Hessenberg matrix's among them (MoM of a
     // 408-unknown cylinder, 10 right-hand sides, restart 200: 1577 block iterations, more than 4000 with those two on
     // the tensor cores and in the small kernels).
-    OzHold plain_(pc != CBFM_PC_CMP);
+    OzHold plain_(pc != CBFM_PC_CMP ? OZ_ONE_ORDER : OZ_FREE);
     c.rnrm.alloc(PCHOL_MAX);
     c.scale.alloc(PCHOL_MAX);
     c.dev.alloc(1 + GD_CTAS);   // the deviation and its per-CTA partials
@@ -1007,22 +1007,24 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     // of its last bits into the currents (SPREAD_MAX), and in the systems without the CMP (above): there the FP64 units'
     // order of sums and the FP32 solution update stay.
     const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.cbf->spread <= SPREAD_MAX);
-    OzMat op;   // FP64 operator cut into digits once per solve
+    OzMat inv;   // complex64 (G^CBF)^{-1} cut into digits (the recovery of mixed systems)
     auto applyB = [&](const z64 *in, z64 *out, int rows) {
         if (pc == CBFM_PC_CMP_INEXACT) {
             if (zin.p == nullptr) zin.alloc((size_t)p * n);
             cmp_inner_apply(rd, in, zin.p, rows, st);
             in = zin.p;
         }
-        if (tc_basis && rd.prec == CBFM_FP64 && oz_takes(rows, n, n)) {
-            if (op.rows == 0) op.pack(pc_op64(rd, pc), false, n, n, n, st);
-            GemmSite site_("site:operator");
-            gemm_oz_rows(op, in, n, out, n, rows, st);
+        if (rd.prec != CBFM_FP64) {
+            rows_times(n, nullptr, pc_op32(rd, pc), in, out, rows, false, st, s_in.p, s_out.p);
             return;
         }
-        if (rd.prec != CBFM_FP64)
-            rows_times(n, nullptr, pc_op32(rd, pc), in, out, rows, false, st, s_in.p, s_out.p);
-        else rows_times(n, pc_op64(rd, pc), nullptr, in, out, rows, false, st, nullptr, nullptr);
+        // FP64 sums: the columns of B = A (G^CBF)^{-1} differ by the CBFs' spread and the basis vectors by its inverse, so
+        // that both lose digits when they are cut below their rows' largest entry (29 FP64 solves of spheroids with a
+        // spread above 1e4 against refined dense solutions: errors of the currents 1.6 times as large as with FP64 sums
+        // of the products and of B, 2.4 times on one body; at n = 686, 45 right-hand sides 13.1 ms instead of 15.6)
+        OzHold plain64_(OZ_FP64_SUMS);
+        GemmSite site_("site:operator");
+        rows_times(n, pc_op64(rd, pc), nullptr, in, out, rows, false, st, nullptr, nullptr);
     };
 
     GmresOut out;
@@ -1100,7 +1102,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
         CBFM_CUDA(cudaMemsetAsync(Rh.p, 0, sizeof(z64) * dcap * dcap, st));
         int p1;
         {
-            OzHold hold_(!tc_basis);
+            OzHold hold_(tc_basis ? OZ_FREE : OZ_ONE_ORDER);
             p1 = cholqr2_rows(c, tmp.p, p, n, V.p, E1S.p, rank_tol, 0.0, drop_tol);
         }
         CBFM_CUDA(cudaMemcpyAsync(Rv.p, E1S.p, sizeof(z64) * dcap2 * p, cudaMemcpyDeviceToDevice, st));
@@ -1131,7 +1133,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             // others are orthogonal to the basis to ~10 u already), gathered into Ws
             {
                 GemmSite site_("site:gs1");
-                OzHold hold_(!tc_basis);
+                OzHold hold_(tc_basis ? OZ_FREE : OZ_ONE_ORDER);
                 gemm_grouped<double>({GemmDesc{pjc, d1, n, 0, n, 0, n, 0, dcap}}, 0, 2, W.p, V.p, tmp2.p, false, st);
                 gemm_grouped<double>({GemmDesc{pjc, n, d1, 0, dcap, 0, n, 0, n}}, 0, 0, tmp2.p, V.p, W.p, true, st,
                                      -1.0);
@@ -1153,7 +1155,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
                 }
             if (!sel.empty()) {
                 GemmSite site_("site:gs2");
-                OzHold hold_(!tc_basis);
+                OzHold hold_(tc_basis ? OZ_FREE : OZ_ONE_ORDER);
                 const int k = (int)sel.size();
                 const bool all = k == pjc;
                 if (!all) {
@@ -1182,7 +1184,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
             // orthonormalise the new block (pivoted: drops dependent directions)
             int r = 0;
             if (wref > 0.0) {
-                OzHold hold_(!tc_basis);
+                OzHold hold_(tc_basis ? OZ_FREE : OZ_ONE_ORDER);
                 r = cholqr2_rows(c, W.p, pjc, n, V.p + d1 * n, Rw.p, rank_tol, wref, drop_tol);
             }
             const int rr = r;
@@ -1310,13 +1312,12 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
         d_x = x_all->p;
     }
     if (pc == CBFM_PC_CMP) {   // G^CBF^{-1} is block diagonal (its two halves)
-        if (tc_basis && oz_takes(p, n / 2, n / 2)) {
-            // the inverse the operator was formed with: the complex64 one on the mixed path
+        if (rd.prec != CBFM_FP64 && tc_basis && oz_takes(p, n / 2, n / 2)) {
+            // the inverse the operator was formed with
             const int64_t h = n / 2;
             for (int64_t o = 0; o < n; o += h) {
-                if (rd.prec != CBFM_FP64) op.pack(rd.Ginv32.p + o * n + o, true, h, h, n, st);
-                else op.pack(rd.Ginv.p + o * n + o, false, h, h, n, st);
-                gemm_oz_rows(op, Y.p + o, n, d_x + o, n, p, st);
+                inv.pack(rd.Ginv32.p + o * n + o, h, h, n, st);
+                gemm_oz_rows(inv, Y.p + o, n, d_x + o, n, p, st);
             }
         } else if (rd.prec != CBFM_FP64) rows_times(n, nullptr, rd.Ginv32.p, Y.p, d_x, p, true, st, s_in.p, s_out.p);
         else rows_times(n, rd.Ginv.p, nullptr, Y.p, d_x, p, true, st, nullptr, nullptr);

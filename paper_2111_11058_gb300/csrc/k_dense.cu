@@ -1670,7 +1670,7 @@ bool gj_blocked(int64_t n, int nbatch, const z64 *Aorig, z64 *inv, cudaStream_t 
 
 // The product's shape as these kernels take it; false where they do not (large, or sums that keep the FP64 tiles' order).
 bool dir_takes(const GemmDesc &d) {
-    return !g_oz_hold && d.M > 0 && d.N > 0 && d.K > 0 && 1.0 * d.M * d.N * d.K <= 2.0e6 && d.M * d.N < (1 << 24);
+    return g_oz_hold < OZ_ONE_ORDER && d.M > 0 && d.N > 0 && d.K > 0 && 1.0 * d.M * d.N * d.K <= 2.0e6 && d.M * d.N < (1 << 24);
 }
 template <typename T>
 void gemm_grouped(const std::vector<GemmDesc> &g, int opA, int opB, const cx<T> *A, const cx<T> *B, cx<T> *C,

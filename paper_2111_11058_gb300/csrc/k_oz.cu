@@ -42,7 +42,7 @@ namespace cbfm {
 
 namespace cg = cooperative_groups;
 thread_local OzWork *g_oz = nullptr;
-thread_local bool g_oz_hold = false;
+thread_local int g_oz_hold = OZ_FREE;
 
 namespace {
 
@@ -648,7 +648,7 @@ struct Scratch {
 }  // namespace
 
 bool oz_takes(int64_t M, int64_t N, int64_t K) {
-    if (g_oz_hold || M < 1 || N < 1 || K < 1 || M > (1 << 24) || N > (1 << 24) || K > (1 << 18)) return false;
+    if (g_oz_hold >= OZ_FP64_SUMS || M < 1 || N < 1 || K < 1 || M > (1 << 24) || N > (1 << 24) || K > (1 << 18)) return false;
     const Shape s = oz_shape(M, N, K);
     if (s.bytes > ((size_t)2 << 30) || s.mt * s.nt > (1 << 24)) return false;
     return 1.0 * M * N * K > 2.0e6;
@@ -677,13 +677,13 @@ void gemm_oz(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z6
     ws.check();
 }
 
-void OzMat::pack(const void *X, bool f32, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st) {
+void OzMat::pack(const c32 *X, int64_t n_rows, int64_t n_k, int64_t ld, cudaStream_t st) {
     rows = n_rows;
     K = n_k;
     const int64_t mt = (rows + OZ_M - 1) / OZ_M;
     const size_t na = (size_t)mt * ((K + 15) / 16) * OZ_A_STAGE;
     buf.alloc(na + 4 * (size_t)(mt * OZ_M));
-    const OzPack p = pack_of(X, f32, 0, ld, 1, false, rows, false, buf.p, reinterpret_cast<int *>(buf.p + na));
+    const OzPack p = pack_of(X, true, 0, ld, 1, false, rows, false, buf.p, reinterpret_cast<int *>(buf.p + na));
     launch_pack(&p, 1, K, st);
 }
 

@@ -84,3 +84,17 @@ def test_one_cell_products_keep_fp64_sums(P):
             n = _launches(P, lambda: P.solve(r, exc, maxit=2, precond=P.PC_NONE, monostatic=True, allow_noconv=True))
     assert np.array_equal(A[0], A[1])
     assert n.get("k_oz_gemm", 0) == 0
+
+
+def test_fp64_operator_keeps_fp64_sums(P):
+    """B = A (G^CBF)^{-1} of an FP64 system, its product with the basis vectors and the recovery: the sizes are such that
+    the operator's products (5 n^2 > 2e6) are the only ones of the solve large enough for the tensor cores."""
+    g = W.cube(8, 1.0)
+    m = P.mesh(g.verts, g.tris, 16, 2.5)
+    r = P.assemble_reduced(m, P.build_cbfs(m, W.plane_wave_set(W.fibonacci_dirs(64))), P.FP64)
+    assert 5 * r.n ** 2 > 2e6 and 5 * (r.n // 2) ** 2 < 2e6
+    assert _launches(P, lambda: P.cmp_setup(r)).get("k_oz_gemm", 0) == 0
+    exc = W.plane_wave_set(W.fibonacci_dirs(3))[:5]
+    n = _launches(P, lambda: P.solve(r, exc, tol=1e-8, maxit=20, restart=r.n + 256, solver=P.BLOCK, monostatic=True,
+                                     allow_noconv=True))
+    assert n.get("k_oz_gemm", 0) == 0
