@@ -1062,7 +1062,23 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
     auto *far = lean ? k_far<T, true> : k_far<T, false>;
     const size_t far_sm = lean ? far_smem<T, true>() : far_smem<T, false>();
     auto *near = lean ? k_near_blocks<T, true> : k_near_blocks<T, false>;
-    bool near_done = false;
+    constexpr int FB = 32 * far_warps<T>();
+    CBFM_CUDA(cudaFuncSetAttribute(far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)far_sm));
+    int far_occ = 0;
+    CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&far_occ, far, FB, far_sm));
+    // the near pairs beside the far ones (FP32, shorter forms; inlined there, the general closed forms would have
+    // their products fused differently than in the near kernel, and they are taken for their bits)
+    const bool both = sizeof(T) == 4 && lean && npairs > 0;
+    const double near_flop = (double)npairs * near_fp64_ops<T>();
+    const double near_bytes = (double)npairs * (2 * TRI_REC * sizeof(double) + 27 * sizeof(cx<T>));
+    // profiled under `name`: the first `ntask` far tasks and, where near_too is set, the near pairs
+    auto run = [&](const char *name, int64_t ntask, bool near_too) {
+        CBFM_CUDA(cudaMemsetAsync(counter.p, 0, 2 * sizeof(unsigned long long), st));
+        ProfScope ps_(name, st);
+        far<<<(unsigned)std::max(1, far_occ) * (unsigned)nsm, FB, far_sm, st>>>(
+            djobs.p, nj, ntask, counter.p, near_too ? npairs : 0, near_too ? 2 * nsm : 0);
+        launched("k_far");
+    };
     for (int rep = 0; rep < reps; ++rep)
     for (size_t ci = 0; ci < cands.size(); ++ci) {
         const int W = cands[ci];
@@ -1074,31 +1090,15 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
             ntask += far_tasks(J);
         }
         CBFM_CUDA(cudaMemcpyAsync(djobs.p, jobs.data(), sizeof(AsmJob<T>) * nj, cudaMemcpyHostToDevice, st));
-        CBFM_CUDA(cudaMemsetAsync(counter.p, 0, 2 * sizeof(unsigned long long), st));
-        constexpr int FB = 32 * far_warps<T>();
-        CBFM_CUDA(cudaFuncSetAttribute(far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)far_sm));
-        int occ = 0;
-        CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, far, FB, far_sm));
-        const unsigned grid = (unsigned)std::max(1, occ) * (unsigned)nsm;
-        // the near pairs beside the far ones (FP32, shorter forms; inlined there, the general closed forms would have
-        // their products fused differently than in the near kernel, and they are taken for their bits)
         if (tuned > 0) {
-            const bool both = sizeof(T) == 4 && lean && npairs > 0;
-            near_done = both;
-            ProfScope ps_("k_far", st);
-            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, both ? npairs : 0, both ? 2 * nsm : 0);
-            launched("k_far");
+            run("k_far", ntask, both);
             break;
         }
         cudaEvent_t e0, e1;
         CBFM_CUDA(cudaEventCreate(&e0));
         CBFM_CUDA(cudaEventCreate(&e1));
         CBFM_CUDA(cudaEventRecord(e0, st));
-        {
-            ProfScope ps_("k_far", st);
-            far<<<grid, FB, far_sm, st>>>(djobs.p, nj, ntask, counter.p, 0, 0);
-            launched("k_far");
-        }
+        run("k_far", ntask, false);
         CBFM_CUDA(cudaEventRecord(e1, st));
         CBFM_CUDA(cudaEventSynchronize(e1));
         float ms_ = 0.f;
@@ -1112,11 +1112,13 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         for (size_t ci = 1; ci < cands.size(); ++ci)
             if (t_ms[ci] < t_ms[bi]) bi = ci;
         tuning_set(key, cands[bi]);
+        // the near pairs by the kernel that takes them on every later call: one piece of code for their bits
+        if (both) run("k_near_blocks", 0, true);
     }
+    // the near pairs' work to the launch that did it
     prof_add_work("k_far", far_flop, far_bytes);
-    prof_add_work("k_near_blocks", (double)npairs * near_fp64_ops<T>(),
-                  (double)npairs * (2 * TRI_REC * sizeof(double) + 27 * sizeof(cx<T>)));
-    if (npairs > 0 && !near_done) {
+    if (npairs > 0) prof_add_work(both && tuned > 0 ? "k_far" : "k_near_blocks", near_flop, near_bytes);
+    if (npairs > 0 && !both) {
         int occ = 0;
         CBFM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, near, 128, 0));
         const unsigned grid = (unsigned)std::min<int64_t>((int64_t)std::max(1, occ) * nsm, ((npairs + 1) / 2 * 32 + 127) / 128);
