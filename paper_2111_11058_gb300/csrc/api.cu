@@ -232,36 +232,61 @@ __global__ void k_gram_times_c(int64_t ne, int64_t nh, const int32_t *__restrict
     }
 }
 
-// |(C^J_l)^H Gf C^M_l| of every CBF l over the RWG functions of its own cell: the modulus of the diagonal of G^CBF.
-// One warp per CBF.
-__global__ void k_cbf_diag(int nc, int64_t nh, const int32_t *__restrict__ cell_off, const int64_t *__restrict__ coff,
-                           const int64_t *__restrict__ boff, const int32_t *__restrict__ Lc,
-                           const double *__restrict__ val, const int32_t *__restrict__ col,
-                           const z64 *__restrict__ CM, const z64 *__restrict__ CJ, double *__restrict__ out) {
-    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (q >= nh) return;
-    int lo = 0, hi = nc - 1;
-    while (lo < hi) {   // last cell with coff <= q
-        const int mid = (lo + hi + 1) / 2;
-        if (coff[mid] <= q) lo = mid;
-        else hi = mid - 1;
-    }
-    const int64_t off = cell_off[lo], end = cell_off[lo + 1], L = Lc[lo], l = q - coff[lo];
-    const z64 *cm = CM + boff[lo] + l, *cj = CJ + boff[lo] + l;
-    z64 acc(0, 0);
-    for (int64_t i = off + (threadIdx.x & 31); i < end; i += 32) {
-        z64 g(0, 0);
-        for (int sl = 0; sl < 6; ++sl) {
-            const int64_t cc = col[6 * i + sl];
-            if (cc >= off && cc < end) g += val[6 * i + sl] * cm[(cc - off) * L];
+// |(C^J_l)^H Gf C^M_l| of every CBF l over the RWG functions of its own cell, the modulus of the diagonal of G^CBF, to
+// FP32 accuracy.  One block per 32 CBFs of a cell (blocks (c, i) past the cell's CBFs leave): lanes over the CBFs, so
+// that the coefficients are read in whole rows, five rows of Gf at a time per warp, their 30 entries converted by
+// 30 lanes and handed round.  Bound: latency of two dependent loads per five rows (import of
+// 12 CBFs on one cell of 450 RWGs 82 us, on two of 576 87 us; 104 and 118 us with a warp per CBF and FP64 sums, whose
+// few blocks held one FP64 pipe each; 50 us without this stage).
+// tab: cell offsets, CBF offsets, block offsets (nc + 1 each) and L (nc).
+constexpr int CD_WARPS = 32;
+__global__ void __launch_bounds__(32 * CD_WARPS)
+    k_cbf_diag(int nc, const int64_t *__restrict__ tab, const double *__restrict__ val, const int32_t *__restrict__ col,
+               const c32 *__restrict__ CM, const c32 *__restrict__ CJ, float *__restrict__ out) {
+    const int c = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t off = tab[c], end = tab[c + 1], L = tab[3 * (nc + 1) + c], l = blockIdx.y * 32LL + lane;
+    if (blockIdx.y * 32LL >= L) return;
+    const c32 *cm = CM + tab[2 * (nc + 1) + c] + l, *cj = CJ + tab[2 * (nc + 1) + c] + l;
+    __shared__ float s_acc[2][CD_WARPS][32];
+    float re = 0.f, im = 0.f;
+    for (int64_t i0 = off + 5 * warp; i0 < end; i0 += 5 * CD_WARPS) {
+        float v = 0.f;
+        int k = -1;
+        if (lane < 30 && i0 + lane / 6 < end) {
+            const int64_t cc = col[6 * i0 + lane];
+            v = (float)val[6 * i0 + lane];
+            if (cc >= off && cc < end) k = (int)(cc - off);
         }
-        cfmaconj(acc, cj[(i - off) * L], g);
+#pragma unroll
+        for (int r = 0; r < 5; ++r) {
+            float gr = 0.f, gi = 0.f;
+#pragma unroll
+            for (int s = 0; s < 6; ++s) {
+                const float w = __shfl_sync(0xffffffffu, v, 6 * r + s);
+                const int kk = __shfl_sync(0xffffffffu, k, 6 * r + s);
+                if (kk >= 0 && l < L) {
+                    const c32 x = cm[kk * L];
+                    gr = fmaf(w, x.re, gr);
+                    gi = fmaf(w, x.im, gi);
+                }
+            }
+            if (l < L && i0 + r < end) {
+                const c32 x = cj[(i0 + r - off) * L];
+                re = fmaf(x.re, gr, fmaf(x.im, gi, re));
+                im = fmaf(x.re, gi, fmaf(-x.im, gr, im));
+            }
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
-        acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+    s_acc[0][warp][lane] = re;
+    s_acc[1][warp][lane] = im;
+    __syncthreads();
+    if (warp == 0 && l < L) {
+        for (int w = 1; w < CD_WARPS; ++w) {
+            re += s_acc[0][w][lane];
+            im += s_acc[1][w][lane];
+        }
+        out[tab[nc + 1 + c] + l] = hypotf(re, im);
     }
-    if ((threadIdx.x & 31) == 0) out[q] = sqrt(norm2(acc));
 }
 
 // complex transpose: dst (cols x rows) = src (rows x cols)^T
@@ -376,23 +401,24 @@ void cbf_make32(Cbf &c, cudaStream_t st) {
 void cbf_spread(Cbf &c, cudaStream_t st) {
     const Mesh &m = *c.mesh;
     const int nc = m.h.ncell;
-    DevBuf<int32_t> dcell, dL;
-    DevBuf<int64_t> dcoff, dboff;
-    DevBuf<double> g;
-    upload(dcell, m.h.cell_off, st);
-    upload(dL, c.L, st);
-    upload(dcoff, c.coff, st);
-    upload(dboff, c.boff, st);
-    g.alloc(c.nhalf);
-    k_cbf_diag<<<nblk(c.nhalf * 32), 256, 0, st>>>(nc, c.nhalf, dcell.p, dcoff.p, dboff.p, dL.p, m.gram_val.p,
-                                                   m.gram_col.p, c.CM.p, c.CJ.p, g.p);
+    std::vector<int64_t> tab(m.h.cell_off.begin(), m.h.cell_off.end());
+    tab.insert(tab.end(), c.coff.begin(), c.coff.end());
+    tab.insert(tab.end(), c.boff.begin(), c.boff.end());
+    tab.insert(tab.end(), c.L.begin(), c.L.end());
+    DevBuf<int64_t> buf;   // the table, then the result
+    buf.alloc(tab.size() + c.nhalf);
+    CBFM_CUDA(cudaMemcpyAsync(buf.p, tab.data(), sizeof(int64_t) * tab.size(), cudaMemcpyHostToDevice, st));
+    float *g = reinterpret_cast<float *>(buf.p + tab.size());
+    const int lmax = *std::max_element(c.L.begin(), c.L.end());
+    k_cbf_diag<<<dim3((unsigned)nc, (unsigned)((lmax + 31) / 32)), 32 * CD_WARPS, 0, st>>>(nc, buf.p, m.gram_val.p, m.gram_col.p,
+                                                                                      c.CM32.p, c.CJ32.p, g);
     launched("k_cbf_diag");
-    std::vector<double> h(c.nhalf);
-    CBFM_CUDA(cudaMemcpyAsync(h.data(), g.p, sizeof(double) * c.nhalf, cudaMemcpyDeviceToHost, st));
+    std::vector<float> h(c.nhalf);
+    CBFM_CUDA(cudaMemcpyAsync(h.data(), g, sizeof(float) * c.nhalf, cudaMemcpyDeviceToHost, st));
     CBFM_CUDA(cudaStreamSynchronize(st));
     const auto mm = std::minmax_element(h.begin(), h.end());
-    c.spread = *mm.first > 0.0 ? *mm.second / *mm.first : INFINITY;
-    for (double v : h)
+    c.spread = *mm.first > 0.f ? (double)*mm.second / *mm.first : INFINITY;
+    for (float v : h)
         if (!(v <= *mm.second)) c.spread = INFINITY;   // a NaN among them
 }
 
