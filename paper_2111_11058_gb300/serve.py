@@ -348,7 +348,9 @@ class Server:
         if not self.joins or g is None or g.state == "done" or g.nrhs + req.nrhs > self.max_rhs:
             return False
         sc = req.scatterer
-        delta = solve_bytes(g.entry.n, g.nrhs + req.nrhs, sc.ne) - solve_bytes(g.entry.n, g.nrhs, sc.ne)
+        # a solved group kept open holds no session: its first request opens one of its own
+        held = solve_bytes(g.entry.n, g.nrhs, sc.ne) if g.nrhs else 0
+        delta = solve_bytes(g.entry.n, g.nrhs + req.nrhs, sc.ne) - held
         if self.resident_bytes() + self.inflight + delta > self.budget:
             return False
         if g.state == "running":
