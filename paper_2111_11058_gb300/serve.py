@@ -377,6 +377,7 @@ class Server:
             if g.key in self.open or not self.joins:
                 return False
             g.members, g.nrhs, g.state, g.session = [], 0, "idle", None
+            g.hit = True      # a request that joins now finds the entry resident
             self.inflight -= g.scratch
             g.scratch = 0
             self.open[g.key] = g

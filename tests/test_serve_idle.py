@@ -66,3 +66,15 @@ def test_nothing_waits_for_an_idle_group(monkeypatch):
     srv.close()
     assert time.perf_counter() - t0 < 0.2
     assert not any(srv.busy) and srv.inflight == 0
+
+
+def test_a_request_on_the_resident_entry_is_a_hit(monkeypatch):
+    """The batch that built the entry missed; a request solved later on the entry it left did not."""
+    monkeypatch.setattr(S, "KEEP_OPEN_S", 5.0)
+    sc = scat("a")
+    srv = S.Server(FakeBackend(build_s=0.2, solve_s=0.01), hbm_budget=10**12, n_streams=1)
+    first = srv.submit(req(sc, 1.0, 4, 0)).result(timeout=30)
+    _idle(srv, ("a", 1.0))
+    second = srv.submit(req(sc, 1.0, 4, 1)).result(timeout=30)
+    srv.close()
+    assert not first.cache_hit and second.cache_hit and second.batch_id == first.batch_id
