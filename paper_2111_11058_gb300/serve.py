@@ -561,7 +561,8 @@ class Server:
                     return
                 groups, transient, bid = self.work[w]
             t_start = time.perf_counter()
-            ev0 = self.be.event(st) if self.t0_event is not None else None
+            timed = self.t0_event is not None
+            ev0 = self.be.event(st) if timed else None
             # builds of the cache misses, together
             misses = [g for g in groups if not g.hit]
             build_err: Optional[BaseException] = None
@@ -591,21 +592,27 @@ class Server:
             # the solves, one session per key; joins reach a session while it runs
             rec = {"batch": bid, "worker": w, "keys": [g.key for g in groups], "requests": 0, "joined": 0, "rhs": 0,
                    "hit": all(g.hit for g in groups), "t_start": t_start}
+            if timed:
+                rec["dev_later_ms"] = []      # solves of a group kept open, after the batch's own interval dev_ms
 
-            def served(counts):   # the batch's record so far
-                ev1 = self.be.event(st) if ev0 is not None else None
+            def served(counts, start):   # the batch's record so far
                 rec.update(requests=rec["requests"] + sum(c[0] for c in counts), rhs=rec["rhs"] + sum(c[1] for c in counts),
                            joined=sum(g.joined for g in groups), t_end=time.perf_counter(),
                            error=any(g.entry.error is not None for g in groups))
-                if ev0 is not None:
-                    rec["dev_ms"] = (self.be.elapsed_ms(self.t0_event, ev0), self.be.elapsed_ms(self.t0_event, ev1))
+                if timed:
+                    span = tuple(self.be.elapsed_ms(self.t0_event, e) for e in (start, self.be.event(st)))
+                    if "dev_ms" in rec:
+                        rec["dev_later_ms"].append(span)
+                    else:
+                        rec["dev_ms"] = span
 
-            served([self._solve_group(g, st, bid) for g in groups])
+            served([self._solve_group(g, st, bid) for g in groups], ev0)
             with self.lock:
                 self.log.append(rec)
             if len(groups) == 1 and not rec["error"] and hasattr(self.be, "open_session"):
                 while self._keep_open(groups[0], min(time.perf_counter() - t_start, KEEP_OPEN_S)):
-                    served([self._solve_group(groups[0], st, bid)])
+                    start = self.be.event(st) if timed else None
+                    served([self._solve_group(groups[0], st, bid)], start)
             with self.lock:
                 for g in groups:
                     g.entry.users -= 1
@@ -643,7 +650,7 @@ def summarize(results: List[Result], log: List[dict], wall_s: float, server: Opt
            "max_batch_requests": max([b["requests"] for b in log], default=0),
            "mean_batch_keys": float(np.mean([len(b.get("keys", [0])) for b in log])) if log else 0.0,
            "joined_requests": int(sum(b.get("joined", 0) for b in log))}
-    dev = [b["dev_ms"] for b in log if "dev_ms" in b]
+    dev = [span for b in log if "dev_ms" in b for span in [b["dev_ms"], *b.get("dev_later_ms", [])]]
     if dev:
         out["device_overlap_ms"] = overlap_ms(dev)
         out["device_busy_ms"] = float(sum(b - a for a, b in dev))

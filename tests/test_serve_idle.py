@@ -78,3 +78,30 @@ def test_a_request_on_the_resident_entry_is_a_hit(monkeypatch):
     second = srv.submit(req(sc, 1.0, 4, 1)).result(timeout=30)
     srv.close()
     assert not first.cache_hit and second.cache_hit and second.batch_id == first.batch_id
+
+
+class TimedBackend(FakeBackend):
+    def event(self, st):
+        return time.perf_counter()
+
+    def elapsed_ms(self, e0, e1):
+        return 1e3 * (e1 - e0)
+
+
+def test_the_idle_gap_is_not_device_time(monkeypatch):
+    monkeypatch.setattr(S, "KEEP_OPEN_S", 5.0)
+    sc = scat("a")
+    srv = S.Server(TimedBackend(build_s=0.3, solve_s=0.02), hbm_budget=10**12, n_streams=1)
+    res = [srv.submit(req(sc, 1.0, 4, 0)).result(timeout=30)]
+    _idle(srv, ("a", 1.0))
+    time.sleep(0.2)
+    res.append(srv.submit(req(sc, 1.0, 4, 1)).result(timeout=30))
+    srv.drain(timeout=10)
+    srv.close()
+    assert len(srv.log) == 1 and srv.log[0]["requests"] == 2 and srv.log[0]["joined"] == 1
+    a, b = srv.log[0]["dev_ms"]
+    (c, d), = srv.log[0]["dev_later_ms"]
+    assert b - a >= 320 and c - b >= 190 and d - c >= 20
+    stats = S.summarize(res, srv.log, 1.0, srv)
+    assert abs(stats["device_busy_ms"] - (b - a) - (d - c)) < 1e-9
+    assert stats["device_busy_ms"] < d - a - 190
