@@ -488,9 +488,9 @@ void gemm_dir(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z
 // Bound: the FP64 pipes, of eight SMs instead of one (16 systems of 147 unknowns
 // with 128 right-hand sides: 8.3 ms -> 2.1 ms), then the step's serial chain (the
 // column through L2, the pivot search, one division).  col, dinv: n entries each
-// per CTA, in shared memory where they fit.  info[b] = 1: singular; 2: a cluster
-// synchronisation expired.
-constexpr int LU_CL = 8;
+// per CTA in shared memory (n <= LU_NMAX, the largest cell system the CBF generation
+// takes).  info[b] = 1: singular; 2: a cluster synchronisation expired.
+constexpr int LU_CL = 8, LU_NMAX = 4096;
 
 // FP64 products with the rounding written out, in this and the next kernel: the CBFs they
 // give decide, through solves that amplify a last bit, the digits of every later result, so
@@ -515,15 +515,14 @@ __device__ __forceinline__ z64 ldcg64(const z64 *p) {
 
 __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
     k_lu_solve(const int64_t *__restrict__ zoff, const int64_t *__restrict__ voff, const int *__restrict__ nsz, int s,
-               z64 *__restrict__ Zall, z64 *__restrict__ Vall, int *__restrict__ info, z64 *__restrict__ scratch,
-               int nmax) {
+               z64 *__restrict__ Zall, z64 *__restrict__ Vall, int *__restrict__ info, int nmax) {
     extern __shared__ __align__(16) unsigned char lu_raw[];
     cg::cluster_group cl = cg::this_cluster();
     const int me = (int)cl.block_rank(), b = blockIdx.x / LU_CL;
     const int n = nsz[b];
     z64 *Z = Zall + zoff[b];
     z64 *V = Vall + voff[b];
-    z64 *col = scratch ? scratch + (int64_t)blockIdx.x * 2 * nmax : reinterpret_cast<z64 *>(lu_raw);
+    z64 *col = reinterpret_cast<z64 *>(lu_raw);
     z64 *dinv = col + nmax;
     __shared__ uint64_t cbar[2];
     __shared__ int piv, s_abort;
@@ -1776,19 +1775,13 @@ void lu_solve_batched(int nb, const int64_t *h_zoff, const int64_t *h_voff, cons
     CBFM_CUDA(cudaMemcpyAsync(nn.p, h_n, nb * sizeof(int), cudaMemcpyHostToDevice, st));
     int nmax = 1;
     for (int k = 0; k < nb; ++k) nmax = std::max(nmax, h_n[k]);
-    size_t smem = sizeof(z64) * 2 * (size_t)nmax;
-    DevBuf<z64> scratch;
-    constexpr size_t LU_SM = 160 * 1024;
-    if (smem > LU_SM) {
-        scratch.alloc((size_t)nb * LU_CL * 2 * nmax);
-        smem = 0;
-    } else {
-        // the same limit from every thread: a smaller one set in between would fail the other's launch
-        CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LU_SM));
-    }
+    CBFM_REQUIRE(nmax <= LU_NMAX, "cell system too large for the LU kernel");
+    const size_t smem = sizeof(z64) * 2 * (size_t)nmax;
+    // the same limit from every thread: a smaller one set in between would fail the other's launch
+    CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(z64) * 2 * LU_NMAX)));
     {
         ProfScope ps_("k_lu_solve", st);
-        k_lu_solve<<<nb * LU_CL, 256, smem, st>>>(zo.p, vo.p, nn.p, s, Z, V, d_info, scratch.p, nmax);
+        k_lu_solve<<<nb * LU_CL, 256, smem, st>>>(zo.p, vo.p, nn.p, s, Z, V, d_info, nmax);
         launched("k_lu_solve");
     }
     CBFM_CUDA(cudaStreamSynchronize(st));
