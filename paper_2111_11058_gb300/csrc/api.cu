@@ -661,15 +661,6 @@ cbfm_status cbfm_mesh(const double *verts, int64_t nv, const int32_t *tris, int6
         upload(dt, h.tris, st);
         upload(m->tri_vid, h.tris, st);
         upload(m->tri_edge, h.tri_edge, st);
-        {
-            // cell of each RWG of each triangle (edges are sorted by cell)
-            std::vector<int32_t> tc((size_t)3 * h.nt);
-            for (size_t k = 0; k < tc.size(); ++k) {
-                const int32_t e = h.tri_edge[k];
-                tc[k] = (int32_t)(std::upper_bound(h.cell_off.begin(), h.cell_off.end(), e) - h.cell_off.begin()) - 1;
-            }
-            upload(m->tri_cell, tc, st);
-        }
         upload(m->edge_tri, h.edge_tri, st);
         upload(m->edge_loc, h.edge_loc, st);
         std::vector<int32_t> ecell(h.ne);

@@ -49,7 +49,6 @@ struct Mesh : HandleBase {
     struct { double *p = nullptr; } far64, geo;
     DevBuf<int32_t> tri_vid;     // nt*3 vertex ids
     DevBuf<int32_t> tri_edge;    // nt*3 internal edge id
-    DevBuf<int32_t> tri_cell;    // nt*3 cell of each of the triangle's RWGs
     DevBuf<int32_t> edge_tri;    // ne*2
     DevBuf<int32_t> edge_loc;    // ne*2
     DevBuf<int32_t> edge_cell;   // ne, cell of each internal edge
@@ -130,7 +129,7 @@ void launch_farfield(const Mesh &m, const z64 *j, int nrhs, const double *d_obs,
 // assembly (k_assembly.cu): local blocks of all triangle pairs, then the RWG
 // matrices Z_op (op = Ks, Ta, Tb), row-major ne x ne, internal edge order.
 template <typename T>
-void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool lean, bool diag_cells = false);
+void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool lean);
 
 // dense complex linear algebra (k_dense.cu)
 struct GemmDesc {
@@ -202,12 +201,6 @@ bool wait_selftest(int kind, double limit_s, cudaStream_t st);
 void jacobi_svd_batched(int nb, int s, z64 *X, z64 *V, double *sig, int *d_info, cudaStream_t st,
                         double keep = 0.0);
 // In-place Gauss-Jordan inverse of an n x n FP64 complex matrix (row-major); info=1 on zero pivot.
-// local blocks and RWG operators of several meshes, one launch per stage (k_assembly.cu)
-// diag_cells: only triangle pairs that support RWGs of a common cell are
-// evaluated (the cells' diagonal blocks of Z); every other entry is zero
-template <typename T>
-void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
-                        bool diag_cells = false);
 // the RWG operators of several meshes as split-TF32 planes Zs[plane][op][i][f], row pitch tc_ldz(ne) floats (k_assembly.cu)
 void assemble_rwg_split(const std::vector<Mesh *> &ms, const std::vector<float *> &Zs, cudaStream_t st, bool lean);
 inline int64_t tc_ldz(int64_t ne) { return (2 * ne + 31) / 32 * 32; }

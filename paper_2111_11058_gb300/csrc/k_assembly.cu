@@ -592,7 +592,6 @@ struct AsmJob {
     const T *rec, *frec;
     const double *rec64, *geo;
     const int32_t *vid, *pairs, *edge_tri, *edge_loc;
-    const int32_t *tri_cell;   // non-null: evaluate only pairs of triangles that share a cell
     cx<T> *Zloc, *Z;
     float *Zs;                 // non-null (FP32): the RWG rows as hi/lo planes instead of Z, row pitch ldz floats
     int64_t ldz;
@@ -613,16 +612,6 @@ __device__ __forceinline__ int find_job(const AsmJob<T> *jobs, int njobs, int64_
         else hi = mid - 1;
     }
     return lo;
-}
-
-__device__ __forceinline__ bool share_cell(const int32_t *__restrict__ tc, int t, int s) {
-    const int a0 = tc[3 * t], a1 = tc[3 * t + 1], a2 = tc[3 * t + 2];
-    bool r = false;
-    for (int k = 0; k < 3; ++k) {
-        const int b = tc[3 * s + k];
-        r |= (b == a0) | (b == a1) | (b == a2);
-    }
-    return r;
 }
 
 // Near pairs of all meshes: two pairs per warp (the pairs of one warp may
@@ -653,7 +642,6 @@ __device__ __forceinline__ void near_loop(const AsmJob<T> *__restrict__ jobs, in
             const int64_t l = pid - J->near0;
             t = J->pairs[2 * l];
             s = J->pairs[2 * l + 1];
-            if (J->tri_cell && !share_cell(J->tri_cell, t, s)) t = s = -1;   // stays zero (written by the far stage)
         }
         cx<T> *blk = (J->nearblk && t >= 0) ? J->nearblk + (pid - J->near0) * NCOMP : nullptr;
         near_pair2<T, LEAN>(t, s, J->nt, J->rec64, J->md, J->mdt, J->rec, J->frec, J->geo, J->Zloc, sh.mom, sh.geo, blk);
@@ -791,14 +779,8 @@ __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
         {
             const AsmJob<T> &J = jobs[cj];
             const int s = cs0 + lane;
-            if (lane < ccnt && s >= ct) {
-                if (J.tri_cell && !share_cell(J.tri_cell, ct, s)) {
-                    const int64_t plane = (int64_t)J.nt * J.nt, base = (int64_t)ct * J.nt + s;
-                    for (int c = 0; c < NCOMP; ++c) J.Zloc[c * plane + base] = cx<T>(0, 0);
-                } else {
-                    far_pair(stage[b], J.nt, stage[b].trial[lane], J.rec64, J.vid, J.alpha, J.mdt, J.Zloc, ct, s);
-                }
-            }
+            if (lane < ccnt && s >= ct)
+                far_pair(stage[b], J.nt, stage[b].trial[lane], J.rec64, J.vid, J.alpha, J.mdt, J.Zloc, ct, s);
         }
         __syncwarp();   // the stage is restaged two items later
         if (!more) break;
@@ -969,26 +951,21 @@ void launch_tri_geo(Mesh &m, cudaStream_t st) {
 
 template <typename T>
 static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
-                           cudaStream_t st, bool lean, bool diag_cells);
-template <typename T>
-void assemble_rwg_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, cudaStream_t st, bool lean,
-                        bool diag_cells) {
-    assemble_batch<T>(ms, Z, {}, st, lean, diag_cells);
-}
+                           cudaStream_t st, bool lean);
 // The RWG operators as the split-TF32 planes of the tensor-core projection (k_tc.cu: row pitch tc_ldz).
 void assemble_rwg_split(const std::vector<Mesh *> &ms, const std::vector<float *> &Zs, cudaStream_t st, bool lean) {
-    assemble_batch<float>(ms, {}, Zs, st, lean, false);
+    assemble_batch<float>(ms, {}, Zs, st, lean);
 }
 
 // One mesh: the batched stages with a batch of one (one code path, so a
 // mesh assembled alone and in a batch gets the same bits).
 template <typename T>
-void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool lean, bool diag_cells) {
-    assemble_rwg_batch<T>(std::vector<Mesh *>{&m}, std::vector<cx<T> *>{Zrwg}, st, lean, diag_cells);
+void assemble_rwg(Mesh &m, cx<T> *Zrwg, cudaStream_t st, bool lean) {
+    assemble_batch<T>({&m}, {Zrwg}, {}, st, lean);
 }
 
-template void assemble_rwg<double>(Mesh &, z64 *, cudaStream_t, bool, bool);
-template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
+template void assemble_rwg<double>(Mesh &, z64 *, cudaStream_t, bool);
+template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool);
 // Local blocks, far/near pairs and RWG gather of several meshes, one launch
 // per stage.  The far stage's strip width (trial triangles per task) is
 // picked once per device and precision by timing the candidates, twice each,
@@ -1000,7 +977,7 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool, bool);
 // systems beyond SPREAD_ASM keep the general ones.
 template <typename T>
 static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,
-                           cudaStream_t st, bool lean, bool diag_cells) {
+                           cudaStream_t st, bool lean) {
     const int nj = (int)ms.size();
     if (nj == 0) return;
     std::vector<DevBuf<cx<T>>> Zloc(nj);
@@ -1021,7 +998,6 @@ static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T
         J.pairs = m.near_pairs.p;
         J.edge_tri = m.edge_tri.p;
         J.edge_loc = m.edge_loc.p;
-        J.tri_cell = diag_cells ? m.tri_cell.p : nullptr;
         J.Zloc = Zloc[k].p;
         J.Z = Z.empty() ? nullptr : Z[k];
         J.Zs = Zs.empty() ? nullptr : Zs[k];
@@ -1207,8 +1183,5 @@ template void near_blocks_compact_t<double>(const std::vector<Mesh *> &, const s
 void near_blocks_compact(const std::vector<Mesh *> &ms, const std::vector<c32 *> &out, cudaStream_t st, bool lean) {
     near_blocks_compact_t<float>(ms, out, st, lean);
 }
-
-template void assemble_rwg_batch<double>(const std::vector<Mesh *> &, const std::vector<z64 *> &, cudaStream_t, bool, bool);
-template void assemble_rwg_batch<float>(const std::vector<Mesh *> &, const std::vector<c32 *> &, cudaStream_t, bool, bool);
 
 }  // namespace cbfm
