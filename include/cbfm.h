@@ -347,8 +347,8 @@ cbfm_status cbfm_gram_inverse(const double *A, int64_t n, int32_t nbatch, double
  *   C = op(A) op(B) (+ C when accumulate), complex128 row-major, host or device;
  *   op(A) is M x K, op(B) K x N; op 0 = as stored, 1 = transposed, 2 =
  *   conjugate transposed, 3 = conjugated
- *   unit  0 = the form the library takes at these sizes, 1 = FP64 units,
- *         2 = tensor cores (operands cut into exact digits)
+ *   unit  0 = the form the block solver's basis takes at these sizes, 1 = FP64
+ *         units, 2 = tensor cores (operands cut into exact digits)
  * Returns CBFM_EINVAL on bad arguments.
  */
 cbfm_status cbfm_matmul_f64(const double *A, const double *B, double *C, int64_t M, int64_t N, int64_t K, int32_t opA,

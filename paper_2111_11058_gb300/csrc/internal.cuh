@@ -66,25 +66,30 @@ struct Cbf : HandleBase {
     std::vector<int64_t> coff;    // CBF offsets per cell (ncell+1), within one half
     std::vector<int64_t> boff;    // block offsets sum N_m L_m (ncell+1)
     int64_t nhalf = 0;            // sum L_m
-    double spread = 0.0;          // largest over smallest modulus on the diagonal of G^CBF (the CBFs' singular values)
+    // largest over smallest modulus on the diagonal of G^CBF.  For dual CBFs (cbfm_build_cbfs, cbfm_build_ipcbfs) these are
+    // their singular values; for imported blocks it is that diagonal and no more (random blocks: the smallest of
+    // several hundred moduli decides; C^M = C^J: the diagonal is zero and the spread infinite)
+    double spread = 0.0;
     DevBuf<z64> CM, CJ;           // blocks N_m x L_m row-major, cells in order
     DevBuf<c32> CM32, CJ32;
 };
 
-// Spread of the CBFs' singular values up to which a mixed-precision block solve takes
-// the faster forms that change the last bits of its basis.  With tiny triangles beside
-// large ones (1.4e4 to 1e5 on spheroids and cylinders with pole triangles; 1e3 to 1e4 on
-// cubes, spheres and even cylinders) the FP32 operator's rounding, which follows those
-// bits, moves the currents by up to 1e-5 of their norm and 1e-3 of their rms at single
-// edges; of 446 drawn solves below 1e4 three moved by more than 2e-5 (8e-5), all above
-// 2.1e3, and below this line none by more than 1.2e-5.  The others keep one order of
-// operations, so that their results stay reproducible.
+// Spread (Cbf::spread) up to which a mixed-precision block solve takes its basis on the tensor cores.  The line bounds
+// the change against the form with the FP64 units' sums, not the error: the FP32 operator's rounding follows the basis'
+// last bits, and with tiny triangles beside large ones (spread 1.4e4 to 1e5 on spheroids and cylinders with pole
+// triangles; 1e3 to 1e4 on cubes, spheres and even cylinders) the currents then move by up to 1e-5 of their norm; of
+// 446 drawn solves below 1e4 three moved by more than 2e-5 (8e-5), all above 2.1e3, and below this line none by more
+// than 1.2e-5.  Against 64 bits both forms are alike on either side of it (57 generated CBF sets, spread 77 to
+// 7e4, dense FP64 solutions: errors of the currents 1.00 times, above 2e3 0.99 times those of the FP64 sums), and both
+// repeat themselves exactly.
 constexpr double SPREAD_MAX = 2e3;
-// The same for the assembly's shorter forms (near pairs' closed forms, barycentric far pairs): their entries
-// round differently (1.4e-7 of the matrix).  CBFs kept to sigma / sigma_1 >= 1e-3 spread over 1e3, and
-// currents on coarse meshes carry such a difference up to 300 times (69 solves drawn from spheres, cubes,
-// cylinders and spheroids: 4.4e-5 of the currents' norm with these forms everywhere, 2.3e-5 with the near
-// pairs' alone; with a line at 800 still 7.4e-5 on a sphere a tenth of a wavelength across).
+// The same for the unfused mixed assembly's shorter entry forms (near pairs' closed forms, barycentric far pairs): their
+// entries round differently (1.4e-7 of the matrix), which currents on coarse meshes carry up to 300 times (69
+// drawn solves: 4.4e-5 of the currents' norm with these forms everywhere, 2.3e-5 with the near pairs' alone; with a line at
+// 800 still 7.4e-5 on a sphere a tenth of a wavelength across).  CBFs kept to sigma / sigma_1 >= 1e-3 spread over 1e3, so
+// generated sets take the general forms.  Against 64 bits the forms are alike here too (the same 57 sets: errors
+// of A 0.99, of the currents 1.00 times the general forms').  The fused form (k_fused.cu) and FP64 have the shorter
+// forms alone, whatever the spread.
 constexpr double SPREAD_ASM = 300.0;
 
 struct Red : HandleBase {

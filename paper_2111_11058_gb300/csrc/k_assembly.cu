@@ -973,7 +973,7 @@ template void assemble_rwg<float>(Mesh &, c32 *, cudaStream_t, bool);
 // is not run again afterwards).  lean: the near pairs' closed forms with the
 // short elementary functions (near pairs of the 9216-unknown cube 1.73 -> 0.89 ms
 // by themselves) and the far pairs in barycentric moments (far_bary.cuh); the conventional MoM, whose
-// long restarted solves carry a last bit of Z into the currents, and mixed
+// long restarted solves carry a last bit of Z into the currents, and unfused mixed
 // systems beyond SPREAD_ASM keep the general ones.
 template <typename T>
 static void assemble_batch(const std::vector<Mesh *> &ms, const std::vector<cx<T> *> &Z, const std::vector<float *> &Zs,

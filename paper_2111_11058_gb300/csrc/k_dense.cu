@@ -495,6 +495,8 @@ constexpr int LU_CL = 8, LU_NMAX = 4096;
 // FP64 products with the rounding written out, in this and the next kernel: the CBFs they
 // give decide, through solves that amplify a last bit, the digits of every later result, so
 // their operations do not follow the compiler's choice of which product of a sum is fused.
+// The two products differ only in the imaginary part's rounding: mul_rn for the multipliers and
+// updates of the LU, mul2_rn for its scaling by the pivots and for the rotations of the SVD.
 __device__ __forceinline__ double norm2_rn(z64 a) { return __fma_rn(a.re, a.re, __dmul_rn(a.im, a.im)); }
 __device__ __forceinline__ z64 mul_rn(z64 a, z64 b) {   // Im: Im a Re b fused
     return z64(__fma_rn(a.re, b.re, -__dmul_rn(a.im, b.im)), __fma_rn(a.im, b.re, __dmul_rn(a.re, b.im)));

@@ -45,6 +45,11 @@
 // a pair on two lanes, one medium each (16 warps of 128 registers), 34 ms, and 20
 // warps of 96, 38 ms; both orbits unrolled, 33 ms.
 //
+// Entries: barycentric far pairs and the near pairs' short closed forms, whatever the CBFs' spread (SPREAD_ASM rules
+// the unfused form only).  17 generated CBF sets (spread 40 to 1.9e3) against 64 bits: A 0.57 times, the RCS 0.87 times
+// and the currents 1.00 times the errors of the earlier kernel with the general quadrature; A 0.4 to 0.8 times those
+// of the unfused form.
+//
 // Triangle pairs whose triangles carry RWGs of several cells are evaluated once
 // per cell pair they feed (about 1.15 x per side on the RCB cells used here).
 //
@@ -922,6 +927,11 @@ void fused_launch(std::vector<FusedJob> &jobs, const std::vector<std::pair<doubl
 
 }  // namespace
 
+// Size of the unfused form, as bytes of its local blocks, RWG operators (complex64 and as split planes) and Y^T.  The
+// complex64 operators are no longer formed (the gather writes the planes), but the line that mixed_takes_fused draws with
+// this sum lies where the fused form is the faster one already: cube of 6912 triangles, just above it, 15.2 ms fused
+// and 26.9 unfused for L = 8 (17.3 and 27.1 for 14, 33.4 and 32.8 for 20), spheroid of 6960 16.5 and 35.4; cube of 3072,
+// below it, 4.6 and 3.1.
 double unfused_scratch_bytes(const Mesh &m, const Cbf &c) {
     const double nt = (double)m.h.nt, ne = (double)m.h.ne, nh = (double)c.nhalf;
     const double ldz = std::ceil(2.0 * ne / 32.0) * 32.0;

@@ -17,6 +17,9 @@
 // i + j >= 7 are left out, so an entry of the product is off by about
 // 2^-56 max|a_k| max|b_k| sqrt(K) (a random walk), against sqrt(K) times the
 // rms of a_k b_k times 2^-53 sqrt(K) / 4 from the roundings of a sum in FP64.
+// Rows and columns of the like size throughout lose nothing by this; where the entries of a row differ by orders of
+// magnitude and meet small ones of the column, FP64 sums are the better (operators of FP64 systems, cell blocks of Z,
+// everything in the long restarted solves without the CMP: OzHold, internal.cuh).
 // All sums in between are integers and exact: a digit pair's product is at most
 // 2^14, at most 7 pairs x 128 values of k meet in one accumulator (< 2^24),
 // and every 128 values of k the accumulators are drained into two 64-bit
