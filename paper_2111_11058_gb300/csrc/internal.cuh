@@ -79,8 +79,8 @@ struct Cbf : HandleBase {
 // last bits, and with tiny triangles beside large ones (spread 1.4e4 to 1e5 on spheroids and cylinders with pole
 // triangles; 1e3 to 1e4 on cubes, spheres and even cylinders) the currents then move by up to 1e-5 of their norm; of
 // 446 drawn solves below 1e4 three moved by more than 2e-5 (8e-5), all above 2.1e3, and below this line none by more
-// than 1.2e-5.  Against 64 bits both forms are alike on either side of it (57 generated CBF sets, spread 77 to
-// 7e4, dense FP64 solutions: errors of the currents 1.00 times, above 2e3 0.99 times those of the FP64 sums), and both
+// than 1.2e-5.  Against 64 bits both forms are alike on either side of it (57 generated CBF sets, spread 33 to
+// 2.3e5, dense FP64 solutions: errors of the currents 1.00 times, above 2e3 0.99 times those of the FP64 sums), and both
 // repeat themselves exactly.
 constexpr double SPREAD_MAX = 2e3;
 // The same for the unfused mixed assembly's shorter entry forms (near pairs' closed forms, barycentric far pairs): their

@@ -708,10 +708,12 @@ int64_t far_tasks(const AsmJob<T> &J) {
 // flight; FP64: four blocks of two warps, where the wider accumulators would
 // otherwise spill.
 //
-// FP32 form with npairs > 0: the near pairs' closed forms are bound by the FP64
+// Shorter FP32 forms with npairs > 0: the near pairs' closed forms are bound by the FP64
 // pipes and the far pairs by the FP32 ones, so the launch does both.  The first
 // near_ctas blocks (two of an SM's three) begin with the near pairs, the others
-// with the far ones, and each goes over to what is left of the other kind.
+// with the far ones, and each goes over to what is left of the other kind.  The
+// general form holds no near pairs: compiled in, their unused code cost its far
+// pairs 5 to 25 % (2304-unknown cube 110 against 88 us, 9216 unknowns 1.29 against 1.21 ms).
 template <typename T, bool LEAN>
 __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
     k_far(const AsmJob<T> *__restrict__ jobs, int njobs, int64_t ntasks, unsigned long long *__restrict__ counter,
@@ -750,7 +752,7 @@ __global__ void __launch_bounds__(32 * far_warps<T>(), sizeof(T) == 4 ? 3 : 4)
     const bool near_first = (int)blockIdx.x < near_ctas;
     for (int phase = 0; phase < 2; ++phase) {
     if ((phase == 0) == near_first) {
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (sizeof(T) == 4 && LEAN) {
             static_assert(sizeof(NearShared<T>) <= 2 * sizeof(Stage), "a warp's far stages hold its near scratch");
             if (npairs > 0) {
                 __syncwarp();
