@@ -648,6 +648,56 @@ __global__ void __launch_bounds__(32 * MO_R) k_matvec64_ord(int64_t n, int nrhs,
     if (mine && c0 + row < n) reinterpret_cast<double *>(out + (r0 + q) * n + c0 + row)[c] = acc;
 }
 
+// The same sums in tiles of 32 right-hand sides x 16 output rows, four outputs a thread: a CTA's four warps keep its SM's
+// FP64 pipe full (1024 clocks a value of k), where the kernel above spends issue slots on the operands of two
+// multiply-adds a lane and reaches 0.57 of the pipe.  For many right-hand sides: product of n = 2304 and 64 of them
+// 2.4 ms against 3.9, 128 4.7 against 7.5; with few, whole tiles are padding (n = 960, 24: 0.60 against 0.32).
+constexpr int MT_R = 32, MT_K = 32;
+__global__ void __launch_bounds__(128) k_matvec64_tile(int64_t n, int nrhs, const z64 *__restrict__ M,
+                                                       const z64 *__restrict__ in, z64 *__restrict__ out,
+                                                       const int *__restrict__ done) {
+    __shared__ z64 Xs[MT_K][MT_R + 1];
+    __shared__ z64 Ms[MT_K][MV_N + 1];
+    const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
+    const int64_t r0 = (int64_t)blockIdx.y * MT_R, c0 = (int64_t)blockIdx.x * MV_N;
+    bool any = false;
+    for (int a = 0; a < MT_R; ++a) any |= r0 + a < nrhs && (!done || done[r0 + a] == 0);
+    if (!any) return;
+    z64 acc[2][2];
+    for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b) acc[a][b] = z64(0, 0);
+    for (int64_t k0 = 0; k0 < n; k0 += MT_K) {
+        for (int e = tid; e < (MT_R + MV_N) * MT_K; e += 128) {
+            const int row = e / MT_K, kk = e % MT_K;
+            const int64_t kx = k0 + kk, r = r0 + row, c = c0 + row - MT_R;
+            if (row < MT_R) Xs[kk][row] = r < nrhs && kx < n ? in[r * n + kx] : z64(0, 0);
+            else Ms[kk][row - MT_R] = c < n && kx < n ? M[c * n + kx] : z64(0, 0);
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int kk = 0; kk < MT_K; ++kk) {
+            const z64 x[2] = {Xs[kk][ty], Xs[kk][ty + 16]}, m[2] = {Ms[kk][tx], Ms[kk][tx + 8]};
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    z64 &o = acc[a][b];
+                    o.re = fma(x[a].im, -m[b].im, fma(x[a].re, m[b].re, o.re));
+                    o.im = fma(x[a].im, m[b].re, fma(x[a].re, m[b].im, o.im));
+                }
+        }
+        __syncthreads();
+    }
+    for (int a = 0; a < 2; ++a) {
+        const int64_t r = r0 + ty + 16 * a;
+        if (r >= nrhs || (done && done[r] != 0)) continue;
+        for (int b = 0; b < 2; ++b) {
+            const int64_t c = c0 + tx + 8 * b;
+            if (c < n) out[r * n + c] = acc[a][b];
+        }
+    }
+}
+
 // ------------------------------------------------- whole cycle on a cluster
 // The Arnoldi cycle of few right-hand sides of moderate order in one launch: a
 // cluster of CC CTAs per right-hand side.  As separate kernels an iteration is
@@ -1007,6 +1057,14 @@ static void apply_rows(int64_t n, const z64 *M64, const c32 *M32, const z64 *in,
         if (nrhs <= 8) k_matvec32<8><<<dim3(gx, (unsigned)((nrhs + 7) / 8)), 128, 0, st>>>(n, nrhs, M32, in32, out, done);
         else k_matvec32<32><<<dim3(gx, (unsigned)((nrhs + 31) / 32)), 256, 0, st>>>(n, nrhs, M32, in32, out, done);
     } else if (ord) {
+        // tiles where their waves (n x 1024 clocks each) beat the row kernel's n^2 nrhs x 3.5 / SMs clocks
+        const int64_t gx = (n + MV_N - 1) / MV_N, gt = (nrhs + MT_R - 1) / MT_R;
+        const int64_t waves = (gx * gt + sm_count() - 1) / sm_count();
+        if (1024.0 * waves * sm_count() < 3.5 * (double)n * nrhs) {
+            k_matvec64_tile<<<dim3((unsigned)gx, (unsigned)gt), 128, 0, st>>>(n, nrhs, M64, in, out, done);
+            launched("k_matvec");
+            return;
+        }
         const dim3 g((unsigned)((n + MV_N - 1) / MV_N), (unsigned)((nrhs + MO_R - 1) / MO_R));
         k_matvec64_ord<<<g, 32 * MO_R, 0, st>>>(n, nrhs, M64, in, out, done);
     } else {
