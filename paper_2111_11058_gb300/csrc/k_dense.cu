@@ -478,7 +478,7 @@ void gemm_dir(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z
 
 // ------------------------------------------------------ batched LU solve
 // Gaussian elimination with partial pivoting on [Z | V], then backward
-// substitution.  One cluster of LU_CL CTAs per system, the columns of Z and V in
+// substitution.  One cluster of CL CTAs per system, the columns of Z and V in
 // blocks of eight dealt to the CTAs: a step's pivot, row exchange and
 // multipliers need only column k, which every CTA reads (through L2) and works
 // through by itself, so a step takes one cluster synchronisation, and the
@@ -490,7 +490,16 @@ void gemm_dir(const GemmDesc &d, int opA, int opB, const z64 *A, const z64 *B, z
 // column through L2, the pivot search, one division).  col, dinv: n entries each
 // per CTA in shared memory (n <= LU_NMAX, the largest cell system the CBF generation
 // takes).  info[b] = 1: singular; 2: a cluster synchronisation expired.
-constexpr int LU_CL = 8, LU_NMAX = 4096;
+constexpr int LU_NMAX = 4096;
+// CTAs per system: eight while the clusters of all systems (four CTAs to an SM) are resident at once, fewer for more
+// systems, whose steps then wait for work and not for one another.  With s = 6 and 128 right-hand sides, 8 / 4 / 2 / 1
+// CTAs: 40 systems of 64 RWGs 1.80 / 1.85 / 2.02 / 2.70 and 2.53 / 3.23 / 4.27 / 7.82 ms; 100 of 25 0.62 / 0.38 / 0.42 /
+// 0.35 and 1.00 / 0.74 / 0.99 / 1.10; 160 of 28 0.84 / 0.56 / 0.55 / 0.54 and 1.48 / 1.32 / 1.54 / 1.99; 300 of 15
+// 0.65 / 0.36 / 0.22 / 0.18 and 1.02 / 0.79 / 0.62 / 0.66.
+inline int lu_ctas(int nb) {
+    const int resident = 17 * sm_count() / 4;
+    return 8 * nb <= resident ? 8 : 4 * nb <= resident ? 4 : nb <= 4 * sm_count() ? 2 : 1;
+}
 
 // FP64 products with the rounding written out, in this and the next kernel: the CBFs they
 // give decide, through solves that amplify a last bit, the digits of every later result, so
@@ -515,12 +524,12 @@ __device__ __forceinline__ z64 ldcg64(const z64 *p) {
     return z64(v.x, v.y);
 }
 
-__global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
+template <int CL>
+__global__ void __launch_bounds__(256)
     k_lu_solve(const int64_t *__restrict__ zoff, const int64_t *__restrict__ voff, const int *__restrict__ nsz, int s,
                z64 *__restrict__ Zall, z64 *__restrict__ Vall, int *__restrict__ info, int nmax) {
     extern __shared__ __align__(16) unsigned char lu_raw[];
-    cg::cluster_group cl = cg::this_cluster();
-    const int me = (int)cl.block_rank(), b = blockIdx.x / LU_CL;
+    const int me = (int)(blockIdx.x % CL), b = blockIdx.x / CL;
     const int n = nsz[b];
     z64 *Z = Zall + zoff[b];
     z64 *V = Vall + voff[b];
@@ -533,11 +542,11 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
     const int c8 = tid & 7, r32 = tid >> 3;   // column within a block of eight, row within 32
     const int nbz = (n + 7) >> 3, nbv = (s + 7) >> 3;
     if (tid == 0) {
-        cl_bar_init(cbar, LU_CL);
+        if (CL > 1) cl_bar_init(cbar, CL);
         s_abort = 0;
     }
     __syncthreads();
-    cl.sync();   // barriers initialised in every CTA (unconditional)
+    if constexpr (CL > 1) cg::this_cluster().sync();   // barriers initialised in every CTA (unconditional)
     bool ok = true;
     for (int k = 0; k < n && ok; ++k) {
         for (int i = k + tid; i < n; i += blockDim.x) col[i] = ldcg64(Z + (int64_t)i * n + k);
@@ -576,7 +585,7 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
         for (int i = k + 1 + tid; i < n; i += blockDim.x) col[i] = mul_rn(col[i], pinv);
         // row exchange in this CTA's columns (of column k only the diagonal is used again)
         if (p != k) {
-            for (int jb = me + LU_CL * r32; jb < nbz; jb += LU_CL * 32) {
+            for (int jb = me + CL * r32; jb < nbz; jb += CL * 32) {
                 const int j = 8 * jb + c8;
                 if (j > k && j < n) {
                     z64 t = Z[(int64_t)k * n + j];
@@ -584,7 +593,7 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
                     Z[(int64_t)p * n + j] = t;
                 }
             }
-            for (int jb = me + LU_CL * r32; jb < nbv; jb += LU_CL * 32) {
+            for (int jb = me + CL * r32; jb < nbv; jb += CL * 32) {
                 const int j = 8 * jb + c8;
                 if (j < s) {
                     z64 t = V[(int64_t)k * s + j];
@@ -596,7 +605,7 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
         __syncthreads();
         if (tid == 0) dinv[k] = pinv;
         // eliminate below
-        for (int jb = me + LU_CL * ((((k + 1) >> 3) + LU_CL - 1 - me) / LU_CL); jb < nbz; jb += LU_CL) {
+        for (int jb = me + CL * ((((k + 1) >> 3) + CL - 1 - me) / CL); jb < nbz; jb += CL) {
             const int j = 8 * jb + c8;
             if (j <= k || j >= n) continue;
             const z64 u = Z[(int64_t)k * n + j];
@@ -606,7 +615,7 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
                 z = sub_rn(z, mul_rn(col[i], u));
             }
         }
-        for (int jb = me; jb < nbv; jb += LU_CL) {
+        for (int jb = me; jb < nbv; jb += CL) {
             const int j = 8 * jb + c8;
             if (j >= s) continue;
             const z64 u = V[(int64_t)k * s + j];
@@ -616,18 +625,19 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
                 v = sub_rn(v, mul_rn(col[i], u));
             }
         }
-        ok = cl_sync(cbar, k, LU_CL, &s_abort, info + b);
+        if constexpr (CL > 1) ok = cl_sync(cbar, k, CL, &s_abort, info + b);
+        else __syncthreads();
     }
     // backward substitution, column oriented, on this CTA's right-hand sides
     for (int k = n - 1; k >= 0 && ok; --k) {
         for (int i = tid; i < k; i += blockDim.x) col[i] = ldcg64(Z + (int64_t)i * n + k);
         const z64 di = dinv[k];
-        for (int jb = me + LU_CL * r32; jb < nbv; jb += LU_CL * 32) {
+        for (int jb = me + CL * r32; jb < nbv; jb += CL * 32) {
             const int j = 8 * jb + c8;
             if (j < s) V[(int64_t)k * s + j] = mul2_rn(V[(int64_t)k * s + j], di);
         }
         __syncthreads();
-        for (int jb = me; jb < nbv; jb += LU_CL) {
+        for (int jb = me; jb < nbv; jb += CL) {
             const int j = 8 * jb + c8;
             if (j >= s) continue;
             const z64 u = V[(int64_t)k * s + j];
@@ -640,7 +650,7 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
         __syncthreads();
     }
     if (!ok && tid == 0) atomicExch(info + b, 2);
-    cl.sync();   // no CTA leaves while another may still arrive on its barriers
+    if constexpr (CL > 1) cg::this_cluster().sync();   // no CTA leaves while another may still arrive on its barriers
 }
 
 // ---------------------------------------------- one-sided Jacobi SVD
@@ -660,15 +670,17 @@ __global__ void __cluster_dims__(LU_CL, 1, 1) __launch_bounds__(256)
 // A round of a CTA's eight pairs: each warp forms the products of its pair, the
 // first warp works out all eight rotations side by side (the chain of square roots
 // and divisions, about 150 FP64 instructions, costs as much as the vector work when
-// every warp issues it for one pair), each warp rotates its columns.  HELD
-// (s <= 32 JS_E): the columns stay in registers between the two, and those of V are
-// loaded before the rotation is known.  Bound: the FP64 pipes (16 matrices of
+// every warp issues it for one pair), each warp rotates its columns.  E > 0
+// (s <= 32 E): the columns stay in registers between the two, and those of V are
+// loaded before the rotation is known; E no larger than s needs, since its registers
+// decide how many clusters are resident (100 matrices of s = 24: 6.1 ms for E = 1, 8.7
+// for 4; of s = 6: 0.49 and 0.74).  Bound: the FP64 pipes (16 matrices of
 // s = 128: 46 -> 36 ms; FP64 pipe 57 % active).
-constexpr int JS_CL = 8, JS_E = 4;
+constexpr int JS_CL = 8;
 
 __device__ __forceinline__ double norm2d(double2 a) { return a.x * a.x + a.y * a.y; }
 
-template <bool HELD>
+template <int E>
 __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
     k_jacobi_svd(int s, z64 *__restrict__ Xall, z64 *__restrict__ Vall, double *__restrict__ sig,
                  int *__restrict__ info, double tol, double keep) {
@@ -733,7 +745,7 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
                 const bool pair = pr < n2 / 2 && j < s;   // j == s: dummy column of odd sizes
                 z64 *xi = X + (int64_t)i * s, *xj = X + (int64_t)j * s;
                 z64 *vi = V + (int64_t)i * s, *vj = V + (int64_t)j * s;
-                z64 xu[JS_E], xv[JS_E], wu[JS_E], wv[JS_E];
+                z64 xu[E + (E == 0)], xv[E + (E == 0)], wu[E + (E == 0)], wv[E + (E == 0)];
                 double al = 0, be = 0;
                 z64 ga(0, 0);
                 auto add = [&](z64 u, z64 v) {
@@ -743,9 +755,9 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
                     ga.im = __fma_rn(-u.im, v.re, __fma_rn(u.re, v.im, ga.im));
                 };
                 if (pair) {
-                    if constexpr (HELD) {
+                    if constexpr (E > 0) {
 #pragma unroll
-                        for (int e = 0; e < JS_E; ++e) {
+                        for (int e = 0; e < E; ++e) {
                             const int r = lane + 32 * e;
                             if (r < s) {
                                 xu[e] = ldcg64(xi + r);
@@ -753,7 +765,7 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
                             }
                         }
 #pragma unroll
-                        for (int e = 0; e < JS_E; ++e) {
+                        for (int e = 0; e < E; ++e) {
                             const int r = lane + 32 * e;
                             if (r < s) {
                                 wu[e] = ldcg64(vi + r);
@@ -761,7 +773,7 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
                             }
                         }
 #pragma unroll
-                        for (int e = 0; e < JS_E; ++e) {
+                        for (int e = 0; e < E; ++e) {
                             if (lane + 32 * e < s) add(xu[e], xv[e]);
                         }
                     } else {
@@ -814,9 +826,9 @@ __global__ void __cluster_dims__(JS_CL, 1, 1) __launch_bounds__(256)
                     *pu = z64(__fma_rn(c, u.re, -a_.re), __fma_rn(c, u.im, -a_.im));
                     *pv = z64(__fma_rn(c, v.re, b_.re), __fma_rn(c, v.im, b_.im));
                 };
-                if constexpr (HELD) {
+                if constexpr (E > 0) {
 #pragma unroll
-                    for (int e = 0; e < JS_E; ++e) {
+                    for (int e = 0; e < E; ++e) {
                         const int r = lane + 32 * e;
                         if (r < s) {
                             turn(xu[e], xv[e], xi + r, xj + r);
@@ -1779,13 +1791,30 @@ void lu_solve_batched(int nb, const int64_t *h_zoff, const int64_t *h_voff, cons
     for (int k = 0; k < nb; ++k) nmax = std::max(nmax, h_n[k]);
     CBFM_REQUIRE(nmax <= LU_NMAX, "cell system too large for the LU kernel");
     const size_t smem = sizeof(z64) * 2 * (size_t)nmax;
-    // the same limit from every thread: a smaller one set in between would fail the other's launch
-    CBFM_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(z64) * 2 * LU_NMAX)));
-    {
+    auto run = [&](auto *f, int cl) {
+        // the same limit from every thread: a smaller one set in between would fail the other's launch
+        CBFM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(z64) * 2 * LU_NMAX)));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(nb * cl), 1, 1);
+        cfg.blockDim = dim3(256, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cl;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
         ProfScope ps_("k_lu_solve", st);
-        k_lu_solve<<<nb * LU_CL, 256, smem, st>>>(zo.p, vo.p, nn.p, s, Z, V, d_info, nmax);
+        CBFM_CUDA(cudaLaunchKernelEx(&cfg, f, (const int64_t *)zo.p, (const int64_t *)vo.p, (const int *)nn.p, s, Z, V, d_info, nmax));
         launched("k_lu_solve");
-    }
+    };
+    const int cl = lu_ctas(nb);
+    if (cl == 8) run(k_lu_solve<8>, 8);
+    else if (cl == 4) run(k_lu_solve<4>, 4);
+    else if (cl == 2) run(k_lu_solve<2>, 2);
+    else run(k_lu_solve<1>, 1);
     CBFM_CUDA(cudaStreamSynchronize(st));
 }
 
@@ -1794,8 +1823,8 @@ void jacobi_svd_batched(int nb, int s, z64 *X, z64 *V, double *sig, int *d_info,
     {
         ProfScope ps_("k_jacobi_svd", st);
         const double tol = 1e-15 * (s > 8 ? s : 8);
-        if (s <= 32 * JS_E) k_jacobi_svd<true><<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, tol, keep);
-        else k_jacobi_svd<false><<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, tol, keep);
+        auto *f = s <= 32 ? k_jacobi_svd<1> : s <= 64 ? k_jacobi_svd<2> : s <= 128 ? k_jacobi_svd<4> : k_jacobi_svd<0>;
+        f<<<nb * JS_CL, 256, 0, st>>>(s, X, V, sig, d_info, tol, keep);
         launched("k_jacobi_svd");
     }
 }
