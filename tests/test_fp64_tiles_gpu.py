@@ -22,7 +22,7 @@ def P():
     return pkg
 
 
-# n = 60 and 972, not multiples of 16 or 32; 33, 64 and 100 right-hand sides: ragged tiles, full ones, several waves
+# n = 60, 324 and 900, not multiples of 16 or 32 but the last takes the tiles: full ones, ragged ones and two waves
 @pytest.mark.parametrize("shape,nrhs", [("ico0", 100), ("cube3", 33), ("cube3", 100), ("cube5", 64), ("cube5", 100)])
 def test_same_bits_alone_and_among_many(P, shape, nrhs):
     n = int(shape[-1])
