@@ -235,9 +235,9 @@ __global__ void k_gram_times_c(int64_t ne, int64_t nh, const int32_t *__restrict
 // |(C^J_l)^H Gf C^M_l| of every CBF l over the RWG functions of its own cell, the modulus of the diagonal of G^CBF, to
 // FP32 accuracy.  One block per 32 CBFs of a cell (blocks (c, i) past the cell's CBFs leave): lanes over the CBFs, so
 // that the coefficients are read in whole rows, five rows of Gf at a time per warp, their 30 entries converted by
-// 30 lanes and handed round.  Bound: latency of two dependent loads per five rows (import of
-// 12 CBFs on one cell of 450 RWGs 82 us, on two of 576 87 us; 104 and 118 us with a warp per CBF and FP64 sums, whose
-// few blocks held one FP64 pipe each; 50 us without this stage).
+// 30 lanes and handed round.  Bound: latency of two dependent loads per five rows (the whole
+// query, 12 CBFs on one cell of 450 RWGs 32 us, on two of 576 35 us; 54 and 66 us with a warp per CBF and FP64 sums,
+// whose few blocks held one FP64 pipe each).
 // tab: cell offsets, CBF offsets, block offsets (nc + 1 each) and L (nc).
 constexpr int CD_WARPS = 32;
 __global__ void __launch_bounds__(32 * CD_WARPS)
@@ -397,31 +397,6 @@ void cbf_make32(Cbf &c, cudaStream_t st) {
     launch_z64_to_c32(c.CJ.p, c.CJ32.p, tot, st);
 }
 
-// c.spread: largest over smallest modulus on the diagonal of G^CBF (waits for the stream)
-void cbf_spread(Cbf &c, cudaStream_t st) {
-    const Mesh &m = *c.mesh;
-    const int nc = m.h.ncell;
-    std::vector<int64_t> tab(m.h.cell_off.begin(), m.h.cell_off.end());
-    tab.insert(tab.end(), c.coff.begin(), c.coff.end());
-    tab.insert(tab.end(), c.boff.begin(), c.boff.end());
-    tab.insert(tab.end(), c.L.begin(), c.L.end());
-    DevBuf<int64_t> buf;   // the table, then the result
-    buf.alloc(tab.size() + c.nhalf);
-    CBFM_CUDA(cudaMemcpyAsync(buf.p, tab.data(), sizeof(int64_t) * tab.size(), cudaMemcpyHostToDevice, st));
-    float *g = reinterpret_cast<float *>(buf.p + tab.size());
-    const int lmax = *std::max_element(c.L.begin(), c.L.end());
-    k_cbf_diag<<<dim3((unsigned)nc, (unsigned)((lmax + 31) / 32)), 32 * CD_WARPS, 0, st>>>(nc, buf.p, m.gram_val.p, m.gram_col.p,
-                                                                                      c.CM32.p, c.CJ32.p, g);
-    launched("k_cbf_diag");
-    std::vector<float> h(c.nhalf);
-    CBFM_CUDA(cudaMemcpyAsync(h.data(), g, sizeof(float) * c.nhalf, cudaMemcpyDeviceToHost, st));
-    CBFM_CUDA(cudaStreamSynchronize(st));
-    const auto mm = std::minmax_element(h.begin(), h.end());
-    c.spread = *mm.first > 0.f ? (double)*mm.second / *mm.first : INFINITY;
-    for (float v : h)
-        if (!(v <= *mm.second)) c.spread = INFINITY;   // a NaN among them
-}
-
 // Steps after the coefficient sets (paper Eqs. (gram_CBF), (gram_CBF_SVD), (CBF)): G'_m = (J^M)^H G_m J^J,
 // SVD, truncation sigma_i / sigma_1 >= delta_svd (at most lmax when > 0), C^M = J^M U_L, C^J = J^J V_L.
 // Vm holds, per cell, [J^M; J^J] (2 N_m x s, row-major) at voff[c].
@@ -544,7 +519,6 @@ std::unique_ptr<Cbf> dual_cbfs(Mesh *m, int s, const z64 *Vm, const std::vector<
     gemm_grouped<double>(gm, 0, 0, Vm, UL.p, cb->CM.p, false, st);
     gemm_grouped<double>(gj, 0, 0, Vm, VL.p, cb->CJ.p, false, st);
     cbf_make32(*cb, st);
-    cbf_spread(*cb, st);
     return cb;
 }
 
@@ -886,7 +860,7 @@ cbfm_status cbfm_cbf_import(cbfm_mesh_t mesh, const int32_t *L_per_cell, const d
         copy_in(cb->CM.p, CM, tot * sizeof(z64), st);
         copy_in(cb->CJ.p, CJ, tot * sizeof(z64), st);
         cbf_make32(*cb, st);
-        cbf_spread(*cb, st);
+        CBFM_CUDA(cudaStreamSynchronize(st));
         *out = (cbfm_cbf_t)cb.release();
     });
 }
@@ -904,6 +878,39 @@ cbfm_status cbfm_cbf_export(cbfm_cbf_t cbf, double *CM, double *CJ, void *stream
 }
 
 }  // extern "C"
+
+namespace cbfm {
+
+// c.spread: largest over smallest modulus on the diagonal of G^CBF.  Asked for by the calls that choose by it, not at
+// import or generation: it costs 30 us, half of an import, which FP64 and fused systems do not need.
+double cbf_spread(Cbf &c, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(c.spread_mu);
+    if (c.spread >= 0.0) return c.spread;
+    const Mesh &m = *c.mesh;
+    const int nc = m.h.ncell;
+    std::vector<int64_t> tab(m.h.cell_off.begin(), m.h.cell_off.end());
+    tab.insert(tab.end(), c.coff.begin(), c.coff.end());
+    tab.insert(tab.end(), c.boff.begin(), c.boff.end());
+    tab.insert(tab.end(), c.L.begin(), c.L.end());
+    DevBuf<int64_t> buf;   // the table, then the result
+    buf.alloc(tab.size() + c.nhalf);
+    CBFM_CUDA(cudaMemcpyAsync(buf.p, tab.data(), sizeof(int64_t) * tab.size(), cudaMemcpyHostToDevice, st));
+    float *g = reinterpret_cast<float *>(buf.p + tab.size());
+    const int lmax = *std::max_element(c.L.begin(), c.L.end());
+    k_cbf_diag<<<dim3((unsigned)nc, (unsigned)((lmax + 31) / 32)), 32 * CD_WARPS, 0, st>>>(nc, buf.p, m.gram_val.p, m.gram_col.p,
+                                                                                      c.CM32.p, c.CJ32.p, g);
+    launched("k_cbf_diag");
+    std::vector<float> h(c.nhalf);
+    CBFM_CUDA(cudaMemcpyAsync(h.data(), g, sizeof(float) * c.nhalf, cudaMemcpyDeviceToHost, st));
+    CBFM_CUDA(cudaStreamSynchronize(st));
+    const auto mm = std::minmax_element(h.begin(), h.end());
+    c.spread = *mm.first > 0.f ? (double)*mm.second / *mm.first : INFINITY;
+    for (float v : h)
+        if (!(v <= *mm.second)) c.spread = INFINITY;   // a NaN among them
+    return c.spread;
+}
+
+}  // namespace cbfm
 
 namespace {
 
@@ -925,7 +932,7 @@ void project(Red &r, cudaStream_t st) {
             return;
         }
     }
-    const bool lean = sizeof(T) == 8 || c.spread <= SPREAD_ASM;
+    const bool lean = sizeof(T) == 8 || cbf_spread(c, st) <= SPREAD_ASM;
     if constexpr (sizeof(T) == 4) {
         if (r.prec == CBFM_MIXED || r.prec == CBFM_MIXED_UNFUSED || r.prec == CBFM_MIXED_FUSED) {
             DevBuf<float> Zs;
@@ -1313,7 +1320,7 @@ cbfm_status cbfm_assemble_reduced_batch(const cbfm_mesh_t *meshes, const cbfm_cb
                 std::vector<Mesh *> lm;
                 std::vector<float *> lz;
                 for (size_t k = 0; k < wm.size(); ++k)
-                    if ((wc[k]->spread <= SPREAD_ASM) == (lean == 1)) {
+                    if ((cbf_spread(*wc[k], st) <= SPREAD_ASM) == (lean == 1)) {
                         lm.push_back(wm[k]);
                         lz.push_back(Zs[k].p);
                     }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -68,8 +69,10 @@ struct Cbf : HandleBase {
     int64_t nhalf = 0;            // sum L_m
     // largest over smallest modulus on the diagonal of G^CBF.  For dual CBFs (cbfm_build_cbfs, cbfm_build_ipcbfs) these are
     // their singular values; for imported blocks it is that diagonal and no more (random blocks: the smallest of
-    // several hundred moduli decides; C^M = C^J: the diagonal is zero and the spread infinite)
-    double spread = 0.0;
+    // several hundred moduli decides; C^M = C^J: the diagonal is zero and the spread infinite).  Found when a mixed
+    // assembly or solve first asks (cbf_spread), under the lock; negative until then
+    double spread = -1.0;
+    std::mutex spread_mu;
     DevBuf<z64> CM, CJ;           // blocks N_m x L_m row-major, cells in order
     DevBuf<c32> CM32, CJ32;
 };
@@ -91,6 +94,7 @@ constexpr double SPREAD_MAX = 2e3;
 // of A 0.99, of the currents 1.00 times the general forms').  The fused form (k_fused.cu) and FP64 have the shorter
 // forms alone, whatever the spread.
 constexpr double SPREAD_ASM = 300.0;
+double cbf_spread(Cbf &c, cudaStream_t st);   // api.cu; the first call waits for the stream
 
 struct Red : HandleBase {
     Mesh *mesh;

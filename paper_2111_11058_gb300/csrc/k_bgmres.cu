@@ -1006,7 +1006,7 @@ GmresOut bgmres_solve(Red &rd, const z64 *d_b, int nrhs, double tol, int maxit, 
     // The basis (Gram-Schmidt and its Cholesky QR) on the tensor cores, except where the FP32 operator would carry a change
     // of its last bits into the currents (SPREAD_MAX), and in the systems without the CMP (above): there the FP64 units'
     // order of sums and the FP32 solution update stay.
-    const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || rd.cbf->spread <= SPREAD_MAX);
+    const bool tc_basis = pc == CBFM_PC_CMP && (rd.prec == CBFM_FP64 || cbf_spread(*rd.cbf, st) <= SPREAD_MAX);
     OzMat inv;   // complex64 (G^CBF)^{-1} cut into digits (the recovery of mixed systems)
     auto applyB = [&](const z64 *in, z64 *out, int rows) {
         if (pc == CBFM_PC_CMP_INEXACT) {
